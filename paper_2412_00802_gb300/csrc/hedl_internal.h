@@ -224,13 +224,15 @@ struct hedl_plan {
 namespace hedl {
 
 void set_error(const std::string &msg);
-// Surrogate dense layer on tcgen05 tensor cores (umma.cu): C[M][N] =
-// act(A[M][K] . B[N][K]^T + bias), A and B bf16 K-major, N % 256 == 0,
-// K % 64 == 0, 16-byte aligned rows; *err (device, may be null) gets bit 0
-// set if an MMA completion wait timed out.
+// Surrogate dense product on tcgen05 tensor cores (umma.cu): C[M][N] =
+// act(A . B^T + bias), FP32 accumulation, N % 64 == 0, 16-byte aligned rows.
+// A is bf16 [M][lda] (K % 64 == 0) or, with a_mn, [K][lda]; B is [N][ldb] or,
+// with b_mn, [K][ldb] (the batch may be the K of a weight gradient: no operand
+// is transposed, rows past K count as zeros).  *err (device, may be null) gets
+// bit 0 set if a completion wait timed out.
 struct UmmaArgs {
-    const void *A;   // bf16 [M][lda]
-    const void *B;   // bf16 [N][ldb]
+    const void *A;
+    const void *B;
     void *C;         // bf16 or float [M][ldc]
     const float *bias;
     int M, N, K, lda, ldb, ldc;
@@ -239,14 +241,23 @@ struct UmmaArgs {
     const void *mask;   // bf16 [M][ldc] or null: outputs where mask <= 0 become 0
     // Optional fused output layer (the surrogate's N = 2 head): with w3 (bf16
     // [2][N]) set, each row's bf16-rounded outputs are also dotted with both
-    // rows of w3 and the two partial sums added atomically to y (float
-    // [M][2], zeroed by the caller); store = 0 then skips writing C.
+    // rows of w3; the sums over column tile t (umma_tile_n wide) go to
+    // y[t][row][2].  store = 0 then skips writing C.
     const void *w3 = nullptr;
     float *y = nullptr;
     int store = 1;
+    int a_mn = 0, b_mn = 0;
+    // K in `splits` equal ranges (whole blocks of 64), range s into C + s * c_split elements
+    int splits = 1;
+    size_t c_split = 0;
+    float *colsum = nullptr;   // or float [ceil(M/128)][N]: column sums of the bf16 outputs of each 128-row tile
 };
+constexpr int UMMA_MAX_HEAD_TILES = 8;   // column tiles of a 512-wide layer at the narrowest tile
 bool umma_shape_ok(const UmmaArgs &a);
-int umma_gemm(const UmmaArgs &a, void *stream);
+// Width of the column tiles that umma_gemm takes for these products.
+int umma_tile_n(const UmmaArgs *a, int count);
+// One launch over one or two independent products.
+int umma_gemm(const UmmaArgs *a, int count, void *stream);
 
 int fail(int code, const std::string &msg);
 int cuda_fail(int cuda_err, const char *what);

@@ -4,11 +4,20 @@
 // paper has no counterpart; the surrogate only orders and prunes the queue of
 // exact evaluations.
 //
-// The dense layers run on the tensor cores through a warp-level BF16 GEMM
-// (mma.sync m16n8k16, operands staged in shared memory and read with
-// ldmatrix, FP32 accumulators in registers) with fused epilogues: bias, ReLU,
-// the ReLU-derivative mask of the backward pass, BF16 or FP32 output, and a
-// split-K mode that accumulates weight gradients with atomics.
+// The dense layers run on tcgen05 (umma.cu).  The comparison engine is a
+// warp-level BF16 GEMM (mma.sync m16n8k16, operands staged in shared memory
+// and read with ldmatrix, FP32 accumulators in registers) with the same
+// epilogues; its split-K mode accumulates weight gradients with atomics.
+//
+// A training step is six launches: two layers forward (the second also dots
+// its rows with the output layer), head_bwd_kernel (output layer, loss and
+// its gradients), dH1, both weight gradients, and update_kernel (partial sums
+// to gradients, Adam).  Every sum over the batch is first a partial sum of a
+// chunk of rows and then a sum over chunks in a fixed order, so a step's
+// gradients do not depend on timing.  At batches of 4,096 this took a step
+// from 785 us to 70 us: the weight gradient of the output layer
+// (584 us) and the bias gradients (2 x 238 us) had been two blocks' loops over
+// the whole batch, and the weight gradients had needed four transposes.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -296,16 +305,21 @@ int gemm(const GemmArgs &a0, bool a_km, bool b_kn, int splits, cudaStream_t s) {
 // With map (DEVICE float[5]: mean0, mean1, scale0, scale1, tail weight), the
 // raw output u is mapped back to the target scale: Y = u * scale + mean.
 // y = (u + b3), mapped back to the target scale when map is set, from the
-// fused output layer's sums u (the unfused path's out_fwd_kernel semantics).
-__global__ void out_map_kernel(const float *u, const float *b3, float *Y, int B, const float *map) {
+// fused output layer's sums u [parts][B][2] (the unfused path's out_fwd_kernel semantics).
+__global__ void out_map_kernel(const float *u, int parts, const float *b3, float *Y, int B, const float *map) {
     for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < B; row += gridDim.x * blockDim.x) {
-        float u0 = u[2 * row] + b3[0], u1 = u[2 * row + 1] + b3[1];
+        float u0 = 0.f, u1 = 0.f;
+        for (int p = 0; p < parts; ++p) {
+            const float2 q = reinterpret_cast<const float2 *>(u)[(size_t)p * B + row];
+            u0 += q.x, u1 += q.y;
+        }
+        u0 += b3[0], u1 += b3[1];
         if (map) {
             u0 = u0 * map[2] + map[0];
             u1 = u1 * map[3] + map[1];
         }
-        Y[2 * row] = u0;
-        Y[2 * row + 1] = u1;
+        Y[2 * (size_t)row] = u0;
+        Y[2 * (size_t)row + 1] = u1;
     }
 }
 
@@ -363,22 +377,79 @@ __global__ void out_fwd_kernel(const __nv_bfloat16 *H2, const __nv_bfloat16 *W3,
     }
 }
 
-// Raw outputs U against mapped targets t' = (T - mean) / scale, row weight
-// w = 1 + tail * max(0, t'_0) (the upper tail of the first target counts
-// more): dU = 2 w (U - t') / B; loss += w (U - t')^2 / B.
-__global__ void loss_kernel(const float *U, const float *T, float *dU, float *loss, int B, const float *map) {
-    float l = 0.f;
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x) {
-        const float t0 = (T[2 * b] - map[0]) / map[2], t1 = (T[2 * b + 1] - map[1]) / map[3];
-        const float w = 1.f + map[4] * fmaxf(t0, 0.f);
-        const float d0 = U[2 * b] - t0, d1 = U[2 * b + 1] - t1;
-        dU[2 * b] = 2.f * w * d0 / (float)B;
-        dU[2 * b + 1] = 2.f * w * d1 / (float)B;
-        l += w * (d0 * d0 + d1 * d1) / (float)B;
-    }
+// Output layer's backward pass over a chunk of HB_ROWS rows a block.
+//   Raw outputs u = sum of y's parts + b3 (b3 null: y is already u), mapped
+//   targets t' = (T - mean) / scale, row weight w = 1 + tail * max(0, t'_0)
+//   (the upper tail of the first target counts more): dU = 2 w (u - t') / B;
+//   loss += w (u - t')^2 / B.
+//   dH2[b][i] = (dU[b] . W3[:, i]) * [H2[b][i] > 0], stored as bf16.
+// The block's partial sums of dW3[j][i] = dU[b][j] H2[b][i], of db2[i] =
+// dH2[b][i] (as stored), of db3 = dU and of the loss go to part[block].  A
+// thread owns two columns and walks the rows eight at a time (their loads
+// in flight together); HB_ROWS = 32 gives a batch of 4,096 128 blocks.  It is
+// bound by reading H2 and writing dH2 (8 MB at 4,096 rows).
+constexpr int HB_ROWS = 32, HB_PART = 3 * DH + 4;   // dW3 [2][512], db2 [512], db3 [2], loss
+__global__ void __launch_bounds__(256) head_bwd_kernel(const float *y, int parts, const float *b3,
+                                                       const __nv_bfloat16 *W3, const float *T, const float *map,
+                                                       const __nv_bfloat16 *H2, __nv_bfloat16 *dH2, float *part, int B) {
+    __shared__ float2 du[HB_ROWS];
+    const int r0 = blockIdx.x * HB_ROWS, rows = min(HB_ROWS, B - r0);
+    part += (size_t)blockIdx.x * HB_PART;
+    if (threadIdx.x < HB_ROWS) {   // one warp: a row a lane
+        const int b = r0 + (int)threadIdx.x;
+        float g0 = 0.f, g1 = 0.f, l = 0.f;
+        if ((int)threadIdx.x < rows) {
+            float u0 = 0.f, u1 = 0.f;
+            for (int p = 0; p < parts; ++p) {
+                const float2 q = reinterpret_cast<const float2 *>(y)[(size_t)p * B + b];
+                u0 += q.x, u1 += q.y;
+            }
+            if (b3) u0 += b3[0], u1 += b3[1];
+            const float t0 = (T[2 * (size_t)b] - map[0]) / map[2], t1 = (T[2 * (size_t)b + 1] - map[1]) / map[3];
+            const float w = 1.f + map[4] * fmaxf(t0, 0.f);
+            const float d0 = u0 - t0, d1 = u1 - t1;
+            g0 = 2.f * w * d0 / (float)B;
+            g1 = 2.f * w * d1 / (float)B;
+            l = w * (d0 * d0 + d1 * d1) / (float)B;
+        }
+        du[threadIdx.x] = make_float2(g0, g1);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
-    if ((threadIdx.x & 31) == 0 && loss) atomicAdd(loss, l);
+        for (int o = 16; o > 0; o >>= 1) {
+            g0 += __shfl_xor_sync(0xFFFFFFFFu, g0, o);
+            g1 += __shfl_xor_sync(0xFFFFFFFFu, g1, o);
+            l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
+        }
+        if (threadIdx.x == 0) part[3 * DH] = g0, part[3 * DH + 1] = g1, part[3 * DH + 2] = l;
+    }
+    __syncthreads();
+    const int c = 2 * (int)threadIdx.x;
+    const __nv_bfloat162 wa = *reinterpret_cast<const __nv_bfloat162 *>(W3 + c);
+    const __nv_bfloat162 wb = *reinterpret_cast<const __nv_bfloat162 *>(W3 + DH + c);
+    const float wa0 = __low2float(wa), wa1 = __high2float(wa), wb0 = __low2float(wb), wb1 = __high2float(wb);
+    float s00 = 0.f, s01 = 0.f, s10 = 0.f, s11 = 0.f, e0 = 0.f, e1 = 0.f;
+#pragma unroll 1
+    for (int r = 0; r < rows; r += 8) {
+        __nv_bfloat162 h[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            h[k] = r + k < rows ? *reinterpret_cast<const __nv_bfloat162 *>(H2 + (size_t)(r0 + r + k) * DH + c)
+                                : __floats2bfloat162_rn(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (r + k >= rows) break;
+            const float2 d = du[r + k];
+            const float h0 = __low2float(h[k]), h1 = __high2float(h[k]);
+            s00 += d.x * h0, s01 += d.x * h1;
+            s10 += d.y * h0, s11 += d.y * h1;
+            const float v0 = h0 > 0.f ? d.x * wa0 + d.y * wb0 : 0.f, v1 = h1 > 0.f ? d.x * wa1 + d.y * wb1 : 0.f;
+            const __nv_bfloat162 o = __floats2bfloat162_rn(v0, v1);
+            *reinterpret_cast<__nv_bfloat162 *>(dH2 + (size_t)(r0 + r + k) * DH + c) = o;
+            e0 += __low2float(o), e1 += __high2float(o);
+        }
+    }
+    *reinterpret_cast<float2 *>(part + c) = make_float2(s00, s01);
+    *reinterpret_cast<float2 *>(part + DH + c) = make_float2(s10, s11);
+    *reinterpret_cast<float2 *>(part + 2 * DH + c) = make_float2(e0, e1);
 }
 
 // Target map from a target set: column means, column standard deviations
@@ -415,82 +486,103 @@ __global__ void fit_map_kernel(const float *T, int B, float tail, float *map) {
     }
 }
 
-// dH2[b][i] = (dY[b][0] W3[0][i] + dY[b][1] W3[1][i]) * [H2[b][i] > 0]  (bf16)
-__global__ void out_bwd_dh_kernel(const float *dY, const __nv_bfloat16 *W3, const __nv_bfloat16 *H2,
-                                  __nv_bfloat16 *dH2, int B) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < (size_t)B * DH;
-         e += (size_t)gridDim.x * blockDim.x) {
-        const size_t b = e / DH, i = e % DH;
-        float v = dY[2 * b] * __bfloat162float(W3[i]) + dY[2 * b + 1] * __bfloat162float(W3[DH + i]);
-        if (!(__bfloat162float(H2[e]) > 0.f)) v = 0.f;
-        dH2[e] = __float2bfloat16_rn(v);
+// Column sums of each 128-row tile of dH (the mma.sync engine's db1; tcgen05's epilogue adds its own).
+__global__ void __launch_bounds__(256) colsum_kernel(const __nv_bfloat16 *dH, float *out, int B) {
+    const int c = 2 * (int)threadIdx.x, r1 = min(((int)blockIdx.x + 1) * 128, B);
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll 8
+    for (int r = blockIdx.x * 128; r < r1; ++r) {
+        const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162 *>(dH + (size_t)r * DH + c);
+        s0 += __low2float(v), s1 += __high2float(v);
     }
+    *reinterpret_cast<float2 *>(out + (size_t)blockIdx.x * DH + c) = make_float2(s0, s1);
 }
 
-// dW3[j][i] = sum_b dY[b][j] H2[b][i]; db3[j] = sum_b dY[b][j] (one thread per i, FP32)
-__global__ void out_bwd_dw_kernel(const float *dY, const __nv_bfloat16 *H2, float *dW3, float *db3, int B) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < DH) {
-        float s0 = 0.f, s1 = 0.f;
-        for (int b = 0; b < B; ++b) {
-            const float h = __bfloat162float(H2[(size_t)b * DH + i]);
-            s0 += dY[2 * b] * h;
-            s1 += dY[2 * b + 1] * h;
-        }
-        dW3[i] = s0;
-        dW3[DH + i] = s1;
-    }
-    if (i == 0) {
-        float s0 = 0.f, s1 = 0.f;
-        for (int b = 0; b < B; ++b) {
-            s0 += dY[2 * b];
-            s1 += dY[2 * b + 1];
-        }
-        db3[0] = s0;
-        db3[1] = s1;
-    }
+// The partial sums of a batch's gradients.
+struct GradParts {
+    const float *w1, *w2;   // [splits][512][512]
+    const float *b1;        // [b1_n][512]: column sums of dH1 by 128-row tile
+    const float *head;      // [head_n][HB_PART]
+    int splits, b1_n, head_n;
+};
+
+struct AdamArgs {
+    float *w, *m, *v;
+    __nv_bfloat16 *wb;
+    float lr, b1, b2, eps, c1, c2;
+};
+
+__device__ __forceinline__ float adam_update(const AdamArgs &a, float g, float &m, float &v, float w) {
+    m = a.b1 * m + (1.f - a.b1) * g;
+    v = a.b2 * v + (1.f - a.b2) * g * g;
+    return w - a.lr * (m / a.c1) / (sqrtf(v / a.c2) + a.eps);
 }
 
-// db[i] = sum_b dH[b][i]
-__global__ void colsum_kernel(const __nv_bfloat16 *dH, float *db, int B, int D) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= D) return;
+// Sums the gradients' parts, stores the gradients and the loss and, with ADAM,
+// updates the FP32 master weights and their BF16 copies.  The first UP_BIG
+// blocks own W1 and W2, four weights a thread; the others own 32 of the
+// remaining 2,051 sums each, eight threads a sum (those have up to one part
+// per HB_ROWS rows).  Bound by memory: 16 MB of moments, weights and gradients
+// plus a megabyte a split and matrix, most of it in L2.
+constexpr int UP_BIG = 2 * DH * DH / 4 / 256, UP_SMALL = (4 * DH + 3 + 31) / 32;
+template <bool ADAM>
+__global__ void __launch_bounds__(256) update_kernel(GradParts p, float *g, float *loss, AdamArgs a) {
+    if (blockIdx.x < UP_BIG) {
+        const int e = (int)(blockIdx.x * 256 + threadIdx.x), half = DH * DH / 4;
+        const bool second = e >= half;
+        const size_t k = second ? e - half : e;   // float4 within the matrix
+        const float4 *src = reinterpret_cast<const float4 *>(second ? p.w2 : p.w1) + k;
+        const size_t at = (second ? (size_t)(DH * DH + DH) : 0) + 4 * k;   // its place among the parameters
+        float4 s = src[0];
+        for (int q = 1; q < p.splits; ++q) {
+            const float4 x = src[(size_t)q * half];
+            s.x += x.x, s.y += x.y, s.z += x.z, s.w += x.w;
+        }
+        *reinterpret_cast<float4 *>(g + at) = s;
+        if constexpr (ADAM) {
+            float4 w = *reinterpret_cast<const float4 *>(a.w + at), m = *reinterpret_cast<const float4 *>(a.m + at),
+                   v = *reinterpret_cast<const float4 *>(a.v + at);
+            w.x = adam_update(a, s.x, m.x, v.x, w.x);
+            w.y = adam_update(a, s.y, m.y, v.y, w.y);
+            w.z = adam_update(a, s.z, m.z, v.z, w.z);
+            w.w = adam_update(a, s.w, m.w, v.w, w.w);
+            *reinterpret_cast<float4 *>(a.w + at) = w;
+            *reinterpret_cast<float4 *>(a.m + at) = m;
+            *reinterpret_cast<float4 *>(a.v + at) = v;
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(w.x, w.y), hi = __floats2bfloat162_rn(w.z, w.w);
+            *reinterpret_cast<uint2 *>(a.wb + at) =
+                make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+        }
+        return;
+    }
+    // b1 [512], b2 [512], W3 [1024], b3 [2], the loss
+    __shared__ float red[8][33];
+    const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5, e = (int)(blockIdx.x - UP_BIG) * 32 + lane;
+    const float *src = nullptr;
+    size_t stride = HB_PART, at = 0;
+    int n = p.head_n;
+    if (e < DH) src = p.b1 + e, stride = DH, n = p.b1_n, at = (size_t)DH * DH + e;
+    else if (e < 2 * DH) src = p.head + DH + e, at = 2 * (size_t)DH * DH + e;               // db2 at 2 * 512 of a part
+    else if (e < 4 * DH) src = p.head + (e - 2 * DH), at = 2 * (size_t)DH * DH + e;         // dW3
+    else if (e < 4 * DH + 3) src = p.head + (e - DH), at = 2 * (size_t)DH * DH + e;         // db3, loss
     float s = 0.f;
-    for (int b = 0; b < B; ++b) s += __bfloat162float(dH[(size_t)b * D + i]);
-    db[i] = s;
-}
-
-// Adam on FP32 master weights; refreshes the BF16 copy.
-// dst[c][r] = src[r][c] for an R x C bf16 matrix (32 x 32 tiles through shared memory).
-__global__ void transpose_bf16_kernel(const __nv_bfloat16 *src, int R, int C, int lds, __nv_bfloat16 *dst, int ldd) {
-    __shared__ __nv_bfloat16 t[32][34];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        if (r < R && c < C) t[i][threadIdx.x] = src[(size_t)r * lds + c];
-    }
+    if (src)
+        for (int q = sub; q < n; q += 8) s += src[(size_t)q * stride];
+    red[sub][lane] = s;
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (r < R && c < C) dst[(size_t)c * ldd + r] = t[threadIdx.x][i];
+    if (sub != 0 || !src) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += red[q][lane];
+    if (e == 4 * DH + 2) {
+        if (loss) *loss = s;
+        return;
     }
-}
-
-void transpose_bf16(const __nv_bfloat16 *src, int R, int C, int lds, __nv_bfloat16 *dst, int ldd, cudaStream_t s) {
-    transpose_bf16_kernel<<<dim3((C + 31) / 32, (R + 31) / 32), dim3(32, 8), 0, s>>>(src, R, C, lds, dst, ldd);
-}
-
-__global__ void adam_kernel(float *w, float *m, float *v, const float *g, __nv_bfloat16 *wb, size_t n, float lr,
-                            float b1, float b2, float eps, float c1, float c2) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-        w[i] = wi;
-        if (wb) wb[i] = __float2bfloat16_rn(wi);
+    g[at] = s;
+    if constexpr (ADAM) {
+        float m = a.m[at], v = a.v[at];
+        const float w = adam_update(a, s, m, v, a.w[at]);
+        a.w[at] = w, a.m[at] = m, a.v[at] = v;
+        a.wb[at] = __float2bfloat16_rn(w);
     }
 }
 
@@ -629,7 +721,6 @@ struct hedl_mlp {
     // the target map (mean0, mean1, scale0, scale1, tail weight)
     float *w = nullptr, *m = nullptr, *v = nullptr, *g = nullptr, *map = nullptr;
     uint32_t *err = nullptr;                  // device: bit 0 = a tensor-core wait timed out
-    __nv_bfloat16 *w2t = nullptr;             // W2 transposed ([in][out], bf16) for the backward GEMM
     unsigned gemm = HEDL_GEMM_TCGEN05;        // engine of the dense layers' forward GEMMs
     __nv_bfloat16 *wb = nullptr;
     size_t n = 0;
@@ -641,19 +732,25 @@ namespace {
 constexpr size_t OFF_W1 = 0, OFF_B1 = OFF_W1 + (size_t)DH * DI, OFF_W2 = OFF_B1 + DH, OFF_B2 = OFF_W2 + (size_t)DH * DH,
                  OFF_W3 = OFF_B2 + DH, OFF_B3 = OFF_W3 + (size_t)DO * DH, N_PARAMS = OFF_B3 + DO;
 
+// K ranges of a weight gradient: 4 give the two 512 x 512 gradients 128 items
+// of 128 x 128; a batch below 193 rows has fewer blocks of 64 to split.
+int grad_splits(uint32_t B) { return (int)std::min<uint32_t>(4, (B + 63) / 64); }
+
 struct MlpWs {
     __nv_bfloat16 *h1, *h2, *dh1, *dh2;
-    float *y, *dy, *loss;
-    __nv_bfloat16 *t0, *t1;   // transposed operands ([512][B]) of the tensor-core weight gradients
+    float *y;             // [UMMA_MAX_HEAD_TILES][B][2]
+    __nv_bfloat16 *x;     // a 16-byte aligned copy of the inputs, if they are not
+    float *head, *b1;     // GradParts
+    float *w1, *w2;
 };
 
-size_t mlp_ws_bytes(uint32_t B) { return 6 * (size_t)B * DH * 2 + 2 * (size_t)B * DO * 4 + 256 + 7 * 256; }
-
-MlpWs carve(void *ws, uint32_t B) {
-    uint8_t *p = (uint8_t *)ws;
+// Lays the workspace out from `ws` (null: only measures it); *end receives its size.
+MlpWs carve(void *ws, uint32_t B, size_t *end = nullptr) {
+    size_t at = 0;
+    uint8_t *base = (uint8_t *)(((uintptr_t)ws + 255) & ~(uintptr_t)255);   // mlp_ws_bytes leaves room for it
     auto take = [&](size_t bytes) {
-        uint8_t *r = p;
-        p += (bytes + 255) & ~size_t(255);
+        uint8_t *r = base + at;
+        at += (bytes + 255) & ~size_t(255);
         return r;
     };
     MlpWs w;
@@ -661,22 +758,27 @@ MlpWs carve(void *ws, uint32_t B) {
     w.h2 = (__nv_bfloat16 *)take((size_t)B * DH * 2);
     w.dh1 = (__nv_bfloat16 *)take((size_t)B * DH * 2);
     w.dh2 = (__nv_bfloat16 *)take((size_t)B * DH * 2);
-    w.y = (float *)take((size_t)B * DO * 4);
-    w.dy = (float *)take((size_t)B * DO * 4);
-    w.loss = (float *)take(4);
-    w.t0 = (__nv_bfloat16 *)take((size_t)B * DH * 2);
-    w.t1 = (__nv_bfloat16 *)take((size_t)B * DH * 2);
+    w.y = (float *)take((size_t)UMMA_MAX_HEAD_TILES * B * DO * 4);
+    w.x = (__nv_bfloat16 *)take((size_t)B * DI * 2);
+    w.head = (float *)take(((size_t)B + HB_ROWS - 1) / HB_ROWS * HB_PART * 4);
+    w.b1 = (float *)take(((size_t)B + 127) / 128 * DH * 4);
+    w.w1 = (float *)take((size_t)grad_splits(B) * DH * DI * 4);
+    w.w2 = (float *)take((size_t)grad_splits(B) * DH * DH * 4);
+    if (end) *end = at;
     return w;
+}
+
+size_t mlp_ws_bytes(uint32_t B) {
+    size_t n = 0;
+    carve(nullptr, B, &n);
+    return n + 256;
 }
 
 uint32_t grid1(size_t n) { return (uint32_t)std::min<size_t>((n + 255) / 256, 4096); }
 
-// One hidden layer, H = relu(A . W^T + b): on tcgen05 when selected (and the
-// shape allows it), else on the mma.sync GEMM.
-int dense_relu(hedl_mlp *mlp, const __nv_bfloat16 *A, const __nv_bfloat16 *W, const float *b, __nv_bfloat16 *H,
-               int M, int K, cudaStream_t s) {
-    UmmaArgs u{A, W, H, b, M, DH, K, K, K, DH, 1, 1, mlp->err, nullptr};
-    if (mlp->gemm == HEDL_GEMM_TCGEN05 && umma_shape_ok(u)) return umma_gemm(u, s);
+// One hidden layer, H = relu(A . W^T + b), on the mma.sync engine.
+int dense_relu(const __nv_bfloat16 *A, const __nv_bfloat16 *W, const float *b, __nv_bfloat16 *H, int M, int K,
+               cudaStream_t s) {
     GemmArgs a{};
     a.A = A;
     a.B = W;
@@ -687,75 +789,77 @@ int dense_relu(hedl_mlp *mlp, const __nv_bfloat16 *A, const __nv_bfloat16 *W, co
     return gemm(a, false, false, 1, s);
 }
 
-int forward_impl(hedl_mlp *mlp, const __nv_bfloat16 *X, uint32_t B, const MlpWs &w, cudaStream_t s,
-                 bool mapped, bool need_h2 = true) {
-    int e = dense_relu(mlp, X, mlp->wb + OFF_W1, mlp->w + OFF_B1, w.h1, (int)B, DI, s);
-    if (e) return e;
-    if (!need_h2 && mlp->gemm == HEDL_GEMM_TCGEN05) {
-        // inference: the second layer's epilogue computes the output layer (h2 is never written)
-        UmmaArgs u{w.h1, mlp->wb + OFF_W2, w.h2, mlp->w + OFF_B2, (int)B, DH, DH, DH, DH, DH, 1, 1, mlp->err, nullptr};
-        u.w3 = mlp->wb + OFF_W3;
-        u.y = w.dy;   // [B][2] sums, zeroed first
-        u.store = 0;
-        if (umma_shape_ok(u)) {
-            e = cudaMemsetAsync(w.dy, 0, (size_t)B * DO * 4, s);
-            if (e) return e;
-            e = umma_gemm(u, s);
-            if (e) return e;
-            out_map_kernel<<<std::min<uint32_t>((B + 255) / 256, 148u * 8u), 256, 0, s>>>(
-                w.dy, mlp->w + OFF_B3, w.y, (int)B, mapped ? mlp->map : nullptr);
-            return cudaGetLastError();
-        }
+// Both hidden layers and the output layer's sums into w.y, whose parts come
+// back in *parts (0: w.y already holds u with b3).  need_h2 = false
+// (inference) leaves the second layer's activations unwritten.
+int forward_impl(hedl_mlp *mlp, const __nv_bfloat16 *X, uint32_t B, const MlpWs &w, cudaStream_t s, bool need_h2,
+                 int *parts) {
+    int e;
+    if (mlp->gemm == HEDL_GEMM_TCGEN05) {
+        UmmaArgs u{X, mlp->wb + OFF_W1, w.h1, mlp->w + OFF_B1, (int)B, DH, DI, DI, DI, DH, 1, 1, mlp->err, nullptr};
+        e = umma_gemm(&u, 1, s);
+        if (e) return e;
+        UmmaArgs v{w.h1, mlp->wb + OFF_W2, w.h2, mlp->w + OFF_B2, (int)B, DH, DH, DH, DH, DH, 1, 1, mlp->err, nullptr};
+        v.w3 = mlp->wb + OFF_W3;
+        v.y = w.y;
+        v.store = need_h2;
+        *parts = DH / umma_tile_n(&v, 1);
+        return umma_gemm(&v, 1, s);
     }
-    e = dense_relu(mlp, w.h1, mlp->wb + OFF_W2, mlp->w + OFF_B2, w.h2, (int)B, DH, s);
+    e = dense_relu(X, mlp->wb + OFF_W1, mlp->w + OFF_B1, w.h1, (int)B, DI, s);
+    if (!e) e = dense_relu(w.h1, mlp->wb + OFF_W2, mlp->w + OFF_B2, w.h2, (int)B, DH, s);
     if (e) return e;
     out_fwd_kernel<<<std::min<uint32_t>((B * 32 + 255) / 256, 148u * 8u), 256, 0, s>>>(
-        w.h2, mlp->wb + OFF_W3, mlp->w + OFF_B3, w.y, (int)B, mapped ? mlp->map : nullptr);
+        w.h2, mlp->wb + OFF_W3, mlp->w + OFF_B3, w.y, (int)B, nullptr);
+    *parts = 0;
     return cudaGetLastError();
 }
 
-int grads_impl(hedl_mlp *mlp, const __nv_bfloat16 *X, const float *T, uint32_t B, const MlpWs &w, cudaStream_t s) {
-    int e = forward_impl(mlp, X, B, w, s, false);
+// TMA and the 16-byte loads need aligned rows: inputs that are not are copied once.
+int aligned_input(const __nv_bfloat16 *&X, uint32_t B, const MlpWs &w, cudaStream_t s) {
+    if (((uintptr_t)X & 15) == 0) return 0;
+    cudaError_t e = cudaMemcpyAsync(w.x, X, (size_t)B * DI * 2, cudaMemcpyDeviceToDevice, s);
+    X = w.x;
+    return e;
+}
+
+// The batch's gradient parts, up to (not including) update_kernel.
+int grads_impl(hedl_mlp *mlp, const __nv_bfloat16 *X, const float *T, uint32_t B, const MlpWs &w, cudaStream_t s,
+               GradParts *out) {
+    if (B == 0) return cudaErrorInvalidConfiguration;
+    int parts = 0, e = aligned_input(X, B, w, s);
+    if (!e) e = forward_impl(mlp, X, B, w, s, true, &parts);
     if (e) return e;
-    e = cudaMemsetAsync(w.loss, 0, 4, s);
-    if (e) return e;
-    e = cudaMemsetAsync(mlp->g, 0, N_PARAMS * 4, s);
-    if (e) return e;
-    loss_kernel<<<grid1(B), 256, 0, s>>>(w.y, T, w.dy, w.loss, (int)B, mlp->map);
-    out_bwd_dw_kernel<<<(DH + 255) / 256, 256, 0, s>>>(w.dy, w.h2, mlp->g + OFF_W3, mlp->g + OFF_B3, (int)B);
-    out_bwd_dh_kernel<<<grid1((size_t)B * DH), 256, 0, s>>>(w.dy, mlp->wb + OFF_W3, w.h2, w.dh2, (int)B);
-    colsum_kernel<<<(DH + 255) / 256, 256, 0, s>>>(w.dh2, mlp->g + OFF_B2, (int)B, DH);
-    if (mlp->gemm == HEDL_GEMM_TCGEN05 && B % 64 == 0) {
-        // Weight gradients dW = dH^T . H on tcgen05 as K-major products over the
-        // batch: both operands are transposed to [512][B] first.
-        transpose_bf16(w.dh2, (int)B, DH, DH, w.t0, (int)B, s);
-        transpose_bf16(w.h1, (int)B, DH, DH, w.t1, (int)B, s);
-        UmmaArgs u{w.t0, w.t1, mlp->g + OFF_W2, nullptr, DH, DH, (int)B, (int)B, (int)B, DH, 0, 0, mlp->err,
-                   nullptr};
-        e = umma_gemm(u, s);
+    const int M = (int)B, splits = grad_splits(B);
+    *out = GradParts{w.w1, w.w2, w.b1, w.head, splits, (M + 127) / 128, (M + HB_ROWS - 1) / HB_ROWS};
+    head_bwd_kernel<<<out->head_n, 256, 0, s>>>(w.y, parts ? parts : 1, parts ? mlp->w + OFF_B3 : nullptr,
+                                                mlp->wb + OFF_W3, T, mlp->map, w.h2, w.dh2, w.head, M);
+    if (mlp->gemm == HEDL_GEMM_TCGEN05) {
+        // dH1 = (dH2 . W2) * [H1 > 0]; W2 [out][in] is the MN-major operand
+        UmmaArgs d{w.dh2, mlp->wb + OFF_W2, w.dh1, nullptr, M, DH, DH, DH, DH, DH, 0, 1, mlp->err, w.h1};
+        d.b_mn = 1;
+        d.colsum = w.b1;
+        e = umma_gemm(&d, 1, s);
         if (e) return e;
-        // dH1 = (dH2 . W2) * [H1 > 0], with W2 kept transposed ([in][out], K-major)
-        UmmaArgs d{w.dh2, mlp->w2t, w.dh1, nullptr, (int)B, DH, DH, DH, DH, DH, 0, 1, mlp->err, w.h1};
-        e = umma_gemm(d, s);
-        if (e) return e;
-        colsum_kernel<<<(DH + 255) / 256, 256, 0, s>>>(w.dh1, mlp->g + OFF_B1, (int)B, DH);
-        transpose_bf16(w.dh1, (int)B, DH, DH, w.t0, (int)B, s);
-        transpose_bf16(X, (int)B, DI, DI, w.t1, (int)B, s);
-        UmmaArgs x{w.t0, w.t1, mlp->g + OFF_W1, nullptr, DH, DI, (int)B, (int)B, (int)B, DI, 0, 0, mlp->err,
-                   nullptr};
-        e = umma_gemm(x, s);
-        if (e) return e;
-        return cudaGetLastError();
+        // dW1 = dH1^T . X and dW2 = dH2^T . H1: contractions over the batch, both operands MN-major
+        UmmaArgs g[2] = {{w.dh1, X, w.w1, nullptr, DH, DI, M, DH, DI, DI, 0, 0, mlp->err, nullptr},
+                         {w.dh2, w.h1, w.w2, nullptr, DH, DH, M, DH, DH, DH, 0, 0, mlp->err, nullptr}};
+        for (UmmaArgs &a : g) a.a_mn = a.b_mn = 1, a.splits = splits, a.c_split = (size_t)DH * DH;
+        return umma_gemm(g, 2, s);
     }
-    const int splits = std::max(1, std::min((int)(B / 256), 64));
+    out->splits = 1;   // the atomics add every K range into the first part
+    e = cudaMemsetAsync(w.w1, 0, (size_t)DH * DI * 4, s);
+    if (!e) e = cudaMemsetAsync(w.w2, 0, (size_t)DH * DH * 4, s);
+    if (e) return e;
+    const int k_splits = std::max(1, std::min((int)(B / 256), 64));
     // dW2 = dH2^T H1   (M = out, N = in, K = batch): A stored [K][M], B stored [K][N]
     GemmArgs a{};
     a.A = w.dh2;
     a.B = w.h1;
-    a.C = mlp->g + OFF_W2;
-    a.M = DH, a.N = DH, a.K = (int)B, a.lda = DH, a.ldb = DH, a.ldc = DH;
+    a.C = w.w2;
+    a.M = DH, a.N = DH, a.K = M, a.lda = DH, a.ldb = DH, a.ldc = DH;
     a.atomic = 1;
-    e = gemm(a, true, true, splits, s);
+    e = gemm(a, true, true, k_splits, s);
     if (e) return e;
     // dH1 = (dH2 W2) * [H1 > 0]   (M = batch, N = in, K = out): A [M][K], B stored [K][N]
     GemmArgs d{};
@@ -763,19 +867,17 @@ int grads_impl(hedl_mlp *mlp, const __nv_bfloat16 *X, const float *T, uint32_t B
     d.B = mlp->wb + OFF_W2;
     d.C = w.dh1;
     d.mask = w.h1;
-    d.M = (int)B, d.N = DH, d.K = DH, d.lda = DH, d.ldb = DH, d.ldc = DH;
+    d.M = M, d.N = DH, d.K = DH, d.lda = DH, d.ldb = DH, d.ldc = DH;
     d.out_bf16 = 1;
     e = gemm(d, false, true, 1, s);
     if (e) return e;
-    colsum_kernel<<<(DH + 255) / 256, 256, 0, s>>>(w.dh1, mlp->g + OFF_B1, (int)B, DH);
+    colsum_kernel<<<out->b1_n, 256, 0, s>>>(w.dh1, w.b1, M);
     // dW1 = dH1^T X
     a.A = w.dh1;
     a.B = X;
-    a.C = mlp->g + OFF_W1;
+    a.C = w.w1;
     a.N = DI, a.ldb = DI;
-    e = gemm(a, true, true, splits, s);
-    if (e) return e;
-    return cudaGetLastError();
+    return gemm(a, true, true, k_splits, s);
 }
 
 }  // namespace
@@ -792,12 +894,11 @@ int hedl_mlp_create(const float *params, hedl_mlp **out) {
     if (!e) e = cudaMalloc(&m->v, N_PARAMS * 4);
     if (!e) e = cudaMalloc(&m->g, N_PARAMS * 4);
     if (!e) e = cudaMalloc(&m->wb, N_PARAMS * 2);
-    if (!e) e = cudaMalloc(&m->map, 5 * 4);
+    if (!e) e = cudaMalloc(&m->map, 7 * 4);
     if (!e) e = cudaMalloc(&m->err, 4);
     if (!e) e = cudaMemset(m->err, 0, 4);
-    if (!e) e = cudaMalloc(&m->w2t, (size_t)DH * DH * 2);
     if (!e) {
-        const float ident[5] = {0.f, 0.f, 1.f, 1.f, 0.f};
+        const float ident[7] = {0.f, 0.f, 1.f, 1.f, 0.f, 0.f, 0.f};   // and two zeros behind it
         e = cudaMemcpy(m->map, ident, sizeof(ident), cudaMemcpyHostToDevice);
     }
     if (!e) e = cudaMemcpy(m->w, params, N_PARAMS * 4, cudaMemcpyHostToDevice);
@@ -805,7 +906,6 @@ int hedl_mlp_create(const float *params, hedl_mlp **out) {
     if (!e) e = cudaMemset(m->v, 0, N_PARAMS * 4);
     if (!e) {
         to_bf16_kernel<<<grid1(N_PARAMS), 256>>>(m->w, m->wb, N_PARAMS);
-        transpose_bf16(m->wb + OFF_W2, DH, DH, DH, m->w2t, DH, 0);
         e = cudaDeviceSynchronize();
     }
     if (e) {
@@ -827,7 +927,6 @@ void hedl_mlp_free(hedl_mlp *m) {
     cudaFree(m->wb);
     cudaFree(m->map);
     cudaFree(m->err);
-    cudaFree(m->w2t);
     delete m;
 }
 
@@ -872,11 +971,18 @@ int hedl_mlp_forward(hedl_mlp *m, const uint16_t *X, uint32_t B, float *Y, void 
                      hedl_stream s) {
     if (!m || !X || !Y) return fail(HEDL_ERR_INVALID_ARG, "NULL argument");
     if (!ws || ws_bytes < mlp_ws_bytes(B)) return fail(HEDL_ERR_WORKSPACE_TOO_SMALL, "MLP workspace too small");
+    if (B == 0) return cuda_fail(cudaErrorInvalidConfiguration, "mlp forward");
     MlpWs w = carve(ws, B);
-    int e = forward_impl(m, (const __nv_bfloat16 *)X, B, w, (cudaStream_t)s, true, false);
+    cudaStream_t st = (cudaStream_t)s;
+    const __nv_bfloat16 *x = (const __nv_bfloat16 *)X;
+    int parts = 0, e = aligned_input(x, B, w, st);
+    if (!e) e = forward_impl(m, x, B, w, st, false, &parts);
     if (e) return cuda_fail(e, "mlp forward");
-    e = cudaMemcpyAsync(Y, w.y, (size_t)B * DO * 4, cudaMemcpyDeviceToDevice, (cudaStream_t)s);
-    return e ? cuda_fail(e, "mlp forward copy") : HEDL_OK;
+    const float *zero_b3 = m->map + 5;   // two zeros behind the map: b3 when w.y already has it
+    out_map_kernel<<<std::min<uint32_t>((B + 255) / 256, 148u * 8u), 256, 0, st>>>(
+        w.y, parts ? parts : 1, parts ? m->w + OFF_B3 : zero_b3, Y, (int)B, m->map);
+    e = cudaGetLastError();
+    return e ? cuda_fail(e, "mlp forward") : HEDL_OK;
 }
 
 int hedl_mlp_gradients(hedl_mlp *m, const uint16_t *X, const float *T, uint32_t B, float *loss, void *ws,
@@ -884,27 +990,29 @@ int hedl_mlp_gradients(hedl_mlp *m, const uint16_t *X, const float *T, uint32_t 
     if (!m || !X || !T) return fail(HEDL_ERR_INVALID_ARG, "NULL argument");
     if (!ws || ws_bytes < mlp_ws_bytes(B)) return fail(HEDL_ERR_WORKSPACE_TOO_SMALL, "MLP workspace too small");
     MlpWs w = carve(ws, B);
-    int e = grads_impl(m, (const __nv_bfloat16 *)X, T, B, w, (cudaStream_t)s);
+    GradParts p;
+    int e = grads_impl(m, (const __nv_bfloat16 *)X, T, B, w, (cudaStream_t)s, &p);
     if (e) return cuda_fail(e, "mlp gradients");
-    if (loss) {
-        e = cudaMemcpyAsync(loss, w.loss, 4, cudaMemcpyDeviceToDevice, (cudaStream_t)s);
-        if (e) return cuda_fail(e, "loss copy");
-    }
-    return HEDL_OK;
+    update_kernel<false><<<UP_BIG + UP_SMALL, 256, 0, (cudaStream_t)s>>>(p, m->g, loss, AdamArgs{});
+    e = cudaGetLastError();
+    return e ? cuda_fail(e, "mlp gradients") : HEDL_OK;
 }
 
 int hedl_mlp_train_step(hedl_mlp *m, const uint16_t *X, const float *T, uint32_t B, float lr, float *loss,
                         void *ws, size_t ws_bytes, hedl_stream s) {
-    int e = hedl_mlp_gradients(m, X, T, B, loss, ws, ws_bytes, s);
-    if (e) return e;
+    if (!m || !X || !T) return fail(HEDL_ERR_INVALID_ARG, "NULL argument");
+    if (!ws || ws_bytes < mlp_ws_bytes(B)) return fail(HEDL_ERR_WORKSPACE_TOO_SMALL, "MLP workspace too small");
+    MlpWs w = carve(ws, B);
+    GradParts p;
+    int e = grads_impl(m, (const __nv_bfloat16 *)X, T, B, w, (cudaStream_t)s, &p);
+    if (e) return cuda_fail(e, "mlp gradients");
     m->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - powf(b1, (float)m->step), c2 = 1.f - powf(b2, (float)m->step);
-    adam_kernel<<<grid1(N_PARAMS), 256, 0, (cudaStream_t)s>>>(m->w, m->m, m->v, m->g, m->wb, N_PARAMS, lr, b1, b2,
-                                                                1e-8f, c1, c2);
-    transpose_bf16(m->wb + OFF_W2, DH, DH, DH, m->w2t, DH, (cudaStream_t)s);
-    cudaError_t ce = cudaGetLastError();
-    return ce ? cuda_fail(ce, "adam launch") : HEDL_OK;
+    update_kernel<true><<<UP_BIG + UP_SMALL, 256, 0, (cudaStream_t)s>>>(
+        p, m->g, loss, AdamArgs{m->w, m->m, m->v, m->wb, lr, b1, b2, 1e-8f, c1, c2});
+    e = cudaGetLastError();
+    return e ? cuda_fail(e, "adam launch") : HEDL_OK;
 }
 
 int hedl_mlp_fit_target_map(hedl_mlp *m, const float *T, uint32_t B, float tail_weight, hedl_stream s) {

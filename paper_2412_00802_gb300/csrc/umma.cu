@@ -1,25 +1,33 @@
-// Dense layer GEMM of the surrogate on the 5th-generation tensor cores:
-// C[M][N] = act(A[M][K] . B[N][K]^T + bias), A and B bf16 and K-major (rows
-// of K contiguous elements), FP32 accumulation in tensor memory (TMEM).
+// Dense products of the surrogate on the 5th-generation tensor cores:
+// C[M][N] = act(A . B^T + bias), bf16 operands, FP32 accumulation in tensor
+// memory (TMEM).  An operand is K-major ([rows][K]) or MN-major ([K][rows],
+// which lets a weight gradient contract over the batch without transposing).
 //
-// A persistent kernel: one CTA per SM walks the 128 x 256 output tiles
-// blockIdx.x, blockIdx.x + gridDim.x, ...  Its six warps have fixed roles:
+// A persistent kernel: one CTA per SM walks the items (128 x UN output tile,
+// K range) blockIdx.x, blockIdx.x + gridDim.x, ... of one or two products.
+// Its six warps have fixed roles:
 //   warp 0 (one thread): the TMA producer.  It loads each 64-wide K block of
-//     the tile's A (128 x 64) and B (256 x 64) with one TMA copy each
-//     (cp.async.bulk.tensor, 128-byte rows in the 128-byte swizzle the
-//     tensor cores read as K-major SWIZZLE_128B operands) into a ring of four
-//     48 KB stages, arming the stage's "full" mbarrier with the byte count;
+//     the item's A (128 x 64) and B (UN x 64) (cp.async.bulk.tensor, 128-byte
+//     rows in the 128-byte swizzle; a K-major operand is one box, an MN-major
+//     one is a box per 64 rows) into a ring of stages, arming the stage's
+//     "full" mbarrier with the byte count;
 //   warp 1 (one thread): the MMA issuer.  Per K block it waits for a full
-//     stage, issues four tcgen05.mma (M 128, N 256, K 16) into one of two
-//     256-column TMEM accumulators and commits them to the stage's "empty"
-//     mbarrier; after a tile's last block it commits to the accumulator's
+//     stage, issues four tcgen05.mma (M 128, N UN, K 16) into one of two
+//     UN-column TMEM accumulators and commits them to the stage's "empty"
+//     mbarrier; after an item's last block it commits to the accumulator's
 //     "tmem full" mbarrier;
 //   warps 2-5: the epilogue.  Each reads its 32-lane quarter of a finished
 //     accumulator with tcgen05.ld, adds the bias, applies ReLU or a mask (the
-//     backward pass's ReLU derivative), stores bf16 or FP32 rows, and arrives
+//     backward pass's ReLU derivative), stores bf16 or FP32 rows, adds up the
+//     tile's columns or the fused output layer's sums where asked, and arrives
 //     on the accumulator's "tmem empty" mbarrier.
-// With two accumulators, the epilogue of one tile overlaps the loads and
+// With two accumulators, the epilogue of one item overlaps the loads and
 // MMAs of the next.
+//
+// Tile width: a layer of a few thousand rows is bound by the latency of one
+// item (8 K blocks through one SM), not by the tensor cores, so the tile is
+// the widest of 256, 128 and 64 columns that still gives most SMs an item
+// (umma_tile_n).
 //
 // Every wait is bounded: a wait that does not complete within 2 s records an
 // error in *err; the CTA then skips the rest of its work and still frees its
@@ -35,29 +43,36 @@
 namespace hedl {
 namespace {
 
-constexpr int UM = 128, UN = 256, UK = 64, STAGES = 4;
+constexpr int UM = 128, UK = 64;
 constexpr uint32_t ROW = UK * 2;                     // 128-byte rows of a block
 constexpr uint32_t A_BYTES = UM * UK * 2;            // 16 KB
-constexpr uint32_t B_BYTES = UN * UK * 2;            // 32 KB
-constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;  // 48 KB
-constexpr uint32_t TMEM_COLS = 2 * UN;               // two FP32 accumulators
+constexpr uint32_t MN_GROUP = 64 * ROW;              // an MN-major box: 64 k rows of 64 elements
 constexpr int THREADS = 192;                         // producer, MMA issuer, 4 epilogue warps
-constexpr size_t UMMA_SMEM = STAGES * STAGE_BYTES + 1024 + 256;
+template <int UN>
+struct Shape {
+    static constexpr uint32_t B_BYTES = UN * UK * 2;
+    static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
+    static constexpr int STAGES = UN == 256 ? 4 : UN == 128 ? 6 : 8;   // 192 KB
+    static constexpr uint32_t TMEM_COLS = 2 * UN;                      // two FP32 accumulators
+    static constexpr uint32_t CS_OFF = STAGES * STAGE_BYTES;           // column sums [4][UN]
+    static constexpr uint32_t BAR_OFF = CS_OFF + 4 * UN * 4;
+    static constexpr size_t SMEM = BAR_OFF + 256 + 1024;
+    // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
+    // (bits 7-9 and 10-12 = 1), operand majors at bits 15 and 16 (0 = K, 1 =
+    // MN), N / 8 at bit 17, M / 16 at bit 24.
+    static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(UN >> 3) << 17) |
+                                      ((uint32_t)(UM >> 4) << 24);
+};
 
-// Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
-// (bits 7-9 and 10-12 = 1), both K-major (bits 15, 16 = 0), N / 8 at bit 17,
-// M / 16 at bit 24.
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(UN >> 3) << 17) |
-                           ((uint32_t)(128 >> 4) << 24);
-
-// Shared-memory matrix descriptor of a K-major SWIZZLE_128B operand
-// (128-byte rows as TMA wrote them): start address / 16 (a K step of 16
-// elements advances it by 32 bytes inside the swizzle atom), leading byte
-// offset unused (1), stride byte offset (next 8 rows: 1024 B) / 16,
-// descriptor version 1, layout type 2 (128-byte swizzle).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1 << 16;
+// Shared-memory matrix descriptor of a SWIZZLE_128B operand block as TMA
+// wrote it, without its start address / 16: leading byte offset / 16 at bit
+// 16, stride byte offset / 16 at bit 32, descriptor version 1, layout type 2.
+//   K-major (128-byte rows of 64 k): leading unused (1), stride = 8 rows
+//     (1024 B); a K step of 16 advances the start by 32 bytes.
+//   MN-major (128-byte rows of 64 m or n, one per k): leading = the next 64
+//     m or n (8 KB), stride = 8 k rows (1024 B); a K step of 16 is 2048 bytes.
+__device__ __forceinline__ uint64_t smem_desc(bool mn) {
+    uint64_t d = (uint64_t)(mn ? MN_GROUP >> 4 : 1u) << 16;
     d |= (uint64_t)((8u * ROW) >> 4) << 32;
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)2 << 61;
@@ -114,8 +129,9 @@ __device__ __forceinline__ void tmem_ld32(uint32_t ta, uint32_t (&r)[32]) {
 }
 
 // Fused output layer on 32 columns of one row: the bf16-rounded activations
-// (what the unfused path stores and reads back) dotted with both rows of w3.
-__device__ __forceinline__ void head32(const UmmaArgs &g, int col, const float (&v)[32], float &a0, float &a1) {
+// (what the unfused path stores and reads back) dotted with both rows of w3,
+// in four partial sums each (shorter FP32 chains).
+__device__ __forceinline__ void head32(const UmmaArgs &g, int col, const float (&v)[32], float (&a0)[4], float (&a1)[4]) {
     const uint4 *w0 = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(g.w3) + col);
     const uint4 *w1 = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(g.w3) + g.N + col);
 #pragma unroll
@@ -128,25 +144,53 @@ __device__ __forceinline__ void head32(const UmmaArgs &g, int col, const float (
             const __nv_bfloat162 wy = *reinterpret_cast<const __nv_bfloat162 *>(&yv[e]);
             const __nv_bfloat162 h = __floats2bfloat162_rn(v[q * 8 + 2 * e], v[q * 8 + 2 * e + 1]);
             const float hl = __low2float(h), hh = __high2float(h);
-            a0 += hl * __low2float(wx) + hh * __high2float(wx);
-            a1 += hl * __low2float(wy) + hh * __high2float(wy);
+            a0[e] += hl * __low2float(wx) + hh * __high2float(wx);
+            a1[e] += hl * __low2float(wy) + hh * __high2float(wy);
         }
     }
 }
 
-// Epilogue of 32 columns of one row: bias, ReLU or mask, bf16 or FP32 store
-// (and the fused output layer's partial sums).
-__device__ __forceinline__ void emit32(const UmmaArgs &g, int row, int col, const uint32_t (&r)[32], float &a0,
-                                       float &a1) {
-    float v[32];
+// Column sums over the warp's 32 rows of v, one row a lane: a butterfly that
+// halves the columns a lane holds at each step; lane l ends with column l's.
+__device__ __forceinline__ float colsum32(float (&v)[32], uint32_t lane) {
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        float x = __uint_as_float(r[j]);
-        if (g.bias) x += g.bias[col + j];
-        if (g.relu) x = fmaxf(x, 0.f);
-        v[j] = x;
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const float keep = up ? v[k + o] : v[k], give = up ? v[k] : v[k + o];
+            v[k] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+        }
     }
-    if (g.mask) {   // keep where the mask (e.g. the forward activation) is positive
+    return v[0];
+}
+
+// Epilogue of 32 columns of one row: bias, ReLU or mask, bf16 or FP32 store,
+// the fused output layer's partial sums, the warp's column sums (cs: its 32
+// entries, or null; all lanes of the warp call together, row < M or not).
+__device__ __forceinline__ void emit32(const UmmaArgs &g, void *C, int row, int col, const uint32_t (&r)[32],
+                                       float (&a0)[4], float (&a1)[4], float *cs, uint32_t lane) {
+    const bool in = row < g.M;
+    float v[32];
+    if (g.bias) {
+        const float4 *b4 = reinterpret_cast<const float4 *>(g.bias + col);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float4 b = __ldg(b4 + q);
+            v[4 * q] = __uint_as_float(r[4 * q]) + b.x;
+            v[4 * q + 1] = __uint_as_float(r[4 * q + 1]) + b.y;
+            v[4 * q + 2] = __uint_as_float(r[4 * q + 2]) + b.z;
+            v[4 * q + 3] = __uint_as_float(r[4 * q + 3]) + b.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+    }
+    if (g.relu) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = fmaxf(v[j], 0.f);
+    }
+    if (g.mask && in) {   // keep where the mask (e.g. the forward activation) is positive
         const uint4 *mk =
             reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(g.mask) + (size_t)row * g.ldc + col);
 #pragma unroll
@@ -162,34 +206,68 @@ __device__ __forceinline__ void emit32(const UmmaArgs &g, int row, int col, cons
         }
     }
     if (g.w3) head32(g, col, v, a0, a1);
-    if (!g.store) return;
-    if (g.out_bf16) {
-        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(g.C) + (size_t)row * g.ldc + col);
+    if (g.store && in) {
+        if (g.out_bf16) {
+            uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(C) + (size_t)row * g.ldc + col);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint32_t w[4];
+            for (int q = 0; q < 4; ++q) {
+                uint32_t w[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const __nv_bfloat162 h = __floats2bfloat162_rn(v[q * 8 + 2 * e], v[q * 8 + 2 * e + 1]);
-                w[e] = *reinterpret_cast<const uint32_t *>(&h);
+                for (int e = 0; e < 4; ++e) {
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(v[q * 8 + 2 * e], v[q * 8 + 2 * e + 1]);
+                    w[e] = *reinterpret_cast<const uint32_t *>(&h);
+                }
+                dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
             }
-            dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    } else {
-        float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(g.C) + (size_t)row * g.ldc + col);
+        } else {
+            float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(C) + (size_t)row * g.ldc + col);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        }
+    }
+    if (cs) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = in ? __bfloat162float(__float2bfloat16_rn(v[j])) : 0.f;
+        cs[lane] = colsum32(v, lane);
     }
 }
 
-__global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant__ CUtensorMap tmA,
-                                                          const __grid_constant__ CUtensorMap tmB, UmmaArgs g) {
+// One or two products of one launch; product 1's items follow product 0's.
+struct Batch {
+    CUtensorMap ta[2], tb[2];
+    UmmaArgs g[2];
+    int items0, items;
+};
+
+// Item -> (product, tile, K blocks): splits innermost, then column tiles.
+// TWO = false (one product) keeps every argument a constant-bank operand.
+template <int UN, bool TWO>
+struct Item {
+    int p, m0, n0, split, kb0, kb1;
+    __device__ __forceinline__ Item(const Batch &b, int t) {
+        p = TWO && t >= b.items0 ? 1 : 0;
+        if (p) t -= b.items0;
+        const UmmaArgs &g = b.g[p];
+        split = t % g.splits;
+        t /= g.splits;
+        const int tiles_n = g.N / UN, nk = (g.K + UK - 1) / UK;   // splits <= nk: no range is empty
+        m0 = (t / tiles_n) * UM;
+        n0 = (t % tiles_n) * UN;
+        kb0 = (int)((long)split * nk / g.splits);
+        kb1 = (int)((long)(split + 1) * nk / g.splits);
+    }
+};
+
+template <int UN, bool TWO>
+__global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant__ Batch b) {
+    using S = Shape<UN>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t *full = reinterpret_cast<uint64_t *>(base + STAGES * STAGE_BYTES);
-    uint64_t *empty = full + STAGES;
-    uint64_t *tfull = empty + STAGES;    // [2]: accumulator ready for the epilogue
-    uint64_t *tempty = tfull + 2;        // [2]: accumulator drained by the epilogue
+    float *csum = reinterpret_cast<float *>(base + S::CS_OFF);
+    uint64_t *full = reinterpret_cast<uint64_t *>(base + S::BAR_OFF);
+    uint64_t *empty = full + S::STAGES;
+    uint64_t *tfull = empty + S::STAGES;    // [2]: accumulator ready for the epilogue
+    uint64_t *tempty = tfull + 2;           // [2]: accumulator drained by the epilogue
     uint32_t *tslot = reinterpret_cast<uint32_t *>(tempty + 2);
     volatile uint32_t *okp = tslot + 1;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
@@ -198,7 +276,7 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
                    tempty0 = smem_u32(tempty);
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < STAGES; ++i) {
+        for (int i = 0; i < S::STAGES; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8u * i) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(empty0 + 8u * i) : "memory");
         }
@@ -211,7 +289,7 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                     "r"(TMEM_COLS)
+                     "r"(S::TMEM_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -220,31 +298,45 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t taddr = *tslot;
 
-    const int nk = g.K / UK;
-    const int tiles_n = g.N / UN, tiles = ((g.M + UM - 1) / UM) * tiles_n;
-
     if (warp == 0 && lane == 0) {
         // producer: the running block count u uses stage u % STAGES
         uint32_t u = 0;
-        for (int t = blockIdx.x; t < tiles && *okp; t += gridDim.x) {
-            const int m0 = (t / tiles_n) * UM, n0 = (t % tiles_n) * UN;
-            for (int kb = 0; kb < nk; ++kb, ++u) {
-                const uint32_t st = u % STAGES;
-                if (u >= STAGES && !mbar_wait(empty0 + 8u * st, ((u - STAGES) / STAGES) & 1u, okp)) {
+        for (int t = blockIdx.x; t < b.items && *okp; t += gridDim.x) {
+            const Item<UN, TWO> it(b, t);
+            const UmmaArgs &g = b.g[it.p];
+            for (int kb = it.kb0; kb < it.kb1; ++kb, ++u) {
+                const uint32_t st = u % S::STAGES;
+                if (u >= S::STAGES && !mbar_wait(empty0 + 8u * st, ((u - S::STAGES) / S::STAGES) & 1u, okp)) {
                     *okp = 0u;
                     break;
                 }
-                const uint32_t fb = full0 + 8u * st, sa = s0 + st * STAGE_BYTES;
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(STAGE_BYTES)
+                const uint32_t fb = full0 + 8u * st, sa = s0 + st * S::STAGE_BYTES;
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(S::STAGE_BYTES)
                              : "memory");
-                tma_2d(sa, &tmA, kb * UK, m0, fb);
-                tma_2d(sa + A_BYTES, &tmB, kb * UK, n0, fb);
+                if (g.a_mn) {
+#pragma unroll
+                    for (int q = 0; q < UM / 64; ++q) tma_2d(sa + q * MN_GROUP, &b.ta[it.p], it.m0 + 64 * q, kb * UK, fb);
+                } else {
+                    tma_2d(sa, &b.ta[it.p], kb * UK, it.m0, fb);
+                }
+                if (g.b_mn) {
+#pragma unroll
+                    for (int q = 0; q < UN / 64; ++q)
+                        tma_2d(sa + A_BYTES + q * MN_GROUP, &b.tb[it.p], it.n0 + 64 * q, kb * UK, fb);
+                } else {
+                    tma_2d(sa + A_BYTES, &b.tb[it.p], kb * UK, it.n0, fb);
+                }
             }
         }
     } else if (warp == 1 && lane == 0) {
-        // MMA issuer: the CTA's j-th tile accumulates into buffer j & 1
+        // MMA issuer: the CTA's j-th item accumulates into buffer j & 1
         uint32_t u = 0, j = 0;
-        for (int t = blockIdx.x; t < tiles && *okp; t += gridDim.x, ++j) {
+        for (int t = blockIdx.x; t < b.items && *okp; t += gridDim.x, ++j) {
+            const Item<UN, TWO> it(b, t);
+            const bool amn = b.g[it.p].a_mn, bmn = b.g[it.p].b_mn;
+            const uint32_t idesc = S::IDESC | (amn ? 1u << 15 : 0u) | (bmn ? 1u << 16 : 0u);
+            const uint64_t adesc = smem_desc(amn), bdesc = smem_desc(bmn);
+            const uint32_t astep = amn ? 16u * ROW : 32u, bstep = bmn ? 16u * ROW : 32u;
             const uint32_t bf = j & 1u;
             if (j >= 2 && !mbar_wait(tempty0 + 8u * bf, ((j >> 1) - 1u) & 1u, okp)) {
                 *okp = 0u;
@@ -253,24 +345,24 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t acc_t = taddr + bf * UN;
             bool good = true;
-            for (int kb = 0; kb < nk; ++kb, ++u) {
-                const uint32_t st = u % STAGES;
-                if (!mbar_wait(full0 + 8u * st, (u / STAGES) & 1u, okp)) {
+            for (int kb = it.kb0; kb < it.kb1; ++kb, ++u) {
+                const uint32_t st = u % S::STAGES;
+                if (!mbar_wait(full0 + 8u * st, (u / S::STAGES) & 1u, okp)) {
                     *okp = 0u;
                     good = false;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t sa = s0 + st * STAGE_BYTES;
+                const uint32_t sa = s0 + st * S::STAGE_BYTES;
 #pragma unroll
                 for (int s = 0; s < UK / 16; ++s) {
-                    const uint64_t ad = smem_desc(sa + (uint32_t)s * 32u);
-                    const uint64_t bd = smem_desc(sa + A_BYTES + (uint32_t)s * 32u);
-                    const uint32_t acc = (kb > 0 || s > 0) ? 1u : 0u;
+                    const uint64_t ad = adesc + ((sa + (uint32_t)s * astep) >> 4);   // smem addresses stay below 2^18
+                    const uint64_t bd = bdesc + ((sa + A_BYTES + (uint32_t)s * bstep) >> 4);
+                    const uint32_t acc = (kb > it.kb0 || s > 0) ? 1u : 0u;
                     asm volatile(
                         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc_t),
-                        "l"(ad), "l"(bd), "r"(IDESC), "r"(acc)
+                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
                         : "memory");
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -287,55 +379,72 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
         // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, the tile rows of that quarter
         const uint32_t q = warp & 3u;
         uint32_t j = 0;
-        for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++j) {
+        for (int t = blockIdx.x; t < b.items; t += gridDim.x, ++j) {
+            const Item<UN, TWO> it(b, t);
+            const UmmaArgs &g = b.g[it.p];
             const uint32_t bf = j & 1u;
             uint32_t ok = 1u;
             if (lane == 0) ok = mbar_wait(tfull0 + 8u * bf, (j >> 1) & 1u, okp) ? 1u : 0u;
             ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+            if (g.colsum)   // the four warps meet at barriers below: they go on, or give up, together
+                asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %0, 0;\n bar.red.and.pred q, 1, 128, p;\n"
+                             " selp.u32 %0, 1, 0, q;\n}\n"
+                             : "+r"(ok)::"memory");
             if (!ok) {
                 if (lane == 0) *okp = 0u;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int m0 = (t / tiles_n) * UM, n0 = (t % tiles_n) * UN;
-            const int row = m0 + (int)(q * 32 + lane);
-            float a0 = 0.f, a1 = 0.f;   // the fused output layer's partial sums over this tile's columns
+            const int row = it.m0 + (int)(q * 32 + lane);
+            void *C = reinterpret_cast<uint8_t *>(g.C) + (size_t)it.split * g.c_split * (g.out_bf16 ? 2 : 4);
+            float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};   // the fused output layer
             for (int c0 = 0; c0 < UN; c0 += 64) {   // two 32-column loads in flight per wait
                 uint32_t ra[32], rb[32];
                 const uint32_t ta = taddr + ((q * 32u) << 16) + bf * UN + (uint32_t)c0;
                 tmem_ld32(ta, ra);
                 tmem_ld32(ta + 32u, rb);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (row < g.M) {
-                    emit32(g, row, n0 + c0, ra, a0, a1);
-                    emit32(g, row, n0 + c0 + 32, rb, a0, a1);
-                }
+                float *cs = g.colsum ? csum + q * UN + c0 : nullptr;
+                emit32(g, C, row, it.n0 + c0, ra, a0, a1, cs, lane);
+                emit32(g, C, row, it.n0 + c0 + 32, rb, a0, a1, cs ? cs + 32 : nullptr, lane);
             }
-            if (g.w3 && row < g.M) {
-                atomicAdd(g.y + 2 * (size_t)row, a0);
-                atomicAdd(g.y + 2 * (size_t)row + 1, a1);
-            }
+            // the accumulator may be overwritten from here on
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * bf) : "memory");
+            if (g.w3 && row < g.M)
+                reinterpret_cast<float2 *>(g.y)[(size_t)(it.n0 / UN) * g.M + row] =
+                    make_float2((a0[0] + a0[1]) + (a0[2] + a0[3]), (a1[0] + a1[1]) + (a1[2] + a1[3]));
+            if (g.colsum) {   // the four warps' sums, added by the 128 epilogue threads
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                for (int c = (int)threadIdx.x - 64; c < UN; c += 128)
+                    g.colsum[(size_t)(it.m0 / UM) * g.N + it.n0 + c] =
+                        (csum[c] + csum[UN + c]) + (csum[2 * UN + c] + csum[3 * UN + c]);
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+            }
         }
     }
     __syncwarp();
     __syncthreads();
-    if (threadIdx.x == 0 && !*okp && g.err) atomicOr(g.err, 1u);
+    if (threadIdx.x == 0 && !*okp && b.g[0].err) atomicOr(b.g[0].err, 1u);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(S::TMEM_COLS)
+                     : "memory");
 }
 
 }  // namespace
 
 bool umma_shape_ok(const UmmaArgs &a) {
-    return a.N % UN == 0 && a.K % UK == 0 && a.K > 0 && a.lda % 8 == 0 && a.ldb % 8 == 0 &&
-           a.ldc % (a.out_bf16 ? 8 : 4) == 0 && ((uintptr_t)a.A & 15) == 0 && ((uintptr_t)a.B & 15) == 0 &&
-           ((uintptr_t)a.C & 15) == 0 && (!a.mask || (a.ldc % 8 == 0 && ((uintptr_t)a.mask & 15) == 0)) &&
-           (!a.w3 || (a.y && ((uintptr_t)a.w3 & 15) == 0 && a.N % 8 == 0));
+    // a K-major operand is contracted in whole 64-wide blocks; an MN-major one
+    // has 64-row boxes along M or N and any K (rows past it read as zeros)
+    return a.N % 64 == 0 && a.N > 0 && a.K > 0 && (a.a_mn ? a.M % 64 == 0 : a.K % UK == 0) &&
+           (a.b_mn || a.K % UK == 0) && a.lda % 8 == 0 && a.ldb % 8 == 0 && a.splits >= 1 &&
+           a.splits <= (a.K + UK - 1) / UK && a.ldc % (a.out_bf16 ? 8 : 4) == 0 && ((uintptr_t)a.A & 15) == 0 &&
+           ((uintptr_t)a.B & 15) == 0 && ((uintptr_t)a.C & 15) == 0 && ((uintptr_t)a.bias & 15) == 0 &&
+           (!a.mask || (a.ldc % 8 == 0 && ((uintptr_t)a.mask & 15) == 0)) &&
+           (!a.w3 || (a.y && ((uintptr_t)a.w3 & 15) == 0 && ((uintptr_t)a.y & 7) == 0));
 }
 
 namespace {
@@ -371,30 +480,63 @@ bool make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int b
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int sm_count() {
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) || n < 1 ? 1 : n;
+    }();
+    return sms;
+}
+
+long item_count(const UmmaArgs &a, int un) { return (long)((a.M + UM - 1) / UM) * (a.N / un) * a.splits; }
+
+template <int UN, bool TWO>
+int launch(const UmmaArgs *a, int count, cudaStream_t s) {
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        umma_kernel<UN, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Shape<UN>::SMEM);
+    if (attr) return (int)attr;
+    Batch b{};
+    for (int p = 0; p < count; ++p) {
+        b.g[p] = a[p];
+        const bool ok = (a[p].a_mn ? make_map(&b.ta[p], a[p].A, a[p].K, a[p].M, a[p].lda, UK)
+                                   : make_map(&b.ta[p], a[p].A, a[p].M, a[p].K, a[p].lda, UM)) &&
+                        (a[p].b_mn ? make_map(&b.tb[p], a[p].B, a[p].K, a[p].N, a[p].ldb, UK)
+                                   : make_map(&b.tb[p], a[p].B, a[p].N, a[p].K, a[p].ldb, UN));
+        if (!ok) return (int)cudaErrorInvalidValue;
+    }
+    b.items0 = (int)item_count(a[0], UN);
+    b.items = b.items0 + (count > 1 ? (int)item_count(a[1], UN) : 0);
+    umma_kernel<UN, TWO><<<(unsigned)std::min(b.items, sm_count()), THREADS, Shape<UN>::SMEM, s>>>(b);
+    return (int)cudaGetLastError();
+}
+
 }  // namespace
 
-int umma_gemm(const UmmaArgs &a, void *stream) {
+int umma_tile_n(const UmmaArgs *a, int count) {
+    for (int un : {256, 128}) {
+        long items = 0;
+        bool fits = true;
+        for (int p = 0; p < count; ++p) {
+            items += item_count(a[p], un);
+            fits = fits && a[p].N % un == 0;
+        }
+        if (fits && 4 * items >= 3l * sm_count()) return un;
+    }
+    return 64;
+}
+
+int umma_gemm(const UmmaArgs *a, int count, void *stream) {
+    if (count < 1 || count > 2) return (int)cudaErrorInvalidValue;
+    for (int p = 0; p < count; ++p) {
+        if (!umma_shape_ok(a[p])) return (int)cudaErrorInvalidValue;
+        if (a[p].M <= 0) return 0;
+    }
+    const int un = umma_tile_n(a, count);
     cudaStream_t s = (cudaStream_t)stream;
-    if (!umma_shape_ok(a)) return (int)cudaErrorInvalidValue;
-    if (a.M <= 0) return 0;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UMMA_SMEM);
-        if (e) return (int)e;
-        attr = true;
-    }
-    CUtensorMap ta, tb;
-    if (!make_map(&ta, a.A, a.M, a.K, a.lda, UM) || !make_map(&tb, a.B, a.N, a.K, a.ldb, UN))
-        return (int)cudaErrorInvalidValue;
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) || sms < 1) sms = 1;
-    }
-    const long tiles = (long)((a.M + UM - 1) / UM) * (a.N / UN);
-    umma_kernel<<<(unsigned)std::min<long>(tiles, sms), THREADS, UMMA_SMEM, s>>>(ta, tb, a);
-    return (int)cudaGetLastError();
+    if (count == 1)
+        return un == 256 ? launch<256, false>(a, 1, s) : un == 128 ? launch<128, false>(a, 1, s) : launch<64, false>(a, 1, s);
+    return un == 256 ? launch<256, true>(a, 2, s) : un == 128 ? launch<128, true>(a, 2, s) : launch<64, true>(a, 2, s);
 }
 
 }  // namespace hedl
