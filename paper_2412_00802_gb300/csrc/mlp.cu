@@ -598,13 +598,21 @@ __global__ void stat_kernel(const float *scores, uint32_t n, int32_t *out) {
         out[i] = (int32_t)rint(((double)scores[2 * i] - 0.5) * 32.0);
 }
 
+// a / b in double, rounded to float.  Below 2^24 both are exact floats, and the
+// FP32 quotient is the same value: a quotient of 24-bit integers is either a
+// float, or further from every midpoint of two floats than double's rounding
+// moves it.  (FP64 divides run at a small fraction of the FP32 rate here.)
+__device__ __forceinline__ float ratio(uint64_t a, uint64_t b) {
+    if (b < (1u << 24) && a < (1u << 24)) return __fdiv_rn((float)(uint32_t)a, (float)(uint32_t)b);
+    return (float)((double)a / (double)b);
+}
+
 __global__ void scores_kernel(const uint32_t *counts, uint32_t H, float *T) {
     for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < H; h += gridDim.x * blockDim.x) {
         const uint4 c = reinterpret_cast<const uint4 *>(counts)[h];
-        const double tot = (double)c.x + c.y + c.z + c.w;
-        const double den = 2.0 * c.x + c.y + c.z;
-        T[2 * h] = tot > 0 ? (float)(((double)c.x + c.w) / tot) : 0.f;
-        T[2 * h + 1] = den > 0 ? (float)(2.0 * c.x / den) : 0.f;
+        const uint64_t tot = (uint64_t)c.x + c.y + c.z + c.w, den = 2ull * c.x + c.y + c.z;
+        T[2ull * h] = tot > 0 ? ratio((uint64_t)c.x + c.w, tot) : 0.f;
+        T[2ull * h + 1] = den > 0 ? ratio(2ull * c.x, den) : 0.f;
     }
 }
 
@@ -617,98 +625,204 @@ __device__ __forceinline__ uint32_t order_key(float x) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// A radix select over 64-bit keys (accuracy key << 32 | F1 key) finds the
-// k-th largest key 8 bits at a time; a single-block stable compaction then
-// picks every larger key and, among equal keys, the lowest indices.
-__global__ void keys_kernel(const float *Y, uint32_t H, unsigned long long *keys) {
-    for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < H; h += gridDim.x * blockDim.x)
-        keys[h] = ((unsigned long long)order_key(Y[2 * h]) << 32) | order_key(Y[2 * h + 1]);
+// The k best of H predictions by a radix select over 64-bit keys (accuracy key
+// << 32 | F1 key), in one launch of one cluster of SEL_CTAS blocks; ties go to
+// the lowest indices, and the indices come out ascending.
+//
+// Block r owns a contiguous range of the predictions and walks it in tiles of
+// SEL_TILE keys in shared memory; up to SEL_CTAS * SEL_TILE predictions (a
+// ranking round's 65,536) a block's range is one tile, read from memory once.
+//   1. The bits in which any key differs from the first one: leading bits that
+//      all share (sign, most of the exponent) need no pass.
+//   2. Up to 10 bits a pass: each block counts its keys that match the bits
+//      chosen so far, the cluster adds the counts through distributed shared
+//      memory, and every block picks the digit of the k-th largest key by a
+//      scan over the 1,024 bins.  A pass ends the search once every key of the
+//      chosen bin is wanted.
+//   3. Each block's picks are counted, their offsets follow from the blocks
+//      before it, and a scan over the tile places them in index order.
+// The cluster's barrier replaces a launch: the eight passes of 8 bits had been
+// 16 launches whose digit was picked by one thread (11 us each), and the
+// compaction one block's walk over all keys (71 us): 171 us at 65,536
+// predictions with the scores, 31 us now, most of it two launches and a few
+// microseconds a pass.
+constexpr uint32_t SEL_CTAS = 8, SEL_THREADS = 1024, SEL_PER = 8, SEL_TILE = SEL_THREADS * SEL_PER;
+constexpr uint32_t SEL_BITS = 10, SEL_BINS = 1u << SEL_BITS, SEL_COPIES = 4;
+struct SelSmem {
+    unsigned long long key[SEL_TILE + SEL_TILE / SEL_PER];   // key i at i + i / SEL_PER: no 8-way bank conflicts
+    uint32_t hist[SEL_COPIES][SEL_BINS];                     // the block's counts, a copy per few warps
+    uint32_t sum[2][SEL_BINS];                               // ... added up, read by the cluster (two passes apart)
+    uint32_t warp_sum[32];
+    unsigned long long diff;                                 // bits in which some key differs from the first
+    uint32_t n_gt, n_eq;                                     // the block's picks
+    uint32_t digit, left, in_bin;
+};
+static_assert(SEL_BINS == SEL_THREADS, "a thread owns a bin");
+
+__device__ __forceinline__ uint32_t cluster_peer(const void *p, uint32_t rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ uint32_t ld_peer(const uint32_t *p, uint32_t rank) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_peer(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long ld_peer(const unsigned long long *p, uint32_t rank) {
+    unsigned long long v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(cluster_peer(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// One pass of the radix select: histogram of the 8 bits at `shift` among the
-// keys whose bits above shift+8 equal the prefix chosen so far (*prefix).
-__global__ void radix_hist_kernel(const unsigned long long *keys, uint32_t H, const unsigned long long *prefix,
-                                  int shift, uint32_t *hist) {
-    __shared__ uint32_t sh[256];
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) sh[i] = 0;
-    __syncthreads();
-    const unsigned long long pmask = shift >= 56 ? 0ull : ~((1ull << (shift + 8)) - 1ull);
-    const unsigned long long pre = *prefix & pmask;
-    for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < H; h += gridDim.x * blockDim.x) {
-        const unsigned long long k = keys[h];
-        if ((k & pmask) == pre) atomicAdd(&sh[(k >> shift) & 0xFF], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x)
-        if (sh[i]) atomicAdd(&hist[i], sh[i]);
-}
-
-// state[0..1] = prefix (64 bits), state[2] = k remaining; picks the bucket
-// holding the k-th largest and narrows the prefix.
-__global__ void radix_pick_kernel(uint32_t *hist, int shift, unsigned long long *state_prefix, uint32_t *state_k) {
-    if (threadIdx.x != 0) return;
-    uint32_t k = *state_k;
-    for (int b = 255; b >= 0; --b) {
-        if (hist[b] >= k) {
-            *state_prefix |= ((unsigned long long)b << shift);
-            break;
-        }
-        k -= hist[b];
-    }
-    *state_k = k;
-    for (int b = 0; b < 256; ++b) hist[b] = 0;
-}
-
-// Stable selection: every key > thr, then the first `ties` keys == thr in
-// index order; output sorted by index.  One block, chunked prefix sums.
-__global__ void select_kernel(const unsigned long long *keys, uint32_t H, const unsigned long long *thr_p,
-                              const uint32_t *ties_p, uint32_t *out) {
-    __shared__ uint32_t warp_sums[32];
-    __shared__ uint32_t base_gt, base_eq;
-    const unsigned long long thr = *thr_p;
-    const uint32_t ties = *ties_p;
-    if (threadIdx.x == 0) base_gt = base_eq = 0;
-    __syncthreads();
-    // output in index order: a picked key's position is (#greater before it) + min(#equal before it, ties)
-    for (uint32_t c0 = 0; c0 < H; c0 += blockDim.x) {
-        const uint32_t h = c0 + threadIdx.x;
-        const unsigned long long k = h < H ? keys[h] : 0ull;
-        const uint32_t gt = (h < H && k > thr) ? 1u : 0u;
-        const uint32_t eq = (h < H && k == thr) ? 1u : 0u;
-        // block-wide exclusive scans of gt and eq (packed 16/16 bits per chunk of <= 1024)
-        uint32_t v = gt | (eq << 16);
-        const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        uint32_t incl = v;
+// Exclusive prefix sum of v over the block's threads; *total receives the sum.
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t *warp_sum, uint32_t *total) {
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    uint32_t incl = v;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= (uint32_t)o) incl += t;
-        }
-        if (lane == 31) warp_sums[w] = incl;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (uint32_t)o) incl += t;
+    }
+    __syncthreads();   // warp_sum may still be read from the scan before
+    if (lane == 31) warp_sum[w] = incl;
+    __syncthreads();
+    uint32_t x = warp_sum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= (uint32_t)o) x += t;
+    }
+    *total = __shfl_sync(0xFFFFFFFFu, x, 31);
+    const uint32_t before = w ? __shfl_sync(0xFFFFFFFFu, x, (int)(w - 1)) : 0u;
+    return before + incl - v;
+}
+
+__global__ void __cluster_dims__(SEL_CTAS, 1, 1) __launch_bounds__(SEL_THREADS)
+    select_kernel(const float *__restrict__ Y, uint32_t H, uint32_t k, uint32_t *out) {
+    extern __shared__ __align__(16) uint8_t sel_raw[];
+    SelSmem &sm = *reinterpret_cast<SelSmem *>(sel_raw);
+    const uint32_t tid = threadIdx.x, rank = blockIdx.x;   // one cluster: the block's rank in it
+    // the block's range, in whole tiles where there are several
+    uint64_t per = ((uint64_t)H + SEL_CTAS - 1) / SEL_CTAS;
+    if (per > SEL_TILE) per = (per + SEL_TILE - 1) / SEL_TILE * SEL_TILE;
+    const uint64_t lo = min((uint64_t)H, rank * per), hi = min((uint64_t)H, lo + per);
+    const bool one_tile = per <= SEL_TILE;
+    auto make_key = [&](uint64_t i) {
+        return ((unsigned long long)order_key(Y[2 * i]) << 32) | order_key(Y[2 * i + 1]);
+    };
+    auto slot = [](uint32_t i) { return i + i / SEL_PER; };
+    // the tile's keys, coalesced; the barrier before it protects the tile read before
+    auto load_tile = [&](uint64_t t0) {
+        const uint32_t n = (uint32_t)min((uint64_t)SEL_TILE, hi - t0);
         __syncthreads();
-        if (w == 0) {
-            const uint32_t nw = (blockDim.x + 31) / 32;
-            uint32_t x = lane < nw ? warp_sums[lane] : 0u;
-            uint32_t y = x;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, y, o);
-                if (lane >= (uint32_t)o) y += t;
+        for (uint32_t i = tid; i < n; i += SEL_THREADS) sm.key[slot(i)] = make_key(t0 + i);
+        __syncthreads();
+        return n;
+    };
+    const unsigned long long key0 = make_key(0);
+    if (tid == 0) sm.diff = 0ull, sm.n_gt = sm.n_eq = 0u;
+    for (uint32_t i = tid; i < SEL_COPIES * SEL_BINS; i += SEL_THREADS) (&sm.hist[0][0])[i] = 0u;
+
+    unsigned long long diff = 0ull;
+    for (uint64_t t0 = lo; t0 < hi; t0 += SEL_TILE) {
+        const uint32_t n = load_tile(t0);
+        for (uint32_t i = tid; i < n; i += SEL_THREADS) diff |= sm.key[slot(i)] ^ key0;
+    }
+    __syncthreads();
+    const uint32_t dh = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)(diff >> 32));
+    const uint32_t dl = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)diff);
+    if ((tid & 31u) == 0) atomicOr(&sm.diff, ((unsigned long long)dh << 32) | dl);
+    cluster_barrier();
+    diff = 0ull;
+    for (uint32_t r = 0; r < SEL_CTAS; ++r) diff |= ld_peer(&sm.diff, r);
+    uint32_t rb = diff ? 64u - (uint32_t)__clzll((long long)diff) : 0u;   // low bits still open
+    unsigned long long prefix = rb >= 64u ? 0ull : (key0 >> rb) << rb;
+    uint32_t left = k;       // wanted among the keys that match the prefix
+    bool whole = false;      // all of them are wanted
+    for (uint32_t pass = 0; rb > 0u && !whole; ++pass) {
+        const uint32_t w = min(SEL_BITS, rb), shift = rb - w, mask = (1u << w) - 1u;
+        uint32_t *mine = sm.hist[(tid >> 5) % SEL_COPIES];
+        for (uint64_t t0 = lo; t0 < hi; t0 += SEL_TILE) {
+            const uint32_t n = one_tile ? (uint32_t)(hi - lo) : load_tile(t0);
+            for (uint32_t i = tid; i < n; i += SEL_THREADS) {
+                const unsigned long long x = sm.key[slot(i)];
+                if (rb >= 64u || (x >> rb) == (prefix >> rb)) atomicAdd(&mine[(uint32_t)(x >> shift) & mask], 1u);
             }
-            if (lane < nw) warp_sums[lane] = y - x;   // exclusive per warp
         }
         __syncthreads();
-        const uint32_t excl = incl - v + warp_sums[w];
-        const uint32_t gt_before = base_gt + (excl & 0xFFFF), eq_before = base_eq + (excl >> 16);
-        if (gt) out[gt_before + min(eq_before, ties)] = h;
-        if (eq && eq_before < ties) out[gt_before + eq_before] = h;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) {
-            base_gt += ((excl + v) & 0xFFFF);
-            base_eq += ((excl + v) >> 16);
+        uint32_t own = 0;
+#pragma unroll
+        for (uint32_t c = 0; c < SEL_COPIES; ++c) {
+            own += sm.hist[c][tid];
+            sm.hist[c][tid] = 0u;
         }
+        sm.sum[pass & 1u][tid] = own;
+        cluster_barrier();
+        // thread t owns bin SEL_BINS - 1 - t, so that a prefix sum counts the larger keys
+        const uint32_t bin = SEL_BINS - 1u - tid;
+        uint32_t cnt = 0;
+#pragma unroll
+        for (uint32_t r = 0; r < SEL_CTAS; ++r) cnt += ld_peer(&sm.sum[pass & 1u][bin], r);
+        uint32_t total;
+        const uint32_t larger = block_scan(cnt, sm.warp_sum, &total);
+        if (larger < left && left <= larger + cnt) sm.digit = bin, sm.left = left - larger, sm.in_bin = cnt;
+        __syncthreads();
+        prefix |= (unsigned long long)sm.digit << shift;
+        left = sm.left;
+        whole = left == sm.in_bin;
+        rb = shift;
         __syncthreads();
     }
+    // picks: keys above the prefix's range and, of those inside, all (whole) or the first `left`
+    const unsigned long long span = rb >= 64u ? ~0ull : (1ull << rb) - 1ull;
+    auto above = [&](unsigned long long x) { return whole ? x >= prefix : x > (prefix | span); };
+    auto inside = [&](unsigned long long x) { return !whole && x >= prefix && x <= (prefix | span); };
+    uint32_t gt = 0, eq = 0;
+    for (uint64_t t0 = lo; t0 < hi; t0 += SEL_TILE) {
+        const uint32_t n = one_tile ? (uint32_t)(hi - lo) : load_tile(t0);
+        for (uint32_t i = tid; i < n; i += SEL_THREADS) {
+            const unsigned long long x = sm.key[slot(i)];
+            gt += above(x), eq += inside(x);
+        }
+    }
+    gt = __reduce_add_sync(0xFFFFFFFFu, gt), eq = __reduce_add_sync(0xFFFFFFFFu, eq);
+    if ((tid & 31u) == 0 && (gt | eq)) atomicAdd(&sm.n_gt, gt), atomicAdd(&sm.n_eq, eq);
+    cluster_barrier();
+    uint32_t gt_before = 0, eq_before = 0;
+    for (uint32_t r = 0; r < rank; ++r) gt_before += ld_peer(&sm.n_gt, r), eq_before += ld_peer(&sm.n_eq, r);
+    // a picked key's place: the larger keys before it + the equal ones before it that are taken
+    for (uint64_t t0 = lo; t0 < hi; t0 += SEL_TILE) {
+        const uint32_t n = one_tile ? (uint32_t)(hi - lo) : load_tile(t0);
+        uint32_t g = 0, e = 0;
+#pragma unroll
+        for (uint32_t q = 0; q < SEL_PER; ++q) {
+            const uint32_t i = tid * SEL_PER + q;
+            if (i < n) {
+                const unsigned long long x = sm.key[slot(i)];
+                g += above(x), e += inside(x);
+            }
+        }
+        uint32_t total;
+        const uint32_t before = block_scan(g | e << 16, sm.warp_sum, &total);   // at most 8,192 each
+        uint32_t pg = gt_before + (before & 0xFFFFu), pe = eq_before + (before >> 16);
+#pragma unroll
+        for (uint32_t q = 0; q < SEL_PER; ++q) {
+            const uint32_t i = tid * SEL_PER + q;
+            if (i >= n) break;
+            const unsigned long long x = sm.key[slot(i)];
+            if (above(x)) out[pg++ + min(pe, left)] = (uint32_t)(t0 + i);
+            else if (inside(x)) {
+                if (pe < left) out[pg + pe] = (uint32_t)(t0 + i);
+                ++pe;
+            }
+        }
+        gt_before += total & 0xFFFFu, eq_before += total >> 16;
+    }
+    cluster_barrier();   // no block leaves while another may still read its counts
 }
 
 }  // namespace
@@ -1087,23 +1201,11 @@ int hedl_select_top(const float *Y, uint32_t H, uint32_t k, uint32_t *idx, void 
     if (!Y || !idx) return fail(HEDL_ERR_INVALID_ARG, "NULL argument");
     if (k == 0 || k > H) return fail(HEDL_ERR_INVALID_ARG, "k must be in 1..H");
     if (!ws || ws_bytes < 8ull * H + 4096 + 256) return fail(HEDL_ERR_WORKSPACE_TOO_SMALL, "select workspace too small");
-    cudaStream_t st = (cudaStream_t)s;
-    uint8_t *p = (uint8_t *)ws;
-    auto *keys = (unsigned long long *)p;
-    uint8_t *q = p + ((8ull * H + 255) & ~255ull);
-    auto *hist = (uint32_t *)q;                          // 256 words
-    auto *prefix = (unsigned long long *)(q + 1024);     // the k-th largest key, built 8 bits at a time
-    auto *krem = (uint32_t *)(q + 1032);                 // rank still sought within the prefix
-    cudaError_t e = cudaMemsetAsync(q, 0, 2048, st);
-    if (!e) e = cudaMemcpyAsync(krem, &k, 4, cudaMemcpyHostToDevice, st);
-    if (e) return cuda_fail(e, "select setup");
-    keys_kernel<<<grid1(H), 256, 0, st>>>(Y, H, keys);
-    for (int shift = 56; shift >= 0; shift -= 8) {
-        radix_hist_kernel<<<grid1(H), 256, 0, st>>>(keys, H, prefix, shift, hist);
-        radix_pick_kernel<<<1, 32, 0, st>>>(hist, shift, prefix, krem);
-    }
-    select_kernel<<<1, 1024, 0, st>>>(keys, H, prefix, krem, idx);
-    e = cudaGetLastError();
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SelSmem));
+    if (attr) return cuda_fail(attr, "select setup");
+    select_kernel<<<SEL_CTAS, SEL_THREADS, sizeof(SelSmem), (cudaStream_t)s>>>(Y, H, k, idx);
+    cudaError_t e = cudaGetLastError();
     return e ? cuda_fail(e, "select launch") : HEDL_OK;
 }
 
