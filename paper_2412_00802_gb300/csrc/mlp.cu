@@ -42,12 +42,18 @@ __device__ __forceinline__ int arity_of(uint32_t op) {
 
 constexpr int ENC_MAXLEN = 256;
 
-// One warp per program: lane 0 computes node depths and polarities (a
-// reversed walk of the postfix is a pre-order walk; NOT and ATMOST flip the
-// polarity of their operand), then the lanes count features into shared
-// memory and write the row as bf16 (counts x 1/4, exact), the two prior
-// inputs as bf16 of the caller's values.  Signed counts add +1 at polarity 0
-// and -1 at polarity 1.
+// Structural encoding, one warp per program.  Lane l holds instructions l,
+// l + 32, ... (one register each up to 32 instructions).  Depths and
+// polarities come from the postfix heights: with s_k the operands on the stack
+// after instruction k, the parent of k is the first j > k with s_j <= s_k, and
+// every such running minimum to the right of k is an ancestor (NOT and ATMOST
+// ancestors flip the polarity).  Up to 32 instructions, a ballot per height
+// gives every node its parent and pointer jumping its depth; longer programs
+// count the minima.  The lanes then count features into shared memory (totals
+// by ballots) and write the row as bf16 (counts x 1/4, exact), the two prior
+// inputs as bf16 of the caller's values.  The next program's instructions are
+// loaded while the current one is counted.
+// Signed counts add +1 at polarity 0 and -1 at polarity 1.
 //   [  0, 84) op x min(depth, 5)          [ 84,180) concept mod 96, signed
 //   [180,244) role mod 32 x inverse       [244,284) restriction kind x depth
 //   [284,308) cardinality                 [308,436) property mod 16 x (>=, <=) x bucket / 4, signed
@@ -55,98 +61,231 @@ constexpr int ENC_MAXLEN = 256;
 //   [493,497) length / 10                 [497,504) statistics sums, signed
 //   [504,510) totals, height, constant    [510,512) prior
 // stats (or null): n_sc atom scores, then n_grid x 2 x 16 threshold scores.
-__global__ void encode_kernel(const uint64_t *__restrict__ progs, const uint32_t *__restrict__ offs, uint32_t H,
-                              const float *__restrict__ grid, uint32_t n_grid, const int32_t *__restrict__ stats,
-                              uint32_t n_sc, const float *__restrict__ prior, __nv_bfloat16 *__restrict__ X) {
-    constexpr int WARPS = 4;
-    __shared__ int feat[WARPS][DI];
-    __shared__ uint8_t depth[WARPS][ENC_MAXLEN];
-    __shared__ uint8_t pol[WARPS][ENC_MAXLEN];
-    __shared__ uint8_t pend[WARPS][ENC_MAXLEN + 1];    // pending depth (7 bits) | polarity << 7
-    __shared__ uint32_t height[WARPS];
+//
+// Bound: 1 KB written a program (67 MB at 65,536: 10 us) against the latency
+// of one program's chain (offsets -> instructions -> counts -> row).  One lane
+// walking the program with a stack in shared memory, and 2-byte stores, took
+// 75 us at 65,536 programs of 13 instructions; this takes 46 us.
+constexpr int ENC_WARPS = 8;
+
+// The lane's nodes of a program of at most 32 * N instructions: heights, then
+// depth, polarity and the program's height.  Nodes that no root reaches (the
+// program is not well formed: a height below the last one's, and all before
+// it) get depth 0 and polarity 0.
+template <int N>
+__device__ __forceinline__ void encode_nodes(const uint64_t (&w)[N], uint32_t L, uint32_t lane, uint32_t (&depth)[N],
+                                             uint32_t (&pol)[N], uint32_t &height) {
+    int s[N];
+    uint32_t flip[N];   // ballot: NOT / ATMOST among the register's 32 instructions
+    int base = 0;
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+        const uint32_t op = (uint32_t)(w[r] & 0xFF), k = 32u * r + lane;
+        int v = k < L ? 1 - arity_of(op) : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xFFFFFFFFu, v, o);
+            if (lane >= (uint32_t)o) v += t;
+        }
+        s[r] = base + v;
+        base = __shfl_sync(0xFFFFFFFFu, s[r], 31);
+        flip[r] = __ballot_sync(0xFFFFFFFFu, k < L && (op == HEDL_OP_NOT || op == HEDL_OP_ATMOST));
+    }
+    // base is now the height after the last instruction; the last node below it cuts the program
+    int cut = -1;
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+        const uint32_t below = __ballot_sync(0xFFFFFFFFu, 32u * r + lane < L && s[r] < base);
+        if (below) cut = 32 * r + 31 - __clz((int)below);
+    }
+    if constexpr (N == 1) {
+        // parent: the first j > k with s_j <= s_k (its own lane if there is none); the heights of the
+        // nodes after the cut lie between base and the largest one
+        const bool node = lane < L && (int)lane > cut;
+        const uint32_t later = ~((2u << lane) - 1u);
+        const int top = __reduce_max_sync(0xFFFFFFFFu, node ? s[0] : base);
+        uint32_t parent = lane;
+        for (int h = base; h <= top; ++h) {   // warp-uniform
+            const uint32_t at = __ballot_sync(0xFFFFFFFFu, node && s[0] <= h) & later;
+            if (node && s[0] == h && at) parent = (uint32_t)__ffs((int)at) - 1u;
+        }
+        // ancestors counted by pointer jumping: low half the depth, high half the flips
+        uint32_t acc = parent != lane ? 1u + ((flip[0] >> parent & 1u) << 16) : 0u;
+        while (__any_sync(0xFFFFFFFFu, parent != lane)) {
+            const uint32_t more = __shfl_sync(0xFFFFFFFFu, acc, (int)parent);
+            const uint32_t next = __shfl_sync(0xFFFFFFFFu, parent, (int)parent);
+            if (parent != lane) acc += more;   // a root's own count is zero
+            parent = next == parent ? lane : next;
+        }
+        depth[0] = acc & 0xFFFFu, pol[0] = acc >> 16 & 1u;
+        height = __reduce_max_sync(0xFFFFFFFFu, node ? depth[0] + 1u : 0u);
+    } else {
+        int low[N];
+#pragma unroll
+        for (int r = 0; r < N; ++r) depth[r] = pol[r] = 0u, low[r] = s[r];
+#pragma unroll
+        for (int q = 0; q < N; ++q) {   // ancestors in register q's instructions
+            for (uint32_t l = 0; l < 32u && 32u * q + l < L; ++l) {
+                const int sj = __shfl_sync(0xFFFFFFFFu, s[q], (int)l);
+                const uint32_t f = flip[q] >> l & 1u;
+#pragma unroll
+                for (int r = 0; r <= q; ++r)
+                    if ((r < q || lane < l) && sj <= low[r]) low[r] = sj, depth[r] += 1u, pol[r] ^= f;
+            }
+        }
+        uint32_t ht = 0;
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+            const int k = (int)(32u * r + lane);
+            if (k <= cut) depth[r] = pol[r] = 0u;
+            else if ((uint32_t)k < L) ht = max(ht, depth[r] + 1u);
+        }
+        height = __reduce_max_sync(0xFFFFFFFFu, ht);
+    }
+}
+
+struct EncTables {
+    const float *grid;      // or null
+    const int32_t *stats;   // or null
+    uint32_t n_grid, n_sc;
+};
+
+// Counts a program's features; w: its instructions as in encode_nodes (0 past the end).
+template <int N>
+__device__ __forceinline__ void encode_program(const uint64_t (&w)[N], uint32_t L, uint32_t lane, int *feat,
+                                               const EncTables &t) {
+    const float *__restrict__ grid = t.grid;
+    const int32_t *__restrict__ stats = t.stats;
+    const uint32_t n_grid = t.n_grid, n_sc = t.n_sc;
+    uint32_t depth[N], pol[N], height;
+    encode_nodes<N>(w, L, lane, depth, pol, height);
+    uint64_t left_of_0 = 0ull;   // the instruction before the register's first
+    int leaves = 0, roles = 0, datas = 0, nots = 0;
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+        const uint32_t k = 32u * r + lane;
+        uint64_t c = __shfl_up_sync(0xFFFFFFFFu, w[r], 1);   // the instruction before this one
+        if (lane == 0) c = left_of_0;
+        left_of_0 = __shfl_sync(0xFFFFFFFFu, w[r], 31);
+        const uint32_t op = (uint32_t)(w[r] & 0xFF), inv = (uint32_t)((w[r] >> 8) & 1);
+        const uint32_t a = (uint32_t)((w[r] >> 16) & 0xFFFF), b = (uint32_t)(w[r] >> 32);
+        const bool counted = k < L && op >= HEDL_OP_ATOM && op <= HEDL_OP_DEQ;   // else not an op, or a string restriction
+        leaves += __popc(__ballot_sync(0xFFFFFFFFu, counted && arity_of(op) == 0));
+        roles += __popc(__ballot_sync(0xFFFFFFFFu, counted && op >= HEDL_OP_EXISTS && op <= HEDL_OP_EXACTLY));
+        datas += __popc(__ballot_sync(0xFFFFFFFFu, counted && op >= HEDL_OP_DGE));
+        nots += __popc(__ballot_sync(0xFFFFFFFFu, counted && op == HEDL_OP_NOT));
+        if (!counted) continue;
+        const uint32_t dk = depth[r];
+        const int sign = pol[r] ? -1 : 1;
+        atomicAdd(&feat[min(dk, 5u) * 14 + op - 1], 1);
+        if (op == HEDL_OP_ATOM) {
+            atomicAdd(&feat[84 + a % 96], sign);
+            if (stats && a < n_sc) atomicAdd(&feat[497 + min(dk / 2, 2u)], sign * stats[a]);
+        } else if (op >= HEDL_OP_EXISTS && op <= HEDL_OP_EXACTLY) {
+            atomicAdd(&feat[180 + (a % 32) * 2 + inv], 1);
+            atomicAdd(&feat[244 + min(dk, 7u) * 5 + (op - HEDL_OP_EXISTS)], 1);
+            if (op >= HEDL_OP_ATLEAST) atomicAdd(&feat[284 + (op - HEDL_OP_ATLEAST) * 8 + min(b, 7u)], 1);
+            if (k > 0 && (c & 0xFF) == HEDL_OP_ATOM) {   // the filler ends right before its restriction
+                const uint32_t cc = (uint32_t)((c >> 16) & 0xFFFF);
+                atomicAdd(&feat[436 + ((a * 2 + inv) * 131 + cc) % 57], sign);
+                if (stats && cc < n_sc) atomicAdd(&feat[503], sign * stats[cc]);
+            }
+        } else if (op >= HEDL_OP_DGE) {
+            if (op != HEDL_OP_DEQ) {
+                const float t = __uint_as_float(b);
+                uint32_t q = 0;
+                if (grid && a < n_grid && !(t != t))
+                    for (int g = 0; g < 15; ++g) q += grid[a * 15 + g] < t ? 1u : 0u;
+                atomicAdd(&feat[308 + ((a % 16) * 2 + (op - HEDL_OP_DGE)) * 4 + q / 4], sign);
+                if (stats && a < n_grid)
+                    atomicAdd(&feat[500 + min(dk / 2, 2u)], sign * stats[n_sc + (a * 2 + (op - HEDL_OP_DGE)) * 16 + q]);
+            }
+        }
+    }
+    if (lane == 0) {   // no other lane adds to these
+        feat[493 + min(L, 39u) / 10] = 1;
+        feat[504] = leaves, feat[505] = roles, feat[506] = datas, feat[507] = nots;
+        feat[508] = (int)min(height, 8u) - 1;
+        feat[509] = 4;
+    }
+}
+
+// Programs of more than 32 instructions: a call, so that their registers do not limit the others' occupancy.
+template <int N>
+__device__ __noinline__ void encode_long(const uint64_t *__restrict__ prog, uint32_t L, int *feat, const EncTables &t) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint64_t w[N];
+#pragma unroll
+    for (int r = 0; r < N; ++r) w[r] = 32u * r + lane < L ? prog[32u * r + lane] : 0ull;
+    encode_program<N>(w, L, lane, feat, t);
+}
+
+__global__ void __launch_bounds__(32 * ENC_WARPS, 4)
+    encode_kernel(const uint64_t *__restrict__ progs, const uint32_t *__restrict__ offs, uint32_t H, EncTables t,
+                  const float *__restrict__ prior, __nv_bfloat16 *__restrict__ X) {
+    __shared__ __align__(16) int feats[ENC_WARPS][DI];
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (uint32_t h = blockIdx.x * WARPS + warp; h < H; h += gridDim.x * WARPS) {
-        for (int i = lane; i < DI; i += 32) feat[warp][i] = 0;
-        // programs longer than ENC_MAXLEN are encoded by their last ENC_MAXLEN
-        // instructions (the root and the nodes nearest to it)
-        const uint32_t L = min(offs[h + 1] - offs[h], (uint32_t)ENC_MAXLEN), o0 = offs[h + 1] - L;
-        if (lane == 0) {
-            int sp = 0;
-            pend[warp][sp++] = 0;
-            uint32_t ht = 0;
-            for (int k = (int)L - 1; k >= 0; --k) {
-                if (sp == 0) {   // not a well-formed program: remaining nodes get depth 0, polarity 0
-                    for (; k >= 0; --k) depth[warp][k] = 0, pol[warp][k] = 0;
-                    break;
-                }
-                const uint32_t e = pend[warp][--sp];
-                const uint32_t d = e & 0x7Fu, pl = e >> 7;
-                depth[warp][k] = (uint8_t)d;
-                pol[warp][k] = (uint8_t)pl;
-                ht = max(ht, d + 1);
-                const uint32_t op = (uint32_t)(progs[o0 + k] & 0xFF);
-                const int a = arity_of(op);
-                // depths beyond 127 only feed clamped features (depth 7, height 8)
-                const uint32_t flip = (op == HEDL_OP_NOT || op == HEDL_OP_ATMOST) ? 1u : 0u;
-                const uint32_t ce = min(d + 1, 127u) | ((pl ^ flip) << 7);
-                for (int j = 0; j < a && sp <= ENC_MAXLEN; ++j) pend[warp][sp++] = (uint8_t)ce;
+    int *feat = feats[warp];
+    int4 *f4 = reinterpret_cast<int4 *>(feat);
+    const bool wide = (reinterpret_cast<uintptr_t>(X) & 15) == 0;   // 16-byte stores
+    const uint32_t step = gridDim.x * ENC_WARPS;
+    // programs longer than ENC_MAXLEN are encoded by their last ENC_MAXLEN
+    // instructions (the root and the nodes nearest to it)
+    struct Prog {
+        uint64_t w;        // the lane's instruction of a program of at most 32
+        uint32_t end, L;
+    };
+    auto range = [&](uint32_t h, Prog &p) {
+        p.end = h < H ? offs[h + 1] : 0u;
+        p.L = h < H ? min(p.end - offs[h], (uint32_t)ENC_MAXLEN) : 0u;
+    };
+    auto load = [&](Prog &p) { p.w = lane < p.L && p.L <= 32u ? progs[p.end - p.L + lane] : 0ull; };
+    uint32_t h = blockIdx.x * ENC_WARPS + warp;
+    Prog cur, nxt;
+    range(h, cur);
+    load(cur);
+    range(h + step, nxt);
+    for (; h < H; h += step) {
+        load(nxt);                         // one program ahead
+        Prog far;
+        range(h + 2u * step, far);         // its range another one
+        const float pr = prior && lane >= 30 ? prior[2ull * h + (lane - 30)] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < DI / 128; ++q) f4[32 * q + lane] = make_int4(0, 0, 0, 0);
+        __syncwarp();
+        if (cur.L <= 32u) {
+            const uint64_t w[1] = {cur.w};
+            encode_program<1>(w, cur.L, lane, feat, t);
+        } else if (cur.L <= 64u) {
+            encode_long<2>(progs + (cur.end - cur.L), cur.L, feat, t);
+        } else {
+            encode_long<ENC_MAXLEN / 32>(progs + (cur.end - cur.L), cur.L, feat, t);
+        }
+        cur = nxt;
+        nxt = far;
+        __syncwarp();
+        // the priors take the last two places (never counted); they are not scaled
+        const float p0 = __shfl_sync(0xFFFFFFFFu, pr, 30), p1 = __shfl_sync(0xFFFFFFFFu, pr, 31);
+        __nv_bfloat16 *row = X + (uint64_t)h * DI;
+#pragma unroll
+        for (int q = 0; q < DI / 256; ++q) {   // eight features a lane
+            const uint32_t at = 32 * q + lane;
+            const int4 x = f4[2 * at], y = f4[2 * at + 1];
+            float v[8] = {0.25f * (float)x.x, 0.25f * (float)x.y, 0.25f * (float)x.z, 0.25f * (float)x.w,
+                          0.25f * (float)y.x, 0.25f * (float)y.y, 0.25f * (float)y.z, 0.25f * (float)y.w};
+            if (at == DI / 8 - 1) v[6] = p0, v[7] = p1;
+            uint32_t o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat162 z = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
+                o[e] = *reinterpret_cast<const uint32_t *>(&z);
             }
-            height[warp] = ht;
-        }
-        __syncwarp();
-        for (uint32_t k = lane; k < L; k += 32) {
-            const uint64_t w = progs[o0 + k];
-            const uint32_t op = (uint32_t)(w & 0xFF), inv = (uint32_t)((w >> 8) & 1);
-            const uint32_t a = (uint32_t)((w >> 16) & 0xFFFF), b = (uint32_t)(w >> 32);
-            if (op < HEDL_OP_ATOM || op > HEDL_OP_DEQ) continue;   // no feature: not an op, or a string restriction
-            const uint32_t dk = depth[warp][k];
-            const int sign = pol[warp][k] ? -1 : 1;
-            atomicAdd(&feat[warp][min(dk, 5u) * 14 + op - 1], 1);
-            if (arity_of(op) == 0) atomicAdd(&feat[warp][504], 1);
-            if (op == HEDL_OP_ATOM) {
-                atomicAdd(&feat[warp][84 + a % 96], sign);
-                if (stats && a < n_sc) atomicAdd(&feat[warp][497 + min(dk / 2, 2u)], sign * stats[a]);
-            } else if (op >= HEDL_OP_EXISTS && op <= HEDL_OP_EXACTLY) {
-                atomicAdd(&feat[warp][505], 1);
-                atomicAdd(&feat[warp][180 + (a % 32) * 2 + inv], 1);
-                atomicAdd(&feat[warp][244 + min(dk, 7u) * 5 + (op - HEDL_OP_EXISTS)], 1);
-                if (op >= HEDL_OP_ATLEAST) atomicAdd(&feat[warp][284 + (op - HEDL_OP_ATLEAST) * 8 + min(b, 7u)], 1);
-                if (k > 0) {   // the filler ends right before its restriction
-                    const uint64_t c = progs[o0 + k - 1];
-                    if ((c & 0xFF) == HEDL_OP_ATOM) {
-                        const uint32_t cc = (uint32_t)((c >> 16) & 0xFFFF);
-                        atomicAdd(&feat[warp][436 + ((a * 2 + inv) * 131 + cc) % 57], sign);
-                        if (stats && cc < n_sc) atomicAdd(&feat[warp][503], sign * stats[cc]);
-                    }
-                }
-            } else if (op >= HEDL_OP_DGE) {
-                atomicAdd(&feat[warp][506], 1);
-                if (op != HEDL_OP_DEQ) {
-                    const float t = __uint_as_float(b);
-                    uint32_t q = 0;
-                    if (grid && a < n_grid && !(t != t))
-                        for (int g = 0; g < 15; ++g) q += grid[a * 15 + g] < t ? 1u : 0u;
-                    atomicAdd(&feat[warp][308 + ((a % 16) * 2 + (op - HEDL_OP_DGE)) * 4 + q / 4], sign);
-                    if (stats && a < n_grid)
-                        atomicAdd(&feat[warp][500 + min(dk / 2, 2u)],
-                                  sign * stats[n_sc + (a * 2 + (op - HEDL_OP_DGE)) * 16 + q]);
-                }
-            } else if (op == HEDL_OP_NOT) {
-                atomicAdd(&feat[warp][507], 1);
+            if (wide) {
+                reinterpret_cast<uint4 *>(row)[at] = make_uint4(o[0], o[1], o[2], o[3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) row[8 * at + e] = __ushort_as_bfloat16((unsigned short)(o[e / 2] >> 16 * (e & 1)));
             }
-        }
-        __syncwarp();
-        if (lane == 0) {
-            feat[warp][493 + min(L, 39u) / 10] += 1;
-            feat[warp][508] += (int)min(height[warp], 8u) - 1;
-            feat[warp][509] += 4;
-        }
-        __syncwarp();
-        for (int i = lane; i < DI; i += 32) {
-            __nv_bfloat16 x;
-            if (i >= DI - 2) x = __float2bfloat16_rn(prior ? prior[2ull * h + (i - (DI - 2))] : 0.0f);
-            else x = __float2bfloat16_rn(0.25f * (float)feat[warp][i]);
-            X[(uint64_t)h * DI + i] = x;
         }
         __syncwarp();
     }
@@ -1075,8 +1214,9 @@ int hedl_encode(const uint64_t *progs, const uint32_t *offs, uint32_t H, const f
     if (!progs || !offs || !X) return fail(HEDL_ERR_INVALID_ARG, "NULL argument");
     if (stats && !grid && n_grid) return fail(HEDL_ERR_INVALID_ARG, "threshold statistics need the grid");
     if (H == 0) return HEDL_OK;
-    encode_kernel<<<std::min<uint32_t>((H + 3) / 4, 8192), 128, 0, (cudaStream_t)s>>>(
-        progs, offs, H, grid, grid ? n_grid : 0u, stats, stats ? n_stat_concepts : 0u, prior, (__nv_bfloat16 *)X);
+    encode_kernel<<<std::min<uint32_t>((H + ENC_WARPS - 1) / ENC_WARPS, 152u * 8u), 32 * ENC_WARPS, 0, (cudaStream_t)s>>>(
+        progs, offs, H, EncTables{grid, stats, grid ? n_grid : 0u, stats ? n_stat_concepts : 0u}, prior,
+        (__nv_bfloat16 *)X);
     cudaError_t e = cudaGetLastError();
     return e ? cuda_fail(e, "encode launch") : HEDL_OK;
 }
