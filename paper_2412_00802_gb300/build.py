@@ -20,7 +20,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libhedl.so")
 SOURCES = ["api.cu", "exec.cu", "plain.cu", "kb.cu", "noalloc.cu", "tune.cu", "mlp.cu", "umma.cu", "plan.cpp",
            "devplan.cu", "search.cpp"]
-HEADERS = ["hedl_internal.h", "device_common.cuh"]
+HEADERS = ["hedl_internal.h", "device_common.cuh", "launch.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

@@ -15,7 +15,7 @@
 // to gradients, Adam).  Every sum over the batch is first a partial sum of a
 // chunk of rows and then a sum over chunks in a fixed order, so a step's
 // gradients do not depend on timing.  At batches of 4,096 this took a step
-// from 785 us to 70 us: the weight gradient of the output layer
+// from 785 us to 61 us: the weight gradient of the output layer
 // (584 us) and the bias gradients (2 x 238 us) had been two blocks' loops over
 // the whole batch, and the weight gradients had needed four transposes.
 #include <cuda_bf16.h>
@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "hedl_internal.h"
+#include "launch.cuh"
 
 namespace hedl {
 namespace {
@@ -446,6 +447,8 @@ int gemm(const GemmArgs &a0, bool a_km, bool b_kn, int splits, cudaStream_t s) {
 // y = (u + b3), mapped back to the target scale when map is set, from the
 // fused output layer's sums u [parts][B][2] (the unfused path's out_fwd_kernel semantics).
 __global__ void out_map_kernel(const float *u, int parts, const float *b3, float *Y, int B, const float *map) {
+    pdl_trigger();
+    pdl_wait();
     for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < B; row += gridDim.x * blockDim.x) {
         float u0 = 0.f, u1 = 0.f;
         for (int p = 0; p < parts; ++p) {
@@ -534,6 +537,17 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const float *y, int parts
     __shared__ float2 du[HB_ROWS];
     const int r0 = blockIdx.x * HB_ROWS, rows = min(HB_ROWS, B - r0);
     part += (size_t)blockIdx.x * HB_PART;
+    pdl_trigger();
+    pdl_wait();
+    const int c = 2 * (int)threadIdx.x;
+    __nv_bfloat162 h[8];   // the first rows, in flight while dU is computed
+    auto fetch = [&](int r) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            h[k] = r + k < rows ? *reinterpret_cast<const __nv_bfloat162 *>(H2 + (size_t)(r0 + r + k) * DH + c)
+                                : __floats2bfloat162_rn(0.f, 0.f);
+    };
+    fetch(0);
     if (threadIdx.x < HB_ROWS) {   // one warp: a row a lane
         const int b = r0 + (int)threadIdx.x;
         float g0 = 0.f, g1 = 0.f, l = 0.f;
@@ -561,23 +575,21 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const float *y, int parts
         if (threadIdx.x == 0) part[3 * DH] = g0, part[3 * DH + 1] = g1, part[3 * DH + 2] = l;
     }
     __syncthreads();
-    const int c = 2 * (int)threadIdx.x;
     const __nv_bfloat162 wa = *reinterpret_cast<const __nv_bfloat162 *>(W3 + c);
     const __nv_bfloat162 wb = *reinterpret_cast<const __nv_bfloat162 *>(W3 + DH + c);
     const float wa0 = __low2float(wa), wa1 = __high2float(wa), wb0 = __low2float(wb), wb1 = __high2float(wb);
     float s00 = 0.f, s01 = 0.f, s10 = 0.f, s11 = 0.f, e0 = 0.f, e1 = 0.f;
 #pragma unroll 1
     for (int r = 0; r < rows; r += 8) {
-        __nv_bfloat162 h[8];
+        __nv_bfloat162 now[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-            h[k] = r + k < rows ? *reinterpret_cast<const __nv_bfloat162 *>(H2 + (size_t)(r0 + r + k) * DH + c)
-                                : __floats2bfloat162_rn(0.f, 0.f);
+        for (int k = 0; k < 8; ++k) now[k] = h[k];
+        if (r + 8 < rows) fetch(r + 8);
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             if (r + k >= rows) break;
             const float2 d = du[r + k];
-            const float h0 = __low2float(h[k]), h1 = __high2float(h[k]);
+            const float h0 = __low2float(now[k]), h1 = __high2float(now[k]);
             s00 += d.x * h0, s01 += d.x * h1;
             s10 += d.y * h0, s11 += d.y * h1;
             const float v0 = h0 > 0.f ? d.x * wa0 + d.y * wb0 : 0.f, v1 = h1 > 0.f ? d.x * wa1 + d.y * wb1 : 0.f;
@@ -666,6 +678,8 @@ __device__ __forceinline__ float adam_update(const AdamArgs &a, float g, float &
 constexpr int UP_BIG = 2 * DH * DH / 4 / 256, UP_SMALL = (4 * DH + 3 + 31) / 32;
 template <bool ADAM>
 __global__ void __launch_bounds__(256) update_kernel(GradParts p, float *g, float *loss, AdamArgs a) {
+    pdl_trigger();
+    pdl_wait();
     if (blockIdx.x < UP_BIG) {
         const int e = (int)(blockIdx.x * 256 + threadIdx.x), half = DH * DH / 4;
         const bool second = e >= half;
@@ -783,7 +797,7 @@ __device__ __forceinline__ uint32_t order_key(float x) {
 // The cluster's barrier replaces a launch: the eight passes of 8 bits had been
 // 16 launches whose digit was picked by one thread (11 us each), and the
 // compaction one block's walk over all keys (71 us): 171 us at 65,536
-// predictions with the scores, 31 us now, most of it two launches and a few
+// predictions with the scores, 30 us now, most of it two launches and a few
 // microseconds a pass.
 constexpr uint32_t SEL_CTAS = 8, SEL_THREADS = 1024, SEL_PER = 8, SEL_TILE = SEL_THREADS * SEL_PER;
 constexpr uint32_t SEL_BITS = 10, SEL_BINS = 1u << SEL_BITS, SEL_COPIES = 4;
@@ -858,7 +872,15 @@ __global__ void __cluster_dims__(SEL_CTAS, 1, 1) __launch_bounds__(SEL_THREADS)
     auto load_tile = [&](uint64_t t0) {
         const uint32_t n = (uint32_t)min((uint64_t)SEL_TILE, hi - t0);
         __syncthreads();
-        for (uint32_t i = tid; i < n; i += SEL_THREADS) sm.key[slot(i)] = make_key(t0 + i);
+        if (n == SEL_TILE) {   // all loads in flight together
+            unsigned long long x[SEL_PER];
+#pragma unroll
+            for (uint32_t q = 0; q < SEL_PER; ++q) x[q] = make_key(t0 + tid + q * SEL_THREADS);
+#pragma unroll
+            for (uint32_t q = 0; q < SEL_PER; ++q) sm.key[slot(tid + q * SEL_THREADS)] = x[q];
+        } else {
+            for (uint32_t i = tid; i < n; i += SEL_THREADS) sm.key[slot(i)] = make_key(t0 + i);
+        }
         __syncthreads();
         return n;
     };
@@ -1085,8 +1107,9 @@ int grads_impl(hedl_mlp *mlp, const __nv_bfloat16 *X, const float *T, uint32_t B
     if (e) return e;
     const int M = (int)B, splits = grad_splits(B);
     *out = GradParts{w.w1, w.w2, w.b1, w.head, splits, (M + 127) / 128, (M + HB_ROWS - 1) / HB_ROWS};
-    head_bwd_kernel<<<out->head_n, 256, 0, s>>>(w.y, parts ? parts : 1, parts ? mlp->w + OFF_B3 : nullptr,
-                                                mlp->wb + OFF_W3, T, mlp->map, w.h2, w.dh2, w.head, M);
+    e = launch_pdl(head_bwd_kernel, out->head_n, 256, 0, s, w.y, parts ? parts : 1, parts ? mlp->w + OFF_B3 : nullptr,
+                   mlp->wb + OFF_W3, T, mlp->map, w.h2, w.dh2, w.head, M);
+    if (e) return e;
     if (mlp->gemm == HEDL_GEMM_TCGEN05) {
         // dH1 = (dH2 . W2) * [H1 > 0]; W2 [out][in] is the MN-major operand
         UmmaArgs d{w.dh2, mlp->wb + OFF_W2, w.dh1, nullptr, M, DH, DH, DH, DH, DH, 0, 1, mlp->err, w.h1};
@@ -1233,9 +1256,8 @@ int hedl_mlp_forward(hedl_mlp *m, const uint16_t *X, uint32_t B, float *Y, void 
     if (!e) e = forward_impl(m, x, B, w, st, false, &parts);
     if (e) return cuda_fail(e, "mlp forward");
     const float *zero_b3 = m->map + 5;   // two zeros behind the map: b3 when w.y already has it
-    out_map_kernel<<<std::min<uint32_t>((B + 255) / 256, 148u * 8u), 256, 0, st>>>(
-        w.y, parts ? parts : 1, parts ? m->w + OFF_B3 : zero_b3, Y, (int)B, m->map);
-    e = cudaGetLastError();
+    e = launch_pdl(out_map_kernel, std::min<uint32_t>((B + 255) / 256, 152u * 8u), 256, 0, st, w.y, parts ? parts : 1,
+                   parts ? m->w + OFF_B3 : zero_b3, Y, (int)B, m->map);
     return e ? cuda_fail(e, "mlp forward") : HEDL_OK;
 }
 
@@ -1247,8 +1269,7 @@ int hedl_mlp_gradients(hedl_mlp *m, const uint16_t *X, const float *T, uint32_t 
     GradParts p;
     int e = grads_impl(m, (const __nv_bfloat16 *)X, T, B, w, (cudaStream_t)s, &p);
     if (e) return cuda_fail(e, "mlp gradients");
-    update_kernel<false><<<UP_BIG + UP_SMALL, 256, 0, (cudaStream_t)s>>>(p, m->g, loss, AdamArgs{});
-    e = cudaGetLastError();
+    e = launch_pdl(update_kernel<false>, UP_BIG + UP_SMALL, 256, 0, (cudaStream_t)s, p, m->g, loss, AdamArgs{});
     return e ? cuda_fail(e, "mlp gradients") : HEDL_OK;
 }
 
@@ -1263,9 +1284,8 @@ int hedl_mlp_train_step(hedl_mlp *m, const uint16_t *X, const float *T, uint32_t
     m->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - powf(b1, (float)m->step), c2 = 1.f - powf(b2, (float)m->step);
-    update_kernel<true><<<UP_BIG + UP_SMALL, 256, 0, (cudaStream_t)s>>>(
-        p, m->g, loss, AdamArgs{m->w, m->m, m->v, m->wb, lr, b1, b2, 1e-8f, c1, c2});
-    e = cudaGetLastError();
+    e = launch_pdl(update_kernel<true>, UP_BIG + UP_SMALL, 256, 0, (cudaStream_t)s, p, m->g, loss,
+                   AdamArgs{m->w, m->m, m->v, m->wb, lr, b1, b2, 1e-8f, c1, c2});
     return e ? cuda_fail(e, "adam launch") : HEDL_OK;
 }
 

@@ -39,6 +39,7 @@
 #include <cuda_runtime.h>
 
 #include "hedl_internal.h"
+#include "launch.cuh"
 
 namespace hedl {
 namespace {
@@ -271,6 +272,7 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
     uint32_t *tslot = reinterpret_cast<uint32_t *>(tempty + 2);
     volatile uint32_t *okp = tslot + 1;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+    pdl_trigger();
     const uint32_t s0 = smem_u32(base);
     const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty), tfull0 = smem_u32(tfull),
                    tempty0 = smem_u32(tempty);
@@ -297,6 +299,7 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t taddr = *tslot;
+    pdl_wait();   // everything above overlaps the kernel before
 
     if (warp == 0 && lane == 0) {
         // producer: the running block count u uses stage u % STAGES
@@ -507,8 +510,7 @@ int launch(const UmmaArgs *a, int count, cudaStream_t s) {
     }
     b.items0 = (int)item_count(a[0], UN);
     b.items = b.items0 + (count > 1 ? (int)item_count(a[1], UN) : 0);
-    umma_kernel<UN, TWO><<<(unsigned)std::min(b.items, sm_count()), THREADS, Shape<UN>::SMEM, s>>>(b);
-    return (int)cudaGetLastError();
+    return (int)launch_pdl(umma_kernel<UN, TWO>, (unsigned)std::min(b.items, sm_count()), THREADS, Shape<UN>::SMEM, s, b);
 }
 
 }  // namespace
