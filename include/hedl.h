@@ -233,10 +233,10 @@ typedef struct hedl_plan hedl_plan;
 #define HEDL_PLAIN      4u   /* one launch per operation per hypothesis */
 #define HEDL_LEVELS     8u   /* one launch per dependency level, no device waits */
 #define HEDL_NO_SLICE  16u   /* evaluate every role restriction on its own CSR walk
-                                (default: up to 32 restrictions of one role and
-                                direction that become ready together share one walk,
-                                formed where at least two restrictions have the same
-                                role, direction and nesting depth of role restrictions) */
+                                (default: up to 64 restrictions of one role and
+                                direction share one walk, at a stage between where
+                                each is ready and where it is needed, formed where at
+                                least two can walk together) */
 #define HEDL_SLICE_ALL 32u   /* put every eligible role restriction in a shared walk,
                                 even a group of one (ignored with HEDL_NO_SLICE) */
 #define HEDL_TEST_UNSAT_DEP 0x100u  /* TEST HOOK: add a dependency nothing

@@ -17,9 +17,10 @@
 //   3. every materialized node and every hypothesis root becomes a segment:
 //      a role-free boolean program whose leaves are atoms, data ranges,
 //      slots and role restrictions over slots or concept rows;
-//   4. role restrictions that share a role, direction and nesting depth with
-//      another one become bit-sliced role groups (up to 32 per group, evaluated
-//      by one transposed-filler walk) instead of living inside a segment;
+//   4. role restrictions that share a role, direction and stage (walk_stages)
+//      with another one become bit-sliced role groups (up to 64 per group,
+//      evaluated by one transposed-filler walk) instead of living inside a
+//      segment;
 //   5. tasks get levels (1 + the deepest producer of a slot they read) and
 //      are grouped by (level, first role read); each group's work items are
 //      (task, tile) pairs in tile-major order so that tasks sweeping the same
@@ -28,7 +29,6 @@
 //      level that walks a role holds too few tasks to fill the GPU.
 #include <algorithm>
 #include <cstring>
-#include <unordered_map>
 
 #include "hedl_internal.h"
 
@@ -45,17 +45,41 @@ struct PNode {
     int32_t k0, k1;
 };
 
-struct Key {
-    uint64_t x, y;
-    bool operator==(const Key &o) const { return x == o.x && y == o.y; }
-};
-struct KeyHash {
-    size_t operator()(const Key &k) const {
-        uint64_t h = k.x * 0x9E3779B97F4A7C15ull ^ (k.y + 0x632BE59BD9B4E019ull + (k.x << 6) + (k.x >> 2));
+// Hash-consing table: open addressing over node indices (no allocation a
+// node; a batch of 4,096 hypotheses makes 50,000), keyed by the node's fields.
+class NodeTable {
+  public:
+    explicit NodeTable(size_t n) {
+        size_t cap = 64;
+        while (cap < 2 * n) cap <<= 1;
+        slots_.assign(cap, -1);
+        mask_ = cap - 1;
+    }
+    // the index of a node equal to n, or -1 with *slot set to where insert puts it
+    int32_t find(const PNode &n, const std::vector<PNode> &nodes, size_t *slot) const {
+        for (size_t at = hash(n) & mask_;; at = (at + 1) & mask_) {
+            const int32_t i = slots_[at];
+            if (i < 0) {
+                *slot = at;
+                return -1;
+            }
+            const PNode &o = nodes[i];
+            if (o.op == n.op && o.inv == n.inv && o.a == n.a && o.b == n.b && o.k0 == n.k0 && o.k1 == n.k1) return i;
+        }
+    }
+    void insert(size_t slot, int32_t i) { slots_[slot] = i; }
+
+  private:
+    static size_t hash(const PNode &n) {
+        const uint64_t x = (uint64_t)n.op | ((uint64_t)n.inv << 8) | ((uint64_t)n.a << 16) | ((uint64_t)n.b << 32);
+        const uint64_t y = (uint64_t)(uint32_t)n.k0 | ((uint64_t)(uint32_t)n.k1 << 32);
+        uint64_t h = x * 0x9E3779B97F4A7C15ull ^ (y + 0x632BE59BD9B4E019ull + (x << 6) + (x >> 2));
         h ^= h >> 31;
         h *= 0xBF58476D1CE4E5B9ull;
         return (size_t)(h ^ (h >> 29));
     }
+    std::vector<int32_t> slots_;
+    size_t mask_ = 0;
 };
 
 inline bool is_role(uint32_t op) { return op >= HEDL_OP_EXISTS && op <= HEDL_OP_EXACTLY; }
@@ -73,12 +97,21 @@ inline uint64_t str_bytes(const hedl_kb *kb, uint32_t op, uint32_t a, uint64_t N
     return 4 * (N + 1) + 4ull * kb->str_host[a].n_vals + (op == HEDL_OP_SCONTAINS ? 4 * kb->contain_words : 0);
 }
 
-inline int arity(uint32_t op) {
-    if (op == HEDL_OP_ATOM || op == HEDL_OP_TOP || op == HEDL_OP_BOT || is_data(op) || is_str(op)) return 0;
-    if (op == HEDL_OP_NOT || is_role(op)) return 1;
-    if (op == HEDL_OP_AND || op == HEDL_OP_OR) return 2;
-    return -1;
-}
+// operands of an op, -1 for an unknown one
+struct Arity {
+    int8_t of[256];
+    constexpr Arity() : of() {
+        for (int op = 0; op < 256; ++op) of[op] = -1;
+        for (int op : {HEDL_OP_ATOM, HEDL_OP_TOP, HEDL_OP_BOT, HEDL_OP_DGE, HEDL_OP_DLE, HEDL_OP_DEQ, HEDL_OP_SEQ,
+                       HEDL_OP_SCONTAINS})
+            of[op] = 0;
+        for (int op : {HEDL_OP_NOT, HEDL_OP_EXISTS, HEDL_OP_FORALL, HEDL_OP_ATLEAST, HEDL_OP_ATMOST, HEDL_OP_EXACTLY})
+            of[op] = 1;
+        of[HEDL_OP_AND] = of[HEDL_OP_OR] = 2;
+    }
+};
+constexpr Arity ARITY;
+inline int arity(uint32_t op) { return ARITY.of[op & 0xFF]; }
 
 const char *op_name(uint32_t op) {
     static const char *names[] = {"?", "ATOM", "TOP", "BOT", "NOT", "AND", "OR", "EXISTS", "FORALL",
@@ -159,6 +192,79 @@ uint64_t put(std::vector<uint8_t> &img, const std::vector<T> &v) {
     return off;
 }
 
+// The stage (1, 2, ...) at which each bit-sliceable role restriction walks;
+// 0 for every other node.  A restriction may walk once those nested in its
+// filler have (a stage later than all of them), and has to by the stage that
+// leaves one stage for each restriction around it, in a plan of as many stages
+// as the deepest nesting.  At each stage a role and direction walks if one of
+// its ready restrictions cannot wait; then all its ready ones walk with it.
+// Otherwise only whole groups of SLICES * MAX_PARTS walk (waiting could not
+// save their walk), the ones with the least time left first.  A role and
+// direction of one or two restrictions does not wait: two lone walks over
+// bitset fillers cost about as much as a shared one with its transpose.
+// Walking every restriction as soon as it is ready (one group per role,
+// direction and nesting depth) took 261 walks for 2,048 refinements over 64
+// roles and directions and 244 for a batch of 4,096 over 32; this takes 134
+// and 186 (2,048 refinements at 4 * 10^6 individuals 57.3 -> 35.4 ms).
+// key_of numbers the (stage, role, direction) triples 0, 1, ... by stage; key_size counts their restrictions.
+void walk_stages(const std::vector<PNode> &nodes, uint32_t n_roles, std::vector<uint32_t> &stage,
+                 std::vector<uint32_t> &key_of, std::vector<uint32_t> &key_size) {
+    const uint32_t NN = (uint32_t)nodes.size(), NEVER = 0xFFFFFFFFu;
+    auto eligible = [&](const PNode &n) {
+        return is_role(n.op) && (n.op == HEDL_OP_EXISTS || n.op == HEDL_OP_FORALL || n.b <= SLICE_MAX_N);
+    };
+    std::vector<uint32_t> done(NN, 0);      // the stage that completes the restrictions in a node's expression
+    std::vector<uint32_t> inner;            // nodes with a restriction in their expression, children first
+    uint32_t last = 0;
+    for (uint32_t i = 0; i < NN; ++i) {
+        const PNode &n = nodes[i];
+        const uint32_t d = std::max(n.k0 >= 0 ? done[n.k0] : 0u, n.k1 >= 0 ? done[n.k1] : 0u);
+        done[i] = d + (is_role(n.op) ? 1u : 0u);
+        if (done[i]) inner.push_back(i);
+        last = std::max(last, done[i]);
+    }
+    std::vector<uint32_t> limit(NN, last);
+    for (auto it = inner.rbegin(); it != inner.rend(); ++it) {
+        const PNode &n = nodes[*it];
+        const uint32_t l = limit[*it] - (is_role(n.op) ? 1u : 0u);
+        if (n.k0 >= 0) limit[n.k0] = std::min(limit[n.k0], l);
+        if (n.k1 >= 0) limit[n.k1] = std::min(limit[n.k1], l);
+    }
+    std::vector<std::vector<uint32_t>> ready(2 * (size_t)n_roles);
+    std::vector<uint32_t> total(2 * (size_t)n_roles, 0);
+    for (uint32_t i : inner)
+        if (eligible(nodes[i])) total[2 * nodes[i].a + nodes[i].inv]++;
+    std::vector<uint32_t> open(inner);   // nodes that a restriction still keeps waiting, children first
+    for (uint32_t s = 1; s <= last; ++s) {
+        size_t kept = 0;
+        for (uint32_t i : open) {
+            const PNode &n = nodes[i];
+            uint32_t d = std::max(n.k0 >= 0 ? done[n.k0] : 0u, n.k1 >= 0 ? done[n.k1] : 0u);
+            if (stage[i]) d = stage[i];
+            else if (eligible(n)) {
+                if (d < s) ready[2 * n.a + n.inv].push_back(i);   // d is NEVER while something nested waits
+                d = NEVER;
+            } else if (is_role(n.op) && d != NEVER) ++d;
+            done[i] = d;
+            if (d == NEVER) open[kept++] = i;
+        }
+        open.resize(kept);
+        for (size_t key = 0; key < ready.size(); ++key) {
+            std::vector<uint32_t> &r = ready[key];
+            bool urgent = total[key] < 3;
+            for (uint32_t i : r) urgent = urgent || limit[i] <= s;
+            if (!urgent) {
+                std::stable_sort(r.begin(), r.end(), [&](uint32_t x, uint32_t y) { return limit[x] < limit[y]; });
+                r.resize(r.size() / (SLICES * MAX_PARTS) * (SLICES * MAX_PARTS));
+            }
+            if (r.empty()) continue;
+            for (uint32_t i : r) stage[i] = s, key_of[i] = (uint32_t)key_size.size();
+            key_size.push_back((uint32_t)r.size());
+            r.clear();
+        }
+    }
+}
+
 }  // namespace
 
 int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, uint32_t H, unsigned flags,
@@ -216,8 +322,7 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     const bool cse = !(flags & HEDL_NO_CSE);
     std::vector<PNode> nodes;
     nodes.reserve(offs[H] + 16);
-    std::unordered_map<Key, int32_t, KeyHash> memo;
-    memo.reserve(cse ? offs[H] * 2 + 16 : 0);
+    NodeTable memo(cse ? offs[H] : 0);   // at most one node an instruction
     auto make = [&](PNode n) -> int32_t {
         // canonical form: ignored fields zeroed, commutative operands ordered
         if (!is_role(n.op)) n.inv = 0;
@@ -228,20 +333,19 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
         if (cse) {
             if ((n.op == HEDL_OP_AND || n.op == HEDL_OP_OR) && n.k0 > n.k1) std::swap(n.k0, n.k1);
             if (n.op == HEDL_OP_NOT && nodes[n.k0].op == HEDL_OP_NOT) return nodes[n.k0].k0;
-            Key k{(uint64_t)n.op | ((uint64_t)n.inv << 8) | ((uint64_t)n.a << 16) | ((uint64_t)n.b << 32),
-                  (uint64_t)(uint32_t)n.k0 | ((uint64_t)(uint32_t)n.k1 << 32)};
-            auto it = memo.find(k);
-            if (it != memo.end()) return it->second;
-            memo.emplace(k, (int32_t)nodes.size());
+            size_t slot;
+            const int32_t same = memo.find(n, nodes, &slot);
+            if (same >= 0) return same;
+            memo.insert(slot, (int32_t)nodes.size());
         }
         nodes.push_back(n);
         return (int32_t)nodes.size() - 1;
     };
 
     std::vector<int32_t> roots(H);
-    std::vector<int32_t> st;
+    int32_t st[HEDL_MAX_STACK];   // validated: no program holds more
     for (uint32_t h = 0; h < H; ++h) {
-        st.clear();
+        int sp = 0;
         for (uint32_t k = offs[h]; k < offs[h + 1]; ++k) {
             uint64_t w = progs[k];
             PNode n{};
@@ -250,19 +354,13 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
             n.a = (uint32_t)((w >> 16) & 0xFFFF);
             n.b = (uint32_t)(w >> 32);
             n.k0 = n.k1 = -1;
-            int ar = arity(n.op);
-            if (ar == 2) {
-                n.k1 = st.back();
-                st.pop_back();
-                n.k0 = st.back();
-                st.pop_back();
-            } else if (ar == 1) {
-                n.k0 = st.back();
-                st.pop_back();
-            }
-            st.push_back(make(n));
+            const int ar = arity(n.op);
+            sp -= ar;
+            if (ar > 0) n.k0 = st[sp];
+            if (ar > 1) n.k1 = st[sp + 1];
+            st[sp++] = make(n);
         }
-        roots[h] = st.back();
+        roots[h] = st[0];
     }
     const uint32_t NN = (uint32_t)nodes.size();
     p->info.n_nodes = NN;
@@ -282,34 +380,19 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
         if (is_role(nodes[i].op) && nodes[nodes[i].k0].op != HEDL_OP_ATOM) mat[nodes[i].k0] = 1;
     // Bit-sliced role restrictions: each is materialized and evaluated by its
     // role group's shared walk (counting ones need n <= SLICE_MAX_N).  A walk
-    // shared by one restriction only costs a transpose and a 32-times larger
-    // filler, so by default a restriction is sliced only when another one has
-    // the same role, direction and depth (role restrictions nested below it,
-    // itself included), the depth standing in for the level it becomes ready at.
+    // costs its edges' gathers, whatever the number of slices up to
+    // SLICES * MAX_PARTS, so restrictions of one role and direction wait for
+    // each other: walk_stages gives every eligible restriction the stage it
+    // walks at.  A walk of one restriction only costs a transpose and a
+    // 32-times larger filler, so by default a restriction is sliced only when
+    // another one has the same role, direction and stage.
     const bool sliced = !(flags & HEDL_NO_SLICE);
     std::vector<uint8_t> sl(NN, 0);
-    std::vector<uint32_t> rdepth(NN, 0);
+    std::vector<uint32_t> stage(NN, 0), key_of(NN, 0), key_size;
     if (sliced) {
-        auto eligible = [&](const PNode &n) {
-            return is_role(n.op) && (n.op == HEDL_OP_EXISTS || n.op == HEDL_OP_FORALL || n.b <= SLICE_MAX_N);
-        };
-        std::unordered_map<uint64_t, uint32_t> same;
-        for (uint32_t i = 0; i < NN; ++i) {
-            const PNode &n = nodes[i];
-            uint32_t d = 0;
-            if (n.k0 >= 0) d = std::max(d, rdepth[n.k0]);
-            if (n.k1 >= 0) d = std::max(d, rdepth[n.k1]);
-            rdepth[i] = d + (is_role(n.op) ? 1u : 0u);
-            if (eligible(n)) same[((uint64_t)rdepth[i] << 32) | (n.a * 2u + n.inv)]++;
-        }
-        for (uint32_t i = 0; i < NN; ++i) {
-            const PNode &n = nodes[i];
-            if (eligible(n) &&
-                ((flags & HEDL_SLICE_ALL) || same[((uint64_t)rdepth[i] << 32) | (n.a * 2u + n.inv)] >= 2)) {
-                sl[i] = 1;
-                mat[i] = 1;
-            }
-        }
+        walk_stages(nodes, kb->n_roles, stage, key_of, key_size);
+        for (uint32_t i = 0; i < NN; ++i)
+            if (stage[i] && ((flags & HEDL_SLICE_ALL) || key_size[key_of[i]] >= 2)) sl[i] = mat[i] = 1;
     }
     std::vector<uint8_t> role_inline(NN, 0);
     std::vector<uint32_t> need(NN, 1);
@@ -377,7 +460,7 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     }
     std::vector<Seg> segs;
     std::vector<DInsn> code;
-    std::vector<std::vector<uint32_t>> seg_slots_read;
+    std::vector<uint32_t> read_list, read_off{0};   // the slots segment s reads: read_list[read_off[s] .. read_off[s + 1])
     std::vector<uint32_t> seg_of_slot(n_slots, 0);
     std::vector<uint32_t> role_key;  // first role read, for grouping
     // Algorithmic bytes, the per-operation model (no credit for sharing a CSR
@@ -387,18 +470,27 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     // 2B + 16, over the operations left after common sub-concepts are shared.
     uint64_t model = 0;
 
-    std::vector<int32_t> work;
+    struct Frame { int32_t n; int state; };
+    std::vector<Frame> fr;
+    std::vector<uint32_t> reads;
+    auto keep_reads = [&](std::vector<uint32_t> &v) {   // sorted, each once
+        if (v.size() > 1) {
+            std::sort(v.begin(), v.end());
+            v.erase(std::unique(v.begin(), v.end()), v.end());
+        }
+        read_list.insert(read_list.end(), v.begin(), v.end());
+        read_off.push_back((uint32_t)read_list.size());
+    };
     auto emit_segment = [&](int32_t root, uint32_t out_slot, uint32_t hyp) {
         Seg s{};
         s.code_off = (uint32_t)code.size();
         s.out_slot = out_slot;
         s.hyp = hyp;
         s.filler = NO_FILLER;
-        std::vector<uint32_t> reads;
+        reads.clear();
         uint32_t rk = 0xFFFFFFFFu;
         // iterative post-order emission, larger stack need first
-        struct Frame { int32_t n; int state; };
-        std::vector<Frame> fr;
+        fr.clear();
         fr.push_back({root, 0});
         int depth = 0, maxdepth = 0;
         while (!fr.empty()) {
@@ -489,9 +581,7 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
         s.code_len = (uint32_t)code.size() - s.code_off;
         p->max_stack = std::max(p->max_stack, (uint32_t)maxdepth);
         if (hyp != NO_HYP) model += 2 * B + 16;
-        std::sort(reads.begin(), reads.end());
-        reads.erase(std::unique(reads.begin(), reads.end()), reads.end());
-        seg_slots_read.push_back(reads);
+        keep_reads(reads);
         role_key.push_back(rk);
         segs.push_back(s);
     };
@@ -513,7 +603,8 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
             d.ref = slot_of[roots[h]];
             code.push_back(d);
             model += 2 * B + 16;
-            seg_slots_read.push_back({slot_of[roots[h]]});
+            reads.assign(1, slot_of[roots[h]]);
+            keep_reads(reads);
             role_key.push_back(0xFFFFFFFFu);
             segs.push_back(s);
             p->max_stack = std::max(p->max_stack, 1u);
@@ -528,73 +619,67 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     const uint32_t NSEG = (uint32_t)segs.size();
     const uint64_t FT_PART = 4ull * 32ull * kb->wp;   // one FT word per individual (>= 4 N bytes)
 
-    // Sliced restrictions are grouped by (role depth, role, direction): one
-    // group key per distinct triple, in a dense numbering.
-    std::vector<uint32_t> key_of(NN, 0xFFFFFFFFu);
-    std::vector<uint64_t> key_val;
-    uint32_t max_rd = 0;
-    {
-        std::unordered_map<uint64_t, uint32_t> ids;
-        for (uint32_t i = 0; i < NN; ++i) {
-            if (!sl[i]) continue;
-            const uint64_t k = ((uint64_t)rdepth[i] << 32) | (nodes[i].a * 2u + nodes[i].inv);
-            auto it = ids.find(k);
-            if (it == ids.end()) {
-                it = ids.emplace(k, (uint32_t)key_val.size()).first;
-                key_val.push_back(k);
-            }
-            key_of[i] = it->second;
-            max_rd = std::max(max_rd, rdepth[i]);
-        }
-    }
+    uint32_t max_stage = 0;   // of the sliced restrictions, grouped by key (stage, role, direction)
+    for (uint32_t i = 0; i < NN; ++i)
+        if (sl[i]) max_stage = std::max(max_stage, stage[i]);
 
-    // Production level of every slot and level of every segment, in node order
-    // (children first).  A segment reading nothing is at level 0 and one level
-    // above the slots it reads.  A sliced role restriction is ready one level
-    // above its filler's transpose, which runs one level above the filler's
-    // producer (level 0 for a concept row); all restrictions of a group key
-    // walk together, at the level of the group's last-ready one.  A filler
-    // holds only restrictions of smaller role depth, so the levels of depth d
-    // are final once those of depths below d are: one pass per depth fixes
-    // them in turn, and a last pass sets every level.
+    // Production level of every slot and level of every segment.  A segment
+    // reading nothing is at level 0 and otherwise one level above the slots it
+    // reads.  A sliced role restriction is ready one level above its filler's
+    // transpose, which runs one level above the filler's producer (level 0 for
+    // a concept row); all restrictions of a group key walk together, at the
+    // level of the group's last-ready one.  A filler holds only sliced
+    // restrictions of earlier stages, so materialized nodes are taken by the
+    // last stage in their expression, children first: the sliced restrictions
+    // of a stage (their fillers belong to earlier ones), then its segments.
     std::vector<uint32_t> slot_level(n_slots, 0), seg_level(NSEG, 0);
-    std::vector<uint32_t> group_level(key_val.size(), 0);
+    std::vector<uint32_t> group_level(key_size.size(), 0);
     auto seg_lvl = [&](uint32_t sidx) {
         uint32_t lvl = 0;
-        for (uint32_t sl2 : seg_slots_read[sidx]) lvl = std::max(lvl, slot_level[sl2] + 1);
+        for (uint32_t q = read_off[sidx]; q < read_off[sidx + 1]; ++q) lvl = std::max(lvl, slot_level[read_list[q]] + 1);
         return lvl;
     };
-    for (uint32_t d = 1; d <= max_rd + 1; ++d) {
-        std::vector<uint32_t> ready(key_val.size(), 0);
+    {
+        std::vector<uint32_t> last_stage(NN, 0), first(max_stage + 2, 0), by_stage;
         for (uint32_t i = 0; i < NN; ++i) {
-            if (!mat[i]) continue;
-            if (sl[i]) {
+            const PNode &n = nodes[i];
+            uint32_t d = std::max(n.k0 >= 0 ? last_stage[n.k0] : 0u, n.k1 >= 0 ? last_stage[n.k1] : 0u);
+            if (sl[i]) d = stage[i];
+            last_stage[i] = d;
+            if (mat[i]) first[d + 1]++;
+        }
+        for (uint32_t d = 1; d < first.size(); ++d) first[d] += first[d - 1];
+        by_stage.resize(first.back());
+        std::vector<uint32_t> at(first.begin(), first.end() - 1);
+        for (uint32_t i = 0; i < NN; ++i)
+            if (mat[i]) by_stage[at[last_stage[i]]++] = i;
+        for (uint32_t d = 0; d <= max_stage; ++d) {
+            for (uint32_t q = first[d]; q < first[d + 1]; ++q) {
+                const uint32_t i = by_stage[q];
+                if (!sl[i]) continue;
                 const int32_t f = nodes[i].k0;
                 const bool concept_filler = nodes[f].op == HEDL_OP_ATOM && !mat[f];
-                const uint32_t own = concept_filler ? 1u : slot_level[slot_of[f]] + 2u;
-                uint32_t lvl = own;
-                if (rdepth[i] < d) lvl = group_level[key_of[i]];
-                else if (rdepth[i] == d) ready[key_of[i]] = std::max(ready[key_of[i]], own);
-                slot_level[slot_of[i]] = lvl;
-            } else {
+                uint32_t &lvl = group_level[key_of[i]];
+                lvl = std::max(lvl, concept_filler ? 1u : slot_level[slot_of[f]] + 2u);
+            }
+            for (uint32_t q = first[d]; q < first[d + 1]; ++q)
+                if (sl[by_stage[q]]) slot_level[slot_of[by_stage[q]]] = group_level[key_of[by_stage[q]]];
+            for (uint32_t q = first[d]; q < first[d + 1]; ++q) {
+                const uint32_t i = by_stage[q];
+                if (sl[i]) continue;
                 const uint32_t sidx = seg_of_slot[slot_of[i]];
-                seg_level[sidx] = seg_lvl(sidx);
-                slot_level[slot_of[i]] = seg_level[sidx];
+                slot_level[slot_of[i]] = seg_level[sidx] = seg_lvl(sidx);
             }
         }
-        for (size_t k = 0; k < key_val.size(); ++k)
-            if ((key_val[k] >> 32) == d) group_level[k] = ready[k];
-        if (!sliced) break;
     }
     for (uint32_t sidx = 0; sidx < NSEG; ++sidx)
         if (segs[sidx].hyp != NO_HYP) seg_level[sidx] = seg_lvl(sidx);
 
-    // role groups: sliced restrictions keyed by (role depth, role, direction), up to
+    // role groups: sliced restrictions keyed by (stage, role, direction), up to
     // SLICES * MAX_PARTS at a time (one FT word per 32 of them)
     std::vector<RGroup> rgroups;
     std::vector<uint32_t> task_level(seg_level);
     std::vector<uint32_t> task_key(role_key);
-    std::vector<std::vector<uint32_t>> task_reads(seg_slots_read);
     uint64_t ft_bytes = 0;
     {
         std::vector<std::pair<uint64_t, uint32_t>> keyed;   // ((level << 32) | role2, node)
@@ -611,7 +696,7 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
             g.role2 = (uint32_t)(keyed[k].first & 0xFFFFFFFFu);
             g.n = (uint32_t)(k2 - k);
             g.parts = g.n > SLICES ? MAX_PARTS : 1u;
-            std::vector<uint32_t> reads;
+            reads.clear();
             for (size_t q = k; q < k2; ++q) {
                 const uint32_t i = keyed[q].second;
                 const PNode &n = nodes[i];
@@ -626,21 +711,18 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
                 }
                 if (n.op == HEDL_OP_FORALL) g.filler[s_] |= REF_NEG;
                 g.out[s_] = slot_of[i];
-                for (uint32_t v = 0; v < 8; ++v) {
-                    bool holds;
-                    switch (n.op) {
-                    case HEDL_OP_EXISTS: holds = v >= 1; break;
-                    case HEDL_OP_FORALL: holds = v == 0; break;   // successors outside C
-                    case HEDL_OP_ATLEAST: holds = v >= n.b; break;
-                    case HEDL_OP_ATMOST: holds = v <= n.b; break;
-                    default: holds = v == n.b; break;
-                    }
-                    if (holds) g.want[s_ / SLICES][v] |= 1u << (s_ % SLICES);
-                }
+                // the counts 0 .. 7 (7: or more) at which the restriction holds
+                const uint32_t le = n.b >= 7 ? 0xFFu : (2u << n.b) - 1u, lt = n.b == 0 ? 0u : le >> 1;
+                uint32_t holds = n.op == HEDL_OP_EXISTS    ? 0xFEu
+                                 : n.op == HEDL_OP_FORALL  ? 0x01u   // successors outside C
+                                 : n.op == HEDL_OP_ATLEAST ? 0xFFu & ~lt
+                                 : n.op == HEDL_OP_ATMOST  ? le
+                                                           : le & ~lt;
+                for (; holds; holds &= holds - 1) g.want[s_ / SLICES][__builtin_ctz(holds)] |= 1u << (s_ % SLICES);
                 p->info.n_role_ops++;
             }
-            std::sort(reads.begin(), reads.end());
-            reads.erase(std::unique(reads.begin(), reads.end()), reads.end());
+            keep_reads(reads);                              // of the transpose
+            read_off.push_back((uint32_t)read_list.size());   // the walk reads no slot
             const uint32_t gi = (uint32_t)rgroups.size();
             const uint32_t wl = (uint32_t)(keyed[k].first >> 32);
             // transpose task, then walk task
@@ -653,14 +735,12 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
             segs.push_back(t);
             task_level.push_back(wl - 1);
             task_key.push_back(g.role2 | 0x80000000u);
-            task_reads.push_back(reads);
             Seg w = t;
             w.kind = TASK_WALK;
             const uint32_t walk_task = (uint32_t)segs.size();
             segs.push_back(w);
             task_level.push_back(wl);
             task_key.push_back(g.role2);
-            task_reads.push_back({});
             for (uint32_t s_ = 0; s_ < g.n; ++s_) seg_of_slot[g.out[s_]] = walk_task;
             const DevCSR &csr = kb->csr_host[g.role2];
             model += (uint64_t)g.n * (4 * (N + 1) + 4ull * csr.n_edges + 2 * B);
@@ -680,7 +760,7 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
         if (segs[s_].kind == TASK_WALK) {
             deps.push_back(s_ - 1);
         } else {
-            for (uint32_t sl2 : task_reads[s_]) deps.push_back(seg_of_slot[sl2]);
+            for (uint32_t q = read_off[s_]; q < read_off[s_ + 1]; ++q) deps.push_back(seg_of_slot[read_list[q]]);
         }
         segs[s_].dep_cnt = (uint32_t)deps.size() - segs[s_].dep_off;
         n_levels = std::max(n_levels, task_level[s_] + 1);
@@ -757,6 +837,9 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
 
     // image: header, tables, counters; then the slots
     std::vector<uint8_t> &img = p->image;
+    img.reserve(sizeof(PlanHeader) + segs.size() * sizeof(Seg) + groups.size() * sizeof(Group) + 4 * gsegs.size() +
+                4 * deps.size() + code.size() * sizeof(DInsn) + 4 * level_items.size() + 4 * (NS + 5 + 2ull * H) +
+                rgroups.size() * sizeof(RGroup) + 10 * 256);
     img.resize(sizeof(PlanHeader));
     PlanHeader hd{};
     hd.n_items = (uint32_t)items;
