@@ -391,6 +391,11 @@ __device__ __forceinline__ void role_stream(const DevCSR g, const uint32_t *fill
     }
 }
 
+template <int WPL>
+struct RowWords {
+    uint32_t v[WPL];
+};
+
 __device__ __forceinline__ bool data_cmp(uint32_t cmp, float x, float t);
 
 // Numeric data-range restriction (Algorithms 9-10): one float compare per
@@ -437,218 +442,263 @@ __device__ __forceinline__ bool data_cmp(uint32_t cmp, float x, float t) {
 // 32-bit word of a float value or of a string id): a float compare (numeric
 // roles, Algorithms 9-10), id equality (string EQUAL, Algorithms 11-12) or a
 // bit of the pattern's containment row (string CONTAIN, Algorithms 13-14).
-// ValueTest carries the kind at run time; exist_words is compiled once per
-// kind (each float compare, IdEqTest, IdBitTest) and dispatched once per
-// restriction.
 struct ValueTest {
-    enum : uint32_t { FLOAT_CMP = 0, ID_EQ = 1, ID_BIT = 2 };
-    uint32_t mode;
-    uint32_t cmp;           // FLOAT_CMP: HEDL_OP_DGE / DLE / DEQ
-    uint32_t arg;           // FLOAT_CMP: the threshold's bits; ID_EQ: the string id
+    enum : uint32_t { GE = 0, LE = 1, EQ = 2, ID_EQ = 3, ID_BIT = 4 };
+    uint32_t kind;
+    uint32_t arg;           // the threshold's bits or the string id
     const uint32_t *bits;   // ID_BIT: the containment row
-};
-template <uint32_t CMP>
-struct FloatTest {
-    float t;
-    __device__ __forceinline__ bool operator()(uint32_t x) const {
-        const float f = __uint_as_float(x);
-        return CMP == HEDL_OP_DGE ? (f >= t) : CMP == HEDL_OP_DLE ? (f <= t) : (f == t);
-    }
-};
-struct IdEqTest {
-    uint32_t id;
-    __device__ __forceinline__ bool operator()(uint32_t x) const { return x == id; }
-};
-struct IdBitTest {
-    const uint32_t *bits;
-    __device__ __forceinline__ bool operator()(uint32_t x) const { return (__ldg(bits + (x >> 5)) >> (x & 31u)) & 1u; }
 };
 
 // Existential restriction on a concrete role with several values per
 // subject (Section III-B): individual i belongs iff one of its values
 // vals[rp[i] .. rp[i+1]) passes the test.  The warp's 32*WPL words are
 // 1024*WPL consecutive individuals, so their values form one contiguous run,
-// and the warp streams that run once, in windows of EX_WIN values.  Each lane
-// loads four 16-byte vectors of a window (each load coalesced over 512
-// bytes), and the warp turns the tests into the window's 512-bit pass mask:
-// lane k < 16 keeps mask word k and the position of the first pass in the
-// words after it.  The row pointers come four words at a time (lane l loads
-// rp[32w + l] of each, the next four in flight), and each lane finds the
-// first pass at or after its row's start with two shuffles and compares it
-// with the row's end.  The next window's values are in flight while the
-// current one is looked up, and the warp's row pointers are requested into L2
-// when it starts (a bulk prefetch hint, which holds no registers).  Hinting
-// the values too was slower where several restrictions read one role's
-// values at once.  A window is loaded only while a row that has
-// not passed yet reaches into it, and the stream jumps straight to the first
-// such row, so a subject already satisfied is skipped (the paper's early
-// exit): a heavy subject costs its values up to the window of its first
-// pass.  Value counts stay below 2^31 (the KB loader's limit), so positions
-// relative to a window fit signed 32-bit arithmetic.
-constexpr uint32_t EX_LOADS = 4;               // 16-byte loads per lane per window
-constexpr uint32_t EX_WIN = 128u * EX_LOADS;   // values per window
-constexpr uint32_t EX_NONE = 0x7FFFFFFFu;      // no pass
+// which the warp streams once, in windows of EX_WIN values that asynchronous
+// 16-byte copies bring into a ring of EX_STAGES windows in shared memory (32
+// warps an SM keep 64 KB in flight and hold no registers for it).  Lane l tests
+// value 32u + l of a window, and a ballot packs 32 tests into a mask word in
+// the order of the values, which lane 0 puts into a ring of masks.  The row
+// pointers come the same way, a batch of four words (128 individuals) ahead.  A
+// batch needs the masks of its run; each lane then looks its rows up with two
+// reads and a funnel shift each (rows over 32 values go on word by word).
+//
+// A batch whose run does not fit the mask ring (a heavy subject) is walked word
+// by word in pieces of EX_STAGES windows, each only as long as a row that has
+// not passed yet reaches into it, jumping to the first such row (the paper's
+// early exit): a heavy subject costs its values up to the piece of its first
+// pass.
+//
+// Bound: HBM (4(N+1) + 4M bytes a restriction), as long as the instructions
+// stay few and fit the instruction cache: about 60 a word of 32 individuals
+// with four values each.  Packing 16-byte loads into masks by shuffles took
+// 138, and with a function a kind of test and the row batches in two register
+// sets warps waited 47 % of their time for instructions.  24 restrictions on 8
+// roles at 10^7 individuals (3.8 GB by the model, each role read three times):
+// 1.96 ms -> 1.26 ms.
+static_assert(EX_RING % EX_LOADS == 0 && EX_LOADS % 4 == 0, "a window's masks are whole 16-byte stores");
 
-// The row pointers of words w0 .. w0+3: r[q] = rp[32(w0 + q) + lane],
-// tail = rp[32 w0 + 128], zero past n (a zero end makes a row empty).
-struct ExRows {
-    uint32_t r[4];
-    uint32_t tail;
-};
-__device__ __forceinline__ void ex_rows(ExRows &b, const uint32_t *rp, uint32_t w0, uint32_t w_end, uint32_t n,
+// Asynchronous copy of src[at .. at + COUNT) to dst, the elements below end
+// only: 16 bytes a lane where they are aligned and all wanted, else 4.
+template <uint32_t COUNT>
+__device__ __forceinline__ void ex_copy(uint32_t *dst, const uint32_t *src, uint32_t at, uint32_t end, bool vec,
                                         uint32_t lane) {
-    if (w0 >= w_end) return;   // warp-uniform; nothing reads this batch
+    const uint32_t to = (uint32_t)__cvta_generic_to_shared(dst);
+    if (vec && at + COUNT <= end) {   // warp-uniform
 #pragma unroll
-    for (uint32_t q = 0; q < 4u; ++q) {
-        const uint32_t i = 32u * (w0 + q) + lane;
-        b.r[q] = i <= n ? ld_stream(rp + i) : 0u;
-    }
-    const uint32_t t = 32u * w0 + 128u;
-    b.tail = t <= n ? ld_stream(rp + t) : 0u;
-}
-
-// the window [c, c + EX_WIN) of a run ending at end (c a multiple of 128):
-// lane l's vector u holds values c + 128u + 4l .. + 3 (zero at and past end)
-__device__ __forceinline__ void ex_fetch(const uint32_t *vals, uint32_t c, uint32_t end, bool vec, uint32_t lane,
-                                         uint4 (&x)[EX_LOADS]) {
-#pragma unroll
-    for (uint32_t u = 0; u < EX_LOADS; ++u) {
-        const uint32_t k = c + 128u * u + 4u * lane;
-        if (vec && k + 4u <= end) {
-            x[u] = ld_stream4(vals + k);
-        } else {
-            x[u].x = k < end ? ld_stream(vals + k) : 0u;
-            x[u].y = k + 1u < end ? ld_stream(vals + k + 1u) : 0u;
-            x[u].z = k + 2u < end ? ld_stream(vals + k + 2u) : 0u;
-            x[u].w = k + 3u < end ? ld_stream(vals + k + 3u) : 0u;
-        }
-    }
-}
-
-// The window's pass mask: word k (values c + 32k .. c + 32k + 31) to lane k
-// < 16, zero to lanes 16..31, and in fn the position of the first pass in
-// words k+1 .. 15 (EX_NONE if none).  Lane l's four values of vector u are
-// bits 4(l mod 8) .. +3 of word 4u + l/8; an OR over each group of eight
-// lanes assembles the word, lane k fetches word k from its group, and a
-// suffix minimum over the lanes gives fn.
-template <class Test>
-__device__ __forceinline__ uint32_t ex_bits(const uint4 (&x)[EX_LOADS], uint32_t lane, const Test &test,
-                                            uint32_t &fn) {
-    uint32_t wu[EX_LOADS];
-#pragma unroll
-    for (uint32_t u = 0; u < EX_LOADS; ++u) {
-        uint32_t q = (uint32_t)test(x[u].x) | (uint32_t)test(x[u].y) << 1 | (uint32_t)test(x[u].z) << 2 |
-                     (uint32_t)test(x[u].w) << 3;
-        q <<= 4u * (lane & 7u);
-        q |= __shfl_xor_sync(FULL, q, 1);
-        q |= __shfl_xor_sync(FULL, q, 2);
-        q |= __shfl_xor_sync(FULL, q, 4);
-        wu[u] = q;
-    }
-    uint32_t bm = 0;
-#pragma unroll
-    for (uint32_t u = 0; u < EX_LOADS; ++u) {
-        const uint32_t t = __shfl_sync(FULL, wu[u], 8u * (lane & 3u));
-        if ((lane >> 2) == u) bm = t;
-    }
-    uint32_t f = bm ? 32u * lane + (uint32_t)__ffs(bm) - 1u : EX_NONE;
-#pragma unroll
-    for (uint32_t o = 1; o < 16u; o <<= 1) f = min(f, __shfl_down_sync(FULL, f, o));
-    fn = __shfl_down_sync(FULL, f, 1);   // lane 31 keeps its own EX_NONE
-    return bm;
-}
-
-template <int WPL, class Test>
-__device__ __forceinline__ void exist_words(const uint32_t *rp, const uint32_t *vals, const Test test, uint32_t n,
-                                            uint32_t n_words, uint32_t wb, uint32_t lane, uint32_t (&v)[WPL]) {
-#pragma unroll
-    for (int s = 0; s < WPL; ++s) v[s] = 0u;
-    const uint32_t w_end = min(wb + 32u * WPL, n_words);   // the warp's words [wb, w_end)
-    if (wb >= w_end) return;
-    const bool vec = (reinterpret_cast<uintptr_t>(vals) & 15u) == 0;
-    const uint32_t end = ld_stream(rp + min(32u * w_end, n));   // the end of the warp's run
-    uint32_t c = ld_stream(rp + 32u * wb) & ~127u;               // the window
-    // the warp's row pointers go to L2 ahead of their loads (a hint that
-    // holds no registers)
-    if ((reinterpret_cast<uintptr_t>(rp) & 15u) == 0) prefetch_range(rp, 32u * wb, min(32u * w_end, n) + 1u, lane);
-    uint4 x[EX_LOADS];
-    ex_fetch(vals, c, end, vec, lane, x);
-    uint32_t fn;
-    uint32_t bm = ex_bits(x, lane, test, fn);
-    ex_fetch(vals, c + EX_WIN, end, vec, lane, x);               // the next window, in flight
-    // row batches alternate between two registers, so a pending load is never copied
-    ExRows ra, rb;
-    ex_rows(ra, rp, wb, w_end, n, lane);
-    ex_rows(rb, rp, wb + 4u, w_end, n, lane);
-    auto batch = [&](uint32_t w0, const ExRows &rows) {
+        for (uint32_t u = 0; u < COUNT; u += 128u)
+            if (COUNT >= 128u || 4u * lane < COUNT)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 4u * u + 16u * lane),
+                             "l"(src + at + u + 4u * lane)
+                             : "memory");
+    } else {
 #pragma unroll 1
-        for (uint32_t j = 0; j < 4u && w0 + j < w_end; ++j) {   // warp-uniform
-            // this lane's row [lo, hi): lane 31's end is the next word's first row pointer
-            const uint32_t lo = j == 0u ? rows.r[0] : j == 1u ? rows.r[1] : j == 2u ? rows.r[2] : rows.r[3];
-            const uint32_t ln = j == 0u ? rows.r[1] : j == 1u ? rows.r[2] : j == 2u ? rows.r[3] : rows.tail;
-            const uint32_t dn = __shfl_down_sync(FULL, lo, 1), up = __shfl_sync(FULL, ln, 0);
-            const uint32_t hi = lane == 31u ? up : dn;
-            bool hit = false;
-            for (;;) {
-                const int rl = (int)(lo - c), rh = (int)(hi - c);   // the row relative to the window
-                const int a = max(rl, 0), b = min(rh, (int)EX_WIN);
-                const uint32_t wa = (uint32_t)a >> 5;
-                const uint32_t ma = __shfl_sync(FULL, bm, wa), fa = __shfl_sync(FULL, fn, wa);
-                const uint32_t m = ma & (FULL << (a & 31));
-                const int first = m ? (int)(32u * wa + (uint32_t)__ffs(m) - 1u) : (int)fa;   // first pass >= a
-                hit = hit || (a < b && first < b);
-                // the first value, past the window, of a row that has not passed yet
-                const bool more = !hit && rh > (int)EX_WIN && rl < rh;
-                const uint32_t nxt = __reduce_min_sync(FULL, more ? (uint32_t)max(rl, (int)EX_WIN) : 0xFFFFFFFFu);
-                if (nxt == 0xFFFFFFFFu) break;
-                const uint32_t cn = c + (nxt & ~127u);
-                if (cn != c + EX_WIN) ex_fetch(vals, cn, end, vec, lane, x);   // a jump: not the window in flight
-                c = cn;
-                bm = ex_bits(x, lane, test, fn);
-                ex_fetch(vals, c + EX_WIN, end, vec, lane, x);
+        for (uint32_t u = lane; u < COUNT; u += 32u)
+            if (at + u < end)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + 4u * u), "l"(src + at + u)
+                             : "memory");
+    }
+}
+
+// Waits until at most `after` of this thread's groups of asynchronous copies
+// are pending (warp-uniform), then for the warp.
+__device__ __forceinline__ void ex_wait(uint32_t after) {
+    if (after == 0u) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    else if (after == 1u) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else if (after == 2u) asm volatile("cp.async.wait_group 2;" ::: "memory");
+    else asm volatile("cp.async.wait_group 3;" ::: "memory");
+    __syncwarp();
+}
+
+// The masks of the window x (value c on; those at and past end fail) to ring[0 .. EX_LOADS).
+__device__ __forceinline__ void ex_masks(const uint32_t *x, uint32_t c, uint32_t end, uint32_t lane, const ValueTest &t,
+                                         uint32_t *ring) {
+    uint32_t v[EX_LOADS], m[EX_LOADS];
+#pragma unroll
+    for (uint32_t u = 0; u < EX_LOADS; ++u) v[u] = x[32u * u + lane];
+    const float f = __uint_as_float(t.arg);
+    switch (t.kind) {   // warp-uniform
+    case ValueTest::GE:
+#pragma unroll
+        for (uint32_t u = 0; u < EX_LOADS; ++u) m[u] = __ballot_sync(FULL, __uint_as_float(v[u]) >= f);
+        break;
+    case ValueTest::LE:
+#pragma unroll
+        for (uint32_t u = 0; u < EX_LOADS; ++u) m[u] = __ballot_sync(FULL, __uint_as_float(v[u]) <= f);
+        break;
+    case ValueTest::EQ:
+#pragma unroll
+        for (uint32_t u = 0; u < EX_LOADS; ++u) m[u] = __ballot_sync(FULL, __uint_as_float(v[u]) == f);
+        break;
+    case ValueTest::ID_EQ:
+#pragma unroll
+        for (uint32_t u = 0; u < EX_LOADS; ++u) m[u] = __ballot_sync(FULL, v[u] == t.arg);
+        break;
+    default: {
+        uint32_t w[EX_LOADS];
+#pragma unroll
+        for (uint32_t u = 0; u < EX_LOADS; ++u)   // past the end the ring holds no id
+            w[u] = c + 32u * u + lane < end ? __ldg(t.bits + (v[u] >> 5)) >> (v[u] & 31u) : 0u;
+#pragma unroll
+        for (uint32_t u = 0; u < EX_LOADS; ++u) m[u] = __ballot_sync(FULL, w[u] & 1u);
+        break;
+    }
+    }
+    if (c + EX_WIN > end) {   // the run's last window
+#pragma unroll
+        for (uint32_t u = 0; u < EX_LOADS; ++u) m[u] &= range_mask(0u, end > c + 32u * u ? min(end - c - 32u * u, 32u) : 0u);
+    }
+    if (lane == 0u) {
+#pragma unroll
+        for (uint32_t u = 0; u < EX_LOADS; u += 4u)
+            *reinterpret_cast<uint4 *>(ring + u) = make_uint4(m[u], m[u + 1], m[u + 2], m[u + 3]);
+    }
+}
+
+// how many values of [lo, hi) pass (hi > lo), by the ring's masks, of the first 32
+__device__ __forceinline__ uint32_t ex_count(const uint32_t *ring, uint32_t lo, uint32_t hi) {
+    const uint32_t k = lo >> 5;
+    const uint32_t f = __funnelshift_r(ring[k % EX_RING], ring[(k + 1u) % EX_RING], lo);   // 32 tests from lo on
+    return __popc(f & (FULL >> (32u - min(hi - lo, 32u))));
+}
+
+// ring: EX_SMEM_WORDS of shared memory of this warp, 16-byte aligned (mask
+// words, row pointers, windows).  The warp's words are wb .. of n_words, n
+// individuals.  A function of its own, so that its registers do not raise the
+// spills of the whole stack machine; a call costs little beside the words that
+// it walks.
+template <int WPL>
+__device__ __noinline__ RowWords<WPL> exist_run(const uint32_t *rp, const uint32_t *vals, const ValueTest test,
+                                                uint32_t n, uint32_t n_words, uint32_t wb, uint32_t *ring) {
+    const uint32_t lane = threadIdx.x & 31u;
+    RowWords<WPL> out;
+#pragma unroll
+    for (int s = 0; s < WPL; ++s) out.v[s] = 0u;
+    const uint32_t w_end = min(wb + 32u * WPL, n_words);   // the warp's words [wb, w_end)
+    if (wb >= w_end) return out;
+    uint32_t *rows = ring + EX_RING, *stages = rows + 2u * EX_ROWS;
+    const bool rvec = (reinterpret_cast<uintptr_t>(rp) & 15u) == 0, vec = (reinterpret_cast<uintptr_t>(vals) & 15u) == 0;
+    const uint32_t i1 = min(32u * w_end, n);                   // past the warp's last individual
+    uint32_t c = ld_stream(rp + 32u * wb) & ~(EX_WIN - 1u);     // the next window to test
+    const uint32_t end = ld_stream(rp + i1);                    // the end of the warp's run
+    // Copy groups, numbered in the order of their commits (empty ones past the
+    // last batch or the run): a batch's row pointers, a window of elements.
+    uint32_t groups = 0;
+    auto commit = [&]() {
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        return groups++;
+    };
+    // row pointers 32w .. 32w + 128 (the last one ends the batch's last row) to their half of rows
+    auto copy_rows = [&](uint32_t w, uint32_t half) {
+        const uint32_t i = 32u * w;
+        if (i < i1) {
+            ex_copy<128>(rows + half * EX_ROWS, rp, i, i1 + 1u, rvec, lane);
+            if (lane == 0u && i + 128u <= i1)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                                 (uint32_t)__cvta_generic_to_shared(rows + half * EX_ROWS + 128u)),
+                             "l"(rp + i + 128u)
+                             : "memory");
+        }
+        return commit();
+    };
+    uint32_t slot = 0;   // window c's place of the ring; the next two follow
+    auto copy_window = [&](uint32_t at, uint32_t to) {
+        if (at < end) ex_copy<EX_WIN>(stages + (to >= EX_STAGES ? to - EX_STAGES : to) * EX_WIN, vals, at, end, vec, lane);
+        return commit();
+    };
+    static_assert(EX_STAGES == 3, "two windows in flight beside the one that is read");
+    if (rvec) prefetch_range(rp, 32u * wb, i1 + 1u, lane);
+    uint32_t half = 0, r = copy_rows(wb, 0u);                            // the next batch's group
+    uint32_t v0 = copy_window(c, 0u), v1 = copy_window(c + EX_WIN, 1u);   // window c's and the next one's
+#pragma unroll 1
+    for (uint32_t w0 = wb; w0 < w_end; w0 += 4u, half ^= 1u) {
+        ex_wait(groups - 1u - r);
+        r = copy_rows(w0 + 4u, half ^ 1u);
+        // this lane's rows [lo, hi); individuals past n have none
+        const uint32_t *p = rows + half * EX_ROWS + lane;
+        uint32_t lo[4], hi[4], longest = 0;
+#pragma unroll
+        for (uint32_t q = 0; q < 4u; ++q) {
+            lo[q] = p[32u * q];
+            hi[q] = p[32u * q + 1u];
+        }
+        if (32u * w0 + 128u > i1) {   // the last batch
+#pragma unroll
+            for (uint32_t q = 0; q < 4u; ++q)
+                if (32u * (w0 + q) + lane >= i1) lo[q] = hi[q] = end;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < 4u; ++q) longest = max(longest, hi[q] - lo[q]);
+        longest = __reduce_max_sync(FULL, longest);
+        const uint32_t e0 = __shfl_sync(FULL, lo[0], 0);
+        const uint32_t e1 = __reduce_max_sync(FULL, max(max(hi[0], hi[1]), max(hi[2], hi[3])));
+        uint32_t hit[4] = {0u, 0u, 0u, 0u};
+        if (e1 <= (e0 & ~(EX_WIN - 1u)) + 32u * EX_RING) {
+            while (c < e1) {
+                ex_wait(groups - 1u - v0);
+                ex_masks(stages + slot * EX_WIN, c, end, lane, test, ring + (c >> 5) % EX_RING);
+                __syncwarp();   // the window has been read, its masks are there
+                v0 = v1, v1 = copy_window(c + 2u * EX_WIN, slot + 2u);   // into the place of the window before c
+                slot = slot + 1u == EX_STAGES ? 0u : slot + 1u;
+                c += EX_WIN;
             }
-            const uint32_t word = __ballot_sync(FULL, hit), k = w0 + j - wb;
+#pragma unroll
+            for (uint32_t q = 0; q < 4u; ++q)
+                if (hi[q] > lo[q]) hit[q] = ex_count(ring, lo[q], hi[q]);
+            if (longest > 32u) {   // warp-uniform
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; ++q)
+#pragma unroll 1
+                    for (uint32_t at = lo[q] + 32u; at < hi[q] && !hit[q]; at += 32u) hit[q] = ex_count(ring, at, hi[q]);
+            }
+        } else {
+#pragma unroll
+            for (uint32_t q = 0; q < 4u; ++q) {
+                uint32_t at = lo[q];   // the row's next untested element
+#pragma unroll 1
+                for (;;) {
+                    const uint32_t first = __reduce_min_sync(FULL, !hit[q] && at < hi[q] ? at : FULL);
+                    if (first == FULL) break;
+                    const uint32_t p0 = first & ~(EX_WIN - 1u), p1 = min(p0 + EX_STAGES * EX_WIN, end);
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    __syncwarp();
+                    for (uint32_t x = 0; p0 + x < p1; x += EX_WIN) ex_copy<EX_WIN>(stages + x, vals, p0 + x, end, vec, lane);
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    __syncwarp();
+#pragma unroll 1
+                    for (uint32_t x = 0; p0 + x < p1; x += EX_WIN)
+                        ex_masks(stages + x, p0 + x, end, lane, test, ring + ((p0 + x) >> 5) % EX_RING);
+                    __syncwarp();
+                    const uint32_t stop = min(hi[q], p1);
+                    for (; at < stop && !hit[q]; at = min(stop, at + 32u)) hit[q] = ex_count(ring, at, stop);
+                    __syncwarp();
+                }
+            }
+            // the rings no longer hold what is before c: go on from this batch's end
+            c = e1 & ~(EX_WIN - 1u);
+            slot = 0;
+            v0 = copy_window(c, 0u), v1 = copy_window(c + EX_WIN, 1u);
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < 4u; ++q) {
+            const uint32_t word = __ballot_sync(FULL, hit[q] != 0u), j = w0 + q - wb;   // past the last word: no rows
 #pragma unroll
             for (int s = 0; s < WPL; ++s)
-                if (lane == k / WPL && k % WPL == (uint32_t)s) v[s] = word;
+                if (lane == j / WPL && j % WPL == (uint32_t)s) out.v[s] = word;
         }
-    };
-    for (uint32_t w0 = wb; w0 < w_end; w0 += 8u) {
-        batch(w0, ra);
-        ex_rows(ra, rp, w0 + 8u, w_end, n, lane);
-        if (w0 + 4u >= w_end) break;
-        batch(w0 + 4u, rb);
-        ex_rows(rb, rp, w0 + 12u, w_end, n, lane);
+        __syncwarp();   // the rows and masks of this batch have been read
     }
-}
-
-// exist_words with the test's kind resolved at compile time (one dispatch per
-// restriction, warp-uniform).
-template <int WPL>
-__device__ __forceinline__ void exist_words(const uint32_t *rp, const uint32_t *vals, const ValueTest &test,
-                                            uint32_t n, uint32_t n_words, uint32_t wb, uint32_t lane,
-                                            uint32_t (&v)[WPL]) {
-    if (test.mode == ValueTest::FLOAT_CMP) {
-        const float t = __uint_as_float(test.arg);
-        if (test.cmp == HEDL_OP_DGE)
-            exist_words<WPL>(rp, vals, FloatTest<HEDL_OP_DGE>{t}, n, n_words, wb, lane, v);
-        else if (test.cmp == HEDL_OP_DLE)
-            exist_words<WPL>(rp, vals, FloatTest<HEDL_OP_DLE>{t}, n, n_words, wb, lane, v);
-        else
-            exist_words<WPL>(rp, vals, FloatTest<HEDL_OP_DEQ>{t}, n, n_words, wb, lane, v);
-    } else if (test.mode == ValueTest::ID_EQ)
-        exist_words<WPL>(rp, vals, IdEqTest{test.arg}, n, n_words, wb, lane, v);
-    else
-        exist_words<WPL>(rp, vals, IdBitTest{test.bits}, n, n_words, wb, lane, v);
+    asm volatile("cp.async.wait_all;" ::: "memory");   // none is left for the next use of the rings
+    __syncwarp();
+    return out;
 }
 
 // The test of a D_DATA instruction on a numeric or string role (op word bit 8
 // or 9; aux = the op; b = threshold bits, string id or pattern id).
 __host__ __device__ __forceinline__ ValueTest value_test(const KBView &kb, uint32_t op_word, uint32_t b) {
     const uint32_t op = (op_word >> 16) & 0xFFu;
-    if (op == HEDL_OP_SEQ) return ValueTest{ValueTest::ID_EQ, 0u, b, nullptr};
-    if (op == HEDL_OP_SCONTAINS) return ValueTest{ValueTest::ID_BIT, 0u, 0u, kb.contain + (uint64_t)b * kb.contain_words};
-    return ValueTest{ValueTest::FLOAT_CMP, op, b, nullptr};
+    if (op == HEDL_OP_SEQ) return ValueTest{ValueTest::ID_EQ, b, nullptr};
+    if (op == HEDL_OP_SCONTAINS) return ValueTest{ValueTest::ID_BIT, 0u, kb.contain + (uint64_t)b * kb.contain_words};
+    return ValueTest{op == HEDL_OP_DGE ? ValueTest::GE : op == HEDL_OP_DLE ? ValueTest::LE : ValueTest::EQ, b, nullptr};
 }
 
 __device__ __forceinline__ uint64_t global_ns() {

@@ -32,6 +32,7 @@ struct ExecArgs {
     uint32_t *counts;     // [H][4] or null
     uint32_t *out_bits;   // [H][wp] or null
     uint32_t item_begin, item_end;
+    uint32_t ring_words;  // shared-memory words of the concrete-role walk's rings (0: no such role)
     uint32_t use_queue;   // 1: dynamic queue with dependency waits; 0: static striding, no waits
 };
 
@@ -42,7 +43,9 @@ struct Smem {
     uint32_t item;
     uint32_t ok;
     uint32_t pad[2];
-    uint32_t filler[1];   // staged plans: the segment's filler row (wp words) from here on
+    // from here on: for KBs with concrete roles EX_SMEM_WORDS a warp (their walk's
+    // rings, ExecArgs::ring_words in all), then a staged plan's filler row (wp words)
+    uint32_t tail[1];
 };
 
 // The last group with item_begin <= item.  A CTA's items only grow (the queue
@@ -192,7 +195,10 @@ __device__ void run_tile(const ExecArgs &A, const PlanHeader &hd, const Seg &seg
                         const uint32_t *rp = str ? kb.str[d.a].rp : kb.num[d.a].rp;
                         const uint32_t *vals =
                             str ? kb.str[d.a].ids : reinterpret_cast<const uint32_t *>(kb.num[d.a].vals);
-                        exist_words<WPL>(rp, vals, value_test(kb, d.op, d.b), kb.n, lim_w, wb, lane, top);
+                        const RowWords<WPL> o = exist_run<WPL>(rp, vals, value_test(kb, d.op, d.b), kb.n, lim_w, wb,
+                                                              sm.tail + warp * EX_SMEM_WORDS);
+#pragma unroll
+                        for (int s = 0; s < WPL; ++s) top[s] = o.v[s];
                     }
                 } else
                     data_words<WPL>(kb.props + (uint64_t)d.a * kb.prop_stride, (d.op >> 16) & 0xFFu,
@@ -203,7 +209,7 @@ __device__ void run_tile(const ExecArgs &A, const PlanHeader &hd, const Seg &seg
                 const DevCSR g = kb.csr[2u * d.a + inv];
                 if constexpr (STAGE) {
                     const uint32_t kind = (d.op >> 16) & 0xFFu;
-                    role_stream<WPL, BLK>(g, sm.filler, kind, d.b, kb.n, lim_w, wb, lane, top, kind == HEDL_OP_FORALL);
+                    role_stream<WPL, BLK>(g, sm.tail + A.ring_words, kind, d.b, kb.n, lim_w, wb, lane, top, kind == HEDL_OP_FORALL);
                 } else {
                     const uint32_t *filler = (d.ref & REF_SLOT) ? slots + (uint64_t)(d.ref & ~REF_SLOT) * kb.wp
                                                                 : kb.concepts + (uint64_t)d.ref * kb.wp;
@@ -557,9 +563,9 @@ __device__ __forceinline__ void stage_filler(const KBView &kb, const uint32_t *s
 // whole stack machine.
 template <int NW, int WPL, bool STAGE, int BLK, bool FULL = false, bool GROUPS = true, bool CONCRETE = true>
 __global__ void __launch_bounds__(NW * 32, (FULL ? 64 : (GROUPS ? 24 : 32)) / NW) exec_kernel(ExecArgs A) {
-    // the host sizes the dynamic shared memory as stack_smem_bytes + 16 (+ a staged filler)
+    // the host sizes the dynamic shared memory (smem_bytes)
     using SmemT = Smem<NW, WPL>;
-    static_assert(offsetof(SmemT, filler) ==
+    static_assert(offsetof(SmemT, tail) ==
                       sizeof(uint32_t) * NW * STACK_MAX * WPL * 32 + sizeof(uint64_t) * NW * PF_SLOTS + 16,
                   "the shared-memory layout and its host-side size disagree");
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -627,7 +633,7 @@ __global__ void __launch_bounds__(NW * 32, (FULL ? 64 : (GROUPS ? 24 : 32)) / NW
         } else {
             if constexpr (STAGE) {
                 if (seg.filler != NO_FILLER) {
-                    stage_filler(A.kb, slots, seg.filler, sm.filler);
+                    stage_filler(A.kb, slots, seg.filler, sm.tail + A.ring_words);
                     __syncthreads();
                 }
             }
@@ -697,8 +703,10 @@ KernelFn pick(const Tuning &t, bool stage, bool groups, bool concrete) {
     return stage ? pick_t<true, 8>(t.warps, t.wpl) : pick_t<false, 8>(t.warps, t.wpl);
 }
 
+uint32_t ring_words(const hedl_kb *kb, const Tuning &t) { return kb->has_concrete() ? t.warps * EX_SMEM_WORDS : 0u; }
+
 size_t smem_bytes(const hedl_kb *kb, const Tuning &t, bool stage) {
-    size_t b = stack_smem_bytes(t) + 16;   // stacks, leaf tables, then item / ok / pad
+    size_t b = stack_smem_bytes(t) + 16 + 4ull * ring_words(kb, t);   // stacks, leaf tables, item / ok / pad, rings
     if (stage) b += 4ull * kb->wp;
     return b;
 }
@@ -715,7 +723,8 @@ int exec_occupancy(const hedl_kb *kb, const Tuning &t, bool groups, int *blocks_
     const bool stage = use_staging(kb, t);
     KernelFn fn = pick(t, stage, groups, kb->has_concrete());
     size_t smem = smem_bytes(kb, t, stage);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit, not this plan's size: plans of other sizes share the kernel
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kb->smem_optin);
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, (int)(t.warps * 32), smem);
     return e;
@@ -732,6 +741,7 @@ int launch_exec(const hedl_kb *kb, const PlanImpl *p, uint32_t *counts, uint32_t
     if (t.ctas_per_sm && (int)t.ctas_per_sm < bps) bps = (int)t.ctas_per_sm;
     ExecArgs A{};
     A.kb = kb->view();
+    A.ring_words = ring_words(kb, t);
     A.ws = (uint8_t *)ws;
     A.counts = counts;
     A.out_bits = out_bits;

@@ -167,6 +167,12 @@ constexpr int PLAN_ONLY_SMS = 152;               // planning-only handles plan f
 // round of a segment, in code order.
 constexpr int PF_SLOTS = 8;
 
+// A concrete-role walk's rings, per warp: mask words, two batches of row
+// pointers (128 and the one after them), EX_STAGES windows of values (4.4 KB,
+// so that 32 warps of a CTA fit beside their stacks).
+constexpr uint32_t EX_RING = 64, EX_ROWS = 132, EX_LOADS = 8, EX_WIN = 32 * EX_LOADS, EX_STAGES = 3;
+constexpr uint32_t EX_SMEM_WORDS = EX_RING + 2 * EX_ROWS + EX_STAGES * EX_WIN;
+
 // Shared-memory bytes of the interpreter's stacks and leaf tables (per CTA).
 inline size_t stack_smem_bytes(const Tuning &t) {
     return sizeof(uint32_t) * (size_t)t.warps * STACK_MAX * t.wpl * 32 + sizeof(uint64_t) * (size_t)t.warps * PF_SLOTS;

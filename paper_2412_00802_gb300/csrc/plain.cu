@@ -57,12 +57,12 @@ __global__ void role_kernel(DevCSR g, const uint32_t *filler, uint32_t kind, uin
 // subject's values).
 __global__ void exist_kernel(const uint32_t *rp, const uint32_t *vals, ValueTest test, uint32_t *out, uint32_t n,
                              uint32_t n_words, uint32_t wp) {
+    __shared__ __align__(16) uint32_t ring[PT / 32][EX_SMEM_WORDS];
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; wg * 32u < wp; wg += warps) {
-        uint32_t v[1];
-        exist_words<1>(rp, vals, test, n, n_words, wg * 32u, lane, v);
-        if (wg * 32u + lane < wp) out[wg * 32u + lane] = v[0];
+        const RowWords<1> v = exist_run<1>(rp, vals, test, n, n_words, wg * 32u, ring[threadIdx.x >> 5]);
+        if (wg * 32u + lane < wp) out[wg * 32u + lane] = v.v[0];
     }
 }
 
