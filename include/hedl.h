@@ -396,7 +396,7 @@ typedef struct {
     uint32_t stage_fillers;    /* 1: copy a role restriction's filler row into shared memory once per
                                   work item when it fits (then a segment reads at most one role
                                   restriction); 0: gather filler bits from global memory */
-    uint32_t role_block;       /* 4 or 8: 32-edge chunks the role walk loads per step */
+    uint32_t role_block;       /* 4 or 8: kept for callers that set it; the role walk's windows have one size */
     uint32_t full_occupancy;   /* 1: with 8 warps, 1 word per lane and no staging, use the build
                                   limited to 32 registers so 8 CTAs fit per SM */
 } hedl_tuning;

@@ -249,20 +249,25 @@ __device__ __forceinline__ void role_words(const DevCSR g, const uint32_t *fille
 // A word whose every lane is decided (cap reached or row ended) makes the
 // stream jump to the next word's first edge.  Word k of the warp goes to lane
 // k / WPL, slot k % WPL.  n_words bounds the warp's words; lanes of
-// individuals >= n hold empty rows and emit 0.
-template <int WPL, int BLK>
-__device__ __forceinline__ void role_stream(const DevCSR g, const uint32_t *filler, uint32_t kind, uint32_t n_arg,
-                                            uint32_t n, uint32_t n_words, uint32_t wb, uint32_t lane,
-                                            uint32_t (&v)[WPL], bool filler_inverted = false) {
-    static_assert(BLK >= 1 && BLK <= 32, "a block holds 1..32 chunks");
-    constexpr uint32_t BE = 32u * BLK;     // edges per block
+// individuals >= n hold empty rows and emit 0.  A function of its own, with
+// registers of its own: inlined, the stack machine around it spilled.
+template <int WPL>
+struct RowWords {
+    uint32_t v[WPL];
+};
+template <int WPL>
+__device__ __noinline__ RowWords<WPL> role_stream(const uint32_t *rp, const uint32_t *col, const uint32_t *filler,
+                                                  uint32_t kind, uint32_t n_arg, uint32_t n, uint32_t n_words,
+                                                  uint32_t wb, bool filler_inverted) {
+    constexpr uint32_t BLK = 4, BE = 32u * BLK;     // chunks and edges per block
+    const uint32_t lane = threadIdx.x & 31u;
+    RowWords<WPL> out;
+    uint32_t (&v)[WPL] = out.v;
     const uint32_t neg = (kind == HEDL_OP_FORALL && !filler_inverted) ? 1u : 0u;
     const uint64_t cap = decide_cap(kind, n_arg);
-    const uint32_t *__restrict__ rp = g.rp;
-    const uint32_t *__restrict__ col = g.col;
 #pragma unroll
     for (int s = 0; s < WPL; ++s) v[s] = 0u;
-    if (wb >= n_words) return;
+    if (wb >= n_words) return out;
     const uint32_t K = min(32u * WPL, n_words - wb);
     auto put = [&](uint32_t k, uint32_t word) {
 #pragma unroll
@@ -272,7 +277,7 @@ __device__ __forceinline__ void role_stream(const DevCSR g, const uint32_t *fill
     auto lane_valid = [&](uint32_t k) { return (wb + k) * 32u + lane < n; };
     if (cap == 0) {   // decided before any edge (at least 0): every individual
         for (uint32_t k = 0; k < K; ++k) put(k, __ballot_sync(FULL, lane_valid(k)));
-        return;
+        return out;
     }
     // row pointers of words k, k+1, k+2 (empty rows for lanes past n or words past K)
     auto ld_rows = [&](uint32_t k, uint32_t &lo, uint32_t &hi) {
@@ -307,7 +312,7 @@ __device__ __forceinline__ void role_stream(const DevCSR g, const uint32_t *fill
     uint32_t pf[BLK];
     auto fetch = [&](uint32_t at) {
 #pragma unroll
-        for (int u = 0; u < BLK; ++u) pf[u] = ld_stream(col + min(at + 32u * u + lane, E1 - 1u));
+        for (uint32_t u = 0; u < BLK; ++u) pf[u] = ld_stream(col + min(at + 32u * u + lane, E1 - 1u));
     };
     // L2 hints (no registers held): the warp's row pointers, and the edge
     // blocks two to four ahead of the one loading into registers
@@ -323,30 +328,30 @@ __device__ __forceinline__ void role_stream(const DevCSR g, const uint32_t *fill
     while (base < E1) {
         uint32_t hit[BLK];
 #pragma unroll
-        for (int u = 0; u < BLK; ++u) hit[u] = pf[u];
+        for (uint32_t u = 0; u < BLK; ++u) hit[u] = pf[u];
         const uint32_t nb = base + BE;
         if (nb < E1) fetch(nb);
         ahead(base + 4u * BE, 1u);
         // Positions past E1 reloaded edge E1-1; they lie beyond every row, so no rank counts them.
 #pragma unroll
-        for (int u = 0; u < BLK; ++u) hit[u] = (__funnelshift_r(filler[hit[u] >> 5], 0u, hit[u]) & 1u) ^ neg;
+        for (uint32_t u = 0; u < BLK; ++u) hit[u] = (__funnelshift_r(filler[hit[u] >> 5], 0u, hit[u]) & 1u) ^ neg;
         uint32_t mc = 0;   // lane c < BLK: mask of chunk c
 #pragma unroll
-        for (int u = 0; u < BLK; ++u) {
+        for (uint32_t u = 0; u < BLK; ++u) {
             const uint32_t m = __ballot_sync(FULL, hit[u]);
-            if (lane == (uint32_t)u) mc = m;
+            if (lane == u) mc = m;
         }
         const uint32_t pc = __popc(mc);
         uint32_t incl = pc;
 #pragma unroll
-        for (int o = 1; o < BLK; o <<= 1) {
+        for (uint32_t o = 1; o < BLK; o <<= 1) {
             const uint32_t t = __shfl_up_sync(FULL, incl, o);
-            if (lane >= (uint32_t)o) incl += t;
+            if (lane >= o) incl += t;
         }
         const uint32_t excl = incl - pc;
         // hits before block-relative position x in [0, BE]
         auto rank = [&](uint32_t x) -> uint32_t {
-            const uint32_t c = min(x >> 5, (uint32_t)BLK - 1);
+            const uint32_t c = min(x >> 5, BLK - 1u);
             const uint32_t e = __shfl_sync(FULL, excl, c);
             const uint32_t m = __shfl_sync(FULL, mc, c);
             const uint32_t sh = x - 32u * c;   // 0..32
@@ -367,12 +372,12 @@ __device__ __forceinline__ void role_stream(const DevCSR g, const uint32_t *fill
             }
             next_word();
         }
-        if (finished) return;
+        if (finished) return out;
         // word k spans past this block: skip the rest of it once every lane is decided
         const bool decided = !lane_valid(k) || hi0 <= nb || (uint64_t)cnt >= cap;
         if (__all_sync(FULL, decided)) {
             put(k, __ballot_sync(FULL, lane_valid(k) && role_pred(kind, cnt, n_arg)));
-            if (++k == K) return;
+            if (++k == K) return out;
             const uint32_t nxt = ew1;                  // the next word's first edge
             next_word();
             if (nxt != nb && nxt < E1) {
@@ -389,12 +394,8 @@ __device__ __forceinline__ void role_stream(const DevCSR g, const uint32_t *fill
         put(k, __ballot_sync(FULL, lane_valid(k) && role_pred(kind, cnt, n_arg)));
         cnt = 0;
     }
+    return out;
 }
-
-template <int WPL>
-struct RowWords {
-    uint32_t v[WPL];
-};
 
 __device__ __forceinline__ bool data_cmp(uint32_t cmp, float x, float t);
 

@@ -1021,7 +1021,7 @@ int build_plan_parallel(const hedl_kb *kb, const uint64_t *progs, const uint32_t
     p->info.n_segments = hd.n_segs;
     p->info.n_slots = hd.n_slots;
     p->info.n_levels = hd.n_levels;
-    p->info.n_items = hd.n_items;
+    p->info.n_items = p->n_items = hd.n_items;
     p->info.tile_words = hd.tile_words;
     p->info.warp_words = hd.warp_words;
     p->info.workspace_bytes = p->ws_bytes;
@@ -1226,7 +1226,7 @@ int build_plan_device(const hedl_kb *kb, const uint64_t *progs, const uint32_t *
     p->info.n_segments = hd.n_segs;
     p->info.n_slots = hd.n_slots;
     p->info.n_levels = hd.n_levels;
-    p->info.n_items = hd.n_items;
+    p->info.n_items = p->n_items = hd.n_items;
     p->info.tile_words = hd.tile_words;
     p->info.warp_words = hd.warp_words;
     p->info.workspace_bytes = p->ws_bytes;

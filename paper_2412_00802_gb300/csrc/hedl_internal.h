@@ -78,6 +78,9 @@ struct DInsn {
 };
 inline uint32_t dop(uint32_t w) { return w & 0xFF; }
 
+// a dependency (an index of a task) on a transpose or walk, whose tiles are the fine ones
+constexpr uint32_t DEP_FINE = 0x80000000u;
+
 constexpr uint32_t NO_SLOT = 0xFFFFFFFFu;
 constexpr uint32_t NO_HYP = 0xFFFFFFFFu;
 
@@ -122,14 +125,18 @@ struct Group {
     uint32_t item_begin;
     uint32_t seg_begin;  // index into gsegs[]
     uint32_t n_segs;
-    uint32_t level;
+    uint32_t level;      // bit 31: transposes or walks (fine tiles, one task a work item)
 };
+constexpr uint32_t GROUP_FINE = 0x80000000u;
 
 // Header at the start of the workspace (plan image).
 struct PlanHeader {
     uint32_t n_items, n_segs, n_groups, n_hyps;
     uint32_t n_tiles, tile_words, n_slots, flags;
-    uint32_t n_levels, n_deps, n_rgroups, warp_words;   // words a warp covers per round (32, 16, 8 or 4)
+    // warp_words: bits 0-7 the words a warp covers per round of a segment (32, 16, 8 or 4),
+    // bits 8-15 the words it covers of a transpose or walk, bits 16-23 the segments of a
+    // work item (plans with role groups; else one)
+    uint32_t n_levels, n_deps, n_rgroups, warp_words;
     uint64_t off_segs, off_groups, off_gsegs, off_deps;
     uint64_t off_code, off_level_items, off_ctr, off_slots;
     uint64_t off_rgroups, off_ft;
@@ -173,9 +180,15 @@ constexpr int PF_SLOTS = 8;
 constexpr uint32_t EX_RING = 64, EX_ROWS = 132, EX_LOADS = 8, EX_WIN = 32 * EX_LOADS, EX_STAGES = 3;
 constexpr uint32_t EX_SMEM_WORDS = EX_RING + 2 * EX_ROWS + EX_STAGES * EX_WIN;
 
-// Shared-memory bytes of the interpreter's stacks and leaf tables (per CTA).
+// Segments a CTA prepares together (one work item), and the instructions of
+// each that it keeps in shared memory.
+constexpr int SEG_BATCH = 8, SEG_CODE = 16;
+
+// Shared-memory bytes of the interpreter's stacks and of a work item's
+// segments: descriptors, code, leaf tables and their sizes (per CTA).
 inline size_t stack_smem_bytes(const Tuning &t) {
-    return sizeof(uint32_t) * (size_t)t.warps * STACK_MAX * t.wpl * 32 + sizeof(uint64_t) * (size_t)t.warps * PF_SLOTS;
+    return sizeof(uint32_t) * (size_t)t.warps * STACK_MAX * t.wpl * 32 +
+           SEG_BATCH * (sizeof(Seg) + SEG_CODE * sizeof(DInsn) + PF_SLOTS * sizeof(uint64_t) + 2 * sizeof(uint32_t));
 }
 
 struct PlanImpl;
@@ -285,6 +298,7 @@ struct PlanImpl {
     int bps = 0;                         // resident CTAs per SM of the interpreter
     bool staged = false;                 // role fillers staged in shared memory (one role leaf per segment)
     uint32_t n_rgroups = 0;              // bit-sliced role groups
+    uint32_t n_items = 0;                // work items
     // plain path: validated programs
     std::vector<uint64_t> progs;
     std::vector<uint32_t> offs;

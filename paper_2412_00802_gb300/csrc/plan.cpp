@@ -758,9 +758,12 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     for (uint32_t s_ = 0; s_ < NS; ++s_) {
         segs[s_].dep_off = (uint32_t)deps.size();
         if (segs[s_].kind == TASK_WALK) {
-            deps.push_back(s_ - 1);
+            deps.push_back((s_ - 1) | DEP_FINE);
         } else {
-            for (uint32_t q = read_off[s_]; q < read_off[s_ + 1]; ++q) deps.push_back(seg_of_slot[read_list[q]]);
+            for (uint32_t q = read_off[s_]; q < read_off[s_ + 1]; ++q) {
+                const uint32_t by = seg_of_slot[read_list[q]];
+                deps.push_back(by | (segs[by].kind == TASK_SEGMENT ? 0u : DEP_FINE));
+            }
         }
         segs[s_].dep_cnt = (uint32_t)deps.size() - segs[s_].dep_off;
         n_levels = std::max(n_levels, task_level[s_] + 1);
@@ -802,11 +805,35 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     }
     const uint32_t TW = t.warps * WW * t.wpl * rounds;
     const uint32_t n_tiles = (kb->wp + TW - 1) / TW;
+    // Transposes and walks have tiles of their own, FW words a warp: 32, or
+    // fewer while the walks of an average level that has some would give the
+    // resident warps (24 an SM at 80 registers) less than four items each to
+    // even out.  (Large batches: 16 items a warp, 8 to 16 words, was no faster.)
+    uint32_t FW = 0, n_fine = 0;
+    if (!rgroups.empty()) {
+        std::vector<uint8_t> walks_at(n_levels, 0);
+        for (uint32_t s_ = NSEG; s_ < NS; ++s_)
+            if (segs[s_].kind == TASK_WALK) walks_at[task_level[s_]] = 1;
+        const uint64_t levels = std::count(walks_at.begin(), walks_at.end(), (uint8_t)1);
+        const uint64_t resident = 24ull * (uint64_t)std::max(kb->n_sms, 1);
+        FW = 32;
+        while (FW > 4 && rgroups.size() * kb->wp < 4 * resident * FW * levels) FW >>= 1;
+        n_fine = (kb->wp + t.warps * FW - 1) / (t.warps * FW);
+    }
+    auto fine = [&](uint32_t task) { return segs[task].kind != TASK_SEGMENT; };
+    // Segments of a work item: as many (up to SEG_BATCH) as leave an average
+    // level two items a resident CTA; a staged filler belongs to one segment.
+    uint32_t SB = 1;
+    if (!rgroups.empty() && !staged) {
+        const uint64_t ctas = std::max<uint64_t>(1, 24ull * (uint64_t)std::max(kb->n_sms, 1) / t.warps);
+        SB = (uint32_t)std::min<uint64_t>(SEG_BATCH, std::max<uint64_t>(1, (uint64_t)NSEG * n_tiles / (2 * ctas * n_levels)));
+    }
     std::vector<uint32_t> order(NS);
     for (uint32_t s = 0; s < NS; ++s) order[s] = s;
     std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
         if (task_level[x] != task_level[y]) return task_level[x] < task_level[y];
-        return task_key[x] < task_key[y];
+        if (task_key[x] != task_key[y]) return task_key[x] < task_key[y];
+        return fine(x) < fine(y);
     });
     std::vector<Group> groups;
     std::vector<uint32_t> gsegs;
@@ -819,14 +846,16 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
         g.seg_begin = (uint32_t)gsegs.size();
         g.level = task_level[s0];
         uint32_t k2 = k;
-        while (k2 < NS && task_level[order[k2]] == g.level && task_key[order[k2]] == task_key[s0]) {
+        while (k2 < NS && task_level[order[k2]] == g.level && task_key[order[k2]] == task_key[s0] &&
+               fine(order[k2]) == fine(s0)) {
             gsegs.push_back(order[k2]);
             ++k2;
         }
         g.n_segs = k2 - k;
-        items += (uint64_t)g.n_segs * n_tiles;
-        groups.push_back(g);
+        items += fine(s0) ? (uint64_t)g.n_segs * n_fine : (uint64_t)((g.n_segs + SB - 1) / SB) * n_tiles;
         level_items[g.level + 1] = (uint32_t)items;
+        if (fine(s0)) g.level |= GROUP_FINE;
+        groups.push_back(g);
         k = k2;
     }
     for (uint32_t l = 1; l <= n_levels; ++l) level_items[l] = std::max(level_items[l], level_items[l - 1]);
@@ -848,7 +877,7 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     hd.n_hyps = H;
     hd.n_tiles = n_tiles;
     hd.tile_words = TW;
-    hd.warp_words = WW;
+    hd.warp_words = WW | FW << 8 | (FW ? SB << 16 : 0u);
     hd.n_slots = n_slots;
     hd.flags = flags;
     hd.n_levels = n_levels;
@@ -883,7 +912,8 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     p->info.n_segments = NS;
     p->info.n_slots = n_slots;
     p->info.n_levels = n_levels;
-    p->info.n_items = (uint32_t)items;
+    p->n_items = (uint32_t)items;
+    p->info.n_items = NS * n_tiles;
     p->info.tile_words = TW;
     p->info.warp_words = WW;
     p->info.workspace_bytes = p->ws_bytes;

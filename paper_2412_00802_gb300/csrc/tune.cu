@@ -21,57 +21,24 @@ bool same_shape(const Tuning &a, const Tuning &b) {
 
 std::vector<Tuning> candidates(const Tuning &base) {
     std::vector<Tuning> out;
+    auto add = [&](uint32_t stage, uint32_t warps, uint32_t wpl, uint32_t rounds, uint32_t full_occupancy) {
+        Tuning t = base;   // role_block included: it shapes no code
+        t.stage = stage;
+        t.warps = warps;
+        t.wpl = wpl;
+        t.rounds = rounds;
+        t.ctas_per_sm = 0;
+        t.full_occupancy = full_occupancy;
+        out.push_back(t);
+    };
     for (uint32_t stage : {1u, 0u})
         for (uint32_t warps : {8u, 16u, 32u})
-            for (uint32_t rounds : {1u, 2u, 4u})
-                for (uint32_t blk : {4u, 8u}) {
-                    Tuning t = base;
-                    t.stage = stage;
-                    t.warps = warps;
-                    t.wpl = 1;
-                    t.rounds = rounds;
-                    t.role_block = blk;
-                    t.ctas_per_sm = 0;
-                    t.full_occupancy = 0;
-                    out.push_back(t);
-                }
+            for (uint32_t rounds : {1u, 2u, 4u}) add(stage, warps, 1, rounds, 0);
     for (uint32_t warps : {1u, 2u})
-        for (uint32_t rounds : {1u, 2u, 4u})
-            for (uint32_t blk : {4u, 8u}) {
-                Tuning t = base;
-                t.stage = 0;
-                t.warps = warps;
-                t.wpl = 1;
-                t.rounds = rounds;
-                t.role_block = blk;
-                t.ctas_per_sm = 0;
-                t.full_occupancy = 0;
-                out.push_back(t);
-            }
-    for (uint32_t rounds : {1u, 2u, 4u})
-        for (uint32_t blk : {4u, 8u}) {
-            Tuning t = base;
-            t.stage = 0;
-            t.warps = 8;
-            t.wpl = 1;
-            t.rounds = rounds;
-            t.role_block = blk;
-            t.ctas_per_sm = 0;
-            t.full_occupancy = 1;
-            out.push_back(t);
-        }
+        for (uint32_t rounds : {1u, 2u, 4u}) add(0, warps, 1, rounds, 0);
+    for (uint32_t rounds : {1u, 2u, 4u}) add(0, 8, 1, rounds, 1);
     for (uint32_t stage : {1u, 0u})
-        for (uint32_t warps : {8u, 16u}) {
-            Tuning t = base;
-            t.stage = stage;
-            t.warps = warps;
-            t.wpl = 4;
-            t.rounds = 1;
-            t.role_block = 8;
-            t.ctas_per_sm = 0;
-            t.full_occupancy = 0;
-            out.push_back(t);
-        }
+        for (uint32_t warps : {8u, 16u}) add(stage, warps, 4, 1, 0);
     return out;
 }
 
