@@ -228,8 +228,8 @@ typedef struct hedl_plan hedl_plan;
 
 #define HEDL_NO_CSE     1u   /* no sharing of common sub-concepts */
 #define HEDL_NO_GRAPH   2u   /* always launch directly (default: a plan's first execution
-                                launches directly, later ones capture and then replay a
-                                CUDA graph) */
+                                launches directly, later ones that score capture and then
+                                replay a CUDA graph) */
 #define HEDL_PLAIN      4u   /* one launch per operation per hypothesis */
 #define HEDL_LEVELS     8u   /* one launch per dependency level, no device waits */
 #define HEDL_NO_SLICE  16u   /* evaluate every role restriction on its own CSR walk

@@ -415,6 +415,9 @@ int execute(hedl_kb *kb, const PlanImpl *pc, uint32_t *counts, uint32_t *out_bit
         // a device-built plan: its image is copied within the device
         e = cudaMemcpyAsync(ws, p->dev_image, p->image_bytes, cudaMemcpyDeviceToDevice, st);
         if (e) return cuda_fail(e, "plan copy");
+    } else if (upload && p->image_bytes <= SMALL_IMAGE) {
+        const int ue = upload_small_plan(p, ws, st);
+        if (ue) return cuda_fail(ue, "plan upload");
     } else if (upload) {
         // pageable source: the copy is complete (staged) when the call returns,
         // so the host image may be reused at once
@@ -424,7 +427,8 @@ int execute(hedl_kb *kb, const PlanImpl *pc, uint32_t *counts, uint32_t *out_bit
         e = cudaMemsetAsync((uint8_t *)ws + p->ctr_off, 0, p->ctr_bytes, st);
         if (e) return cuda_fail(e, "counter reset");
     }
-    const bool use_graph = !(p->flags & (HEDL_NO_GRAPH | HEDL_LEVELS)) && p->runs++ > 0;
+    // a graph saves the launch of a second kernel: sets alone need only the interpreter
+    const bool use_graph = counts && !(p->flags & (HEDL_NO_GRAPH | HEDL_LEVELS)) && p->runs++ > 0;
     if (!use_graph) {
         int le = launch_exec(kb, p, counts, out_bits, ws, st);
         return le ? cuda_fail(le, "exec launch") : HEDL_OK;

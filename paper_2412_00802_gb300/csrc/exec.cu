@@ -19,8 +19,10 @@
 #include <cuda_runtime.h>
 
 #include <cstddef>
+#include <cstring>
 
 #include "device_common.cuh"
+#include "launch.cuh"
 
 namespace hedl {
 
@@ -78,7 +80,7 @@ __device__ __forceinline__ Group find_group(const Group *groups, uint32_t n_grou
 
 // Bounded wait for one producer task (dep: its index, DEP_FINE if it has fine tiles).
 __device__ __forceinline__ bool wait_dep(const PlanHeader &hd, uint32_t dep, uint32_t *done, Counters *ctr,
-                                         uint32_t fine_tiles) {
+                                         uint32_t fine_tiles, uint32_t *status) {
     const uint32_t *flag = done + (dep & ~DEP_FINE);
     const uint32_t target = dep & DEP_FINE ? fine_tiles : hd.n_tiles;
     if (ld_acquire(flag) >= target) return true;
@@ -88,7 +90,7 @@ __device__ __forceinline__ bool wait_dep(const PlanHeader &hd, uint32_t dep, uin
     while (ld_acquire(flag) < target) {
         if (*(volatile uint32_t *)&ctr->abort) return false;
         if (global_ns() - t0 > hd.timeout_ns || ++spins > max_spins) {
-            atomicOr(&ctr->err, ST_TIMEOUT);
+            atomicOr(status, ST_TIMEOUT);
             atomicExch(&ctr->abort, 1u);
             return false;
         }
@@ -151,7 +153,7 @@ __device__ bool prepare_task(const ExecArgs &A, const PlanHeader &hd, Smem<NW, W
     bool ok = true;
     if (A.use_queue) {
         const uint32_t *deps = reinterpret_cast<const uint32_t *>(A.ws + hd.off_deps) + dep_off;
-        for (uint32_t k = lane; k < dep_cnt && ok; k += 32) ok = wait_dep(hd, deps[k], done, ctr, fine_tiles);
+        for (uint32_t k = lane; k < dep_cnt && ok; k += 32) ok = wait_dep(hd, deps[k], done, ctr, fine_tiles, A.kb.status);
     }
     return __all_sync(FULL, ok);
 }
@@ -675,6 +677,7 @@ __global__ void __launch_bounds__(NW * 32, (FULL ? 64 : (GROUPS ? 24 : 32)) / NW
                   "the shared-memory layout and its host-side size disagree");
     extern __shared__ __align__(16) uint8_t smem_raw[];
     Smem<NW, WPL> &sm = *reinterpret_cast<Smem<NW, WPL> *>(smem_raw);
+    pdl_wait();   // for a plan that upload_kernel puts into the workspace
     const PlanHeader hd = *reinterpret_cast<const PlanHeader *>(A.ws);
     const Group *groups = reinterpret_cast<const Group *>(A.ws + hd.off_groups);
     const uint32_t *gsegs = reinterpret_cast<const uint32_t *>(A.ws + hd.off_gsegs);
@@ -726,7 +729,7 @@ __global__ void __launch_bounds__(NW * 32, (FULL ? 64 : (GROUPS ? 24 : 32)) / NW
         if (seg.kind != TASK_SEGMENT && !GROUPS) {
             // a build without role groups was given a plan with them (the host never does this)
             if (threadIdx.x == 0) {
-                atomicOr(&ctr->err, ST_DEVICE_CHECK);
+                atomicOr(A.kb.status, ST_DEVICE_CHECK);
                 atomicExch(&ctr->abort, 1u);
             }
         } else if (seg.kind == TASK_TRANSPOSE) {
@@ -771,18 +774,29 @@ __global__ void __launch_bounds__(NW * 32, (FULL ? 64 : (GROUPS ? 24 : 32)) / NW
     }
 }
 
-// (TP, FP) accumulators -> (TP, FP, FN, TN); records a device error on the handle.
+// (TP, FP) accumulators -> (TP, FP, FN, TN).
 __global__ void finalize_kernel(KBView kb, const uint8_t *ws, uint32_t *counts) {
     const PlanHeader *hd = reinterpret_cast<const PlanHeader *>(ws);
     const Counters *ctr = reinterpret_cast<const Counters *>(ws + hd->off_ctr);
     const uint32_t *acc = reinterpret_cast<const uint32_t *>(ctr + 1) + hd->n_segs + 1;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && ctr->err) atomicOr(kb.status, ctr->err);
-    if (!counts) return;
     for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < hd->n_hyps; h += gridDim.x * blockDim.x) {
         const uint32_t tp = acc[2 * h], fp = acc[2 * h + 1];
         uint4 c = make_uint4(tp, fp, kb.n_pos - tp, kb.n_neg - fp);
         *reinterpret_cast<uint4 *>(counts + 4ull * h) = c;
     }
+}
+
+// Puts a small plan's image, which comes as the kernel's argument, into the
+// workspace.  A host-to-device copy of 2 KB waits for the copy engine and the
+// interpreter for it; this is one more short kernel, which the interpreter's
+// blocks start behind (pdl_wait).
+struct SmallImage {
+    uint4 data[SMALL_IMAGE / 16];
+};
+__global__ void upload_kernel(const __grid_constant__ SmallImage img, uint4 *ws, uint32_t n) {
+    pdl_trigger();
+    pdl_wait();   // an earlier launch may still use the workspace
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) ws[i] = img.data[i];
 }
 
 using KernelFn = void (*)(ExecArgs);
@@ -843,6 +857,12 @@ int exec_occupancy(const hedl_kb *kb, const Tuning &t, bool groups, int *blocks_
     return e;
 }
 
+int upload_small_plan(const PlanImpl *p, void *ws, void *stream) {
+    SmallImage img;
+    memcpy(img.data, p->image.data(), p->image_bytes);
+    return launch_pdl(upload_kernel, 1u, 128u, 0, (cudaStream_t)stream, img, (uint4 *)ws, (uint32_t)(p->image_bytes / 16));
+}
+
 int launch_exec(const hedl_kb *kb, const PlanImpl *p, uint32_t *counts, uint32_t *out_bits, void *ws,
                 void *stream) {
     cudaStream_t s = (cudaStream_t)stream;
@@ -877,10 +897,10 @@ int launch_exec(const hedl_kb *kb, const PlanImpl *p, uint32_t *counts, uint32_t
         A.item_begin = 0;
         A.item_end = n_items;
         uint32_t grid = std::min<uint32_t>(std::max<uint32_t>(n_items, 1), (uint32_t)(bps * kb->n_sms));
-        fn<<<grid, t.warps * 32, smem, s>>>(A);
-        cudaError_t le = cudaGetLastError();
+        const cudaError_t le = launch_pdl(fn, grid, t.warps * 32, smem, s, A);
         if (le != cudaSuccess) return le;
     }
+    if (!counts) return cudaSuccess;
     finalize_kernel<<<std::max<uint32_t>(1, std::min<uint32_t>((p->n_hyps + 255) / 256, 1024)), 256, 0, s>>>(
         kb->view(), (const uint8_t *)ws, counts);
     return cudaGetLastError();

@@ -329,6 +329,9 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
 uint64_t hash_programs(const uint64_t *progs, const uint32_t *offs, uint32_t H);
 
 // exec.cu / plain.cu / kb.cu launchers (return cudaError_t as int)
+// Plans of up to SMALL_IMAGE bytes (a lone hypothesis has 2 KB) go to the workspace as a kernel's argument.
+constexpr size_t SMALL_IMAGE = 3840;
+int upload_small_plan(const PlanImpl *p, void *ws, void *stream);
 int launch_exec(const hedl_kb *kb, const PlanImpl *p, uint32_t *counts, uint32_t *out_bits, void *ws,
                 void *stream);
 // Whether plans for this KB and launch shape stage role fillers in shared memory.
