@@ -84,15 +84,18 @@ __device__ __forceinline__ bool wait_dep(const PlanHeader &hd, uint32_t dep, uin
     const uint32_t *flag = done + (dep & ~DEP_FINE);
     const uint32_t target = dep & DEP_FINE ? fine_tiles : hd.n_tiles;
     if (ld_acquire(flag) >= target) return true;
-    const uint64_t t0 = global_ns();
-    uint64_t spins = 0;
+    uint64_t t0 = 0, spins = 0;
     const uint64_t max_spins = hd.timeout_ns / 16 + 1000000ull;
     while (ld_acquire(flag) < target) {
-        if (*(volatile uint32_t *)&ctr->abort) return false;
-        if (global_ns() - t0 > hd.timeout_ns || ++spins > max_spins) {
-            atomicOr(status, ST_TIMEOUT);
-            atomicExch(&ctr->abort, 1u);
-            return false;
+        if ((++spins & 15u) == 0u) {   // the clock costs more than a look at the flag
+            if (*(volatile uint32_t *)&ctr->abort) return false;
+            const uint64_t t = global_ns();
+            if (!t0) t0 = t;
+            if (t - t0 > hd.timeout_ns || spins > max_spins) {
+                atomicOr(status, ST_TIMEOUT);
+                atomicExch(&ctr->abort, 1u);
+                return false;
+            }
         }
         __nanosleep(32);
     }
