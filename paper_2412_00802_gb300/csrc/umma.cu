@@ -5,7 +5,7 @@
 //
 // A persistent kernel: one CTA per SM walks the items (128 x UN output tile,
 // K range) blockIdx.x, blockIdx.x + gridDim.x, ... of one or two products.
-// Its six warps have fixed roles:
+// Its ten warps have fixed roles:
 //   warp 0 (one thread): the TMA producer.  It loads each 64-wide K block of
 //     the item's A (128 x 64) and B (UN x 64) (cp.async.bulk.tensor, 128-byte
 //     rows in the 128-byte swizzle; a K-major operand is one box, an MN-major
@@ -16,13 +16,23 @@
 //     UN-column TMEM accumulators and commits them to the stage's "empty"
 //     mbarrier; after an item's last block it commits to the accumulator's
 //     "tmem full" mbarrier;
-//   warps 2-5: the epilogue.  Each reads its 32-lane quarter of a finished
-//     accumulator with tcgen05.ld, adds the bias, applies ReLU or a mask (the
-//     backward pass's ReLU derivative), stores bf16 or FP32 rows, adds up the
-//     tile's columns or the fused output layer's sums where asked, and arrives
-//     on the accumulator's "tmem empty" mbarrier.
+//   warps 2-9: the epilogue.  Each reads its 32-lane quarter and one half of
+//     the columns of a finished accumulator with tcgen05.ld, adds the bias,
+//     applies ReLU or a mask (the backward pass's ReLU derivative), stores
+//     bf16 (through shared memory and TMA) or FP32 rows, adds up the tile's
+//     columns or the fused output layer's sums where asked, and arrives on the
+//     accumulator's "tmem empty" mbarrier.
 // With two accumulators, the epilogue of one item overlaps the loads and
 // MMAs of the next.
+//
+// What bounds a layer of many rows: with no epilogue at all the two layers of
+// 65,536 rows take 55 us, with no MMAs either 44 (an SM takes in 48 KB a K block
+// at 64 B a clock).  Four epilogue warps that stored from registers made it 96
+// us (76 without the stores, 64 without the output layer too): one warp a
+// scheduler waits out every latency, and its 16-byte stores touch 32 lines
+// each.  Eight warps, the next 32 columns loaded ahead, outputs by TMA, bias
+// and output weights (as FP32) from shared memory: 68.8 us; a training step of
+// 4,096 rows 61 -> 56 us.
 //
 // Tile width: a layer of a few thousand rows is bound by the latency of one
 // item (8 K blocks through one SM), not by the tensor cores, so the tile is
@@ -48,15 +58,22 @@ constexpr int UM = 128, UK = 64;
 constexpr uint32_t ROW = UK * 2;                     // 128-byte rows of a block
 constexpr uint32_t A_BYTES = UM * UK * 2;            // 16 KB
 constexpr uint32_t MN_GROUP = 64 * ROW;              // an MN-major box: 64 k rows of 64 elements
-constexpr int THREADS = 192;                         // producer, MMA issuer, 4 epilogue warps
+constexpr int EPI = 256;                             // threads of the epilogue's eight warps
+constexpr int THREADS = 64 + EPI;                    // producer, MMA issuer, epilogue
+constexpr int HEAD_N = 512;                          // columns whose bias and output weights fit in shared memory
+constexpr uint32_t OUT_BYTES = 32 * 32 * 2;          // a warp's 32 x 32 bf16 outputs
 template <int UN>
 struct Shape {
     static constexpr uint32_t B_BYTES = UN * UK * 2;
     static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
     static constexpr int STAGES = UN == 256 ? 4 : UN == 128 ? 6 : 8;   // 192 KB
     static constexpr uint32_t TMEM_COLS = 2 * UN;                      // two FP32 accumulators
-    static constexpr uint32_t CS_OFF = STAGES * STAGE_BYTES;           // column sums [4][UN]
-    static constexpr uint32_t BAR_OFF = CS_OFF + 4 * UN * 4;
+    static constexpr uint32_t OUT_OFF = STAGES * STAGE_BYTES;          // outputs on their way to TMA [8 warps]
+    static constexpr uint32_t CS_OFF = OUT_OFF + 8 * OUT_BYTES;        // column sums [4][UN]
+    static constexpr uint32_t BIAS_OFF = CS_OFF + 4 * UN * 4;          // [HEAD_N]
+    static constexpr uint32_t W3_OFF = BIAS_OFF + HEAD_N * 4;          // [2][HEAD_N], as FP32
+    static constexpr uint32_t HS_OFF = W3_OFF + 2 * HEAD_N * 4;        // the other half's output sums [2][128][2]
+    static constexpr uint32_t BAR_OFF = HS_OFF + 2 * UM * 2 * 4;
     static constexpr size_t SMEM = BAR_OFF + 256 + 1024;
     // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
     // (bits 7-9 and 10-12 = 1), operand majors at bits 15 and 16 (0 = K, 1 =
@@ -129,26 +146,25 @@ __device__ __forceinline__ void tmem_ld32(uint32_t ta, uint32_t (&r)[32]) {
         : "memory");
 }
 
-// Fused output layer on 32 columns of one row: the bf16-rounded activations
-// (what the unfused path stores and reads back) dotted with both rows of w3,
-// in four partial sums each (shorter FP32 chains).
-__device__ __forceinline__ void head32(const UmmaArgs &g, int col, const float (&v)[32], float (&a0)[4], float (&a1)[4]) {
-    const uint4 *w0 = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(g.w3) + col);
-    const uint4 *w1 = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(g.w3) + g.N + col);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const uint4 x = __ldg(w0 + q), y = __ldg(w1 + q);
-        const uint32_t xv[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 wx = *reinterpret_cast<const __nv_bfloat162 *>(&xv[e]);
-            const __nv_bfloat162 wy = *reinterpret_cast<const __nv_bfloat162 *>(&yv[e]);
-            const __nv_bfloat162 h = __floats2bfloat162_rn(v[q * 8 + 2 * e], v[q * 8 + 2 * e + 1]);
-            const float hl = __low2float(h), hh = __high2float(h);
-            a0[e] += hl * __low2float(wx) + hh * __high2float(wx);
-            a1[e] += hl * __low2float(wy) + hh * __high2float(wy);
-        }
-    }
+// Waits for the loads so far; tied to r, so that nothing reads r earlier.
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                   "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]),
+                   "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]),
+                   "+r"(r[30]), "+r"(r[31])::"memory");
+}
+
+__device__ __forceinline__ float2 unpack(uint32_t w) {   // two bf16
+    return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+}
+// a += b * c, two FP32 at a time
+__device__ __forceinline__ void fma2(float2 &a, float2 b, float2 c) {
+    asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %3};\n mov.b64 c, {%4, %5};\n"
+        " fma.rn.f32x2 a, b, c, a;\n mov.b64 {%0, %1}, a;\n}"
+        : "+f"(a.x), "+f"(a.y)
+        : "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
 }
 
 // Column sums over the warp's 32 rows of v, one row a lane: a butterfly that
@@ -166,26 +182,39 @@ __device__ __forceinline__ float colsum32(float (&v)[32], uint32_t lane) {
     return v[0];
 }
 
+// What the epilogue keeps in shared memory.
+struct EpiSmem {
+    const float *bias, *w3;   // [N], [2][N]
+    uint32_t out;             // this warp's 32 x 32 outputs, rows of 64 bytes in the 64-byte swizzle
+};
+
 // Epilogue of 32 columns of one row: bias, ReLU or mask, bf16 or FP32 store,
-// the fused output layer's partial sums, the warp's column sums (cs: its 32
-// entries, or null; all lanes of the warp call together, row < M or not).
-__device__ __forceinline__ void emit32(const UmmaArgs &g, void *C, int row, int col, const uint32_t (&r)[32],
-                                       float (&a0)[4], float (&a1)[4], float *cs, uint32_t lane) {
+// the fused output layer's partial sums (of the bf16-rounded outputs, which
+// the unfused path stores and reads back; four sums a row of w3, so that the
+// FP32 chains are short), the warp's column sums (cs: its 32 entries, or
+// null).  All lanes of the warp call together, row < M or not.
+//
+// A lane holds 64 contiguous bytes of one row: stored from registers, each of
+// its 16-byte stores touches 32 lines, and these stores took a fifth of a
+// forward pass.  The warp's 32 rows go through shared memory instead (no bank
+// conflicts in the 64-byte swizzle), from where TMA writes whole sectors.
+__device__ __forceinline__ void emit32(const UmmaArgs &g, const CUtensorMap *tc, void *C, int row, int col,
+                                       const uint32_t (&r)[32], const EpiSmem &es, float2 (&a0)[2], float2 (&a1)[2],
+                                       float *cs, uint32_t lane) {
     const bool in = row < g.M;
     float v[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
     if (g.bias) {
-        const float4 *b4 = reinterpret_cast<const float4 *>(g.bias + col);
+        const float4 *b4 = reinterpret_cast<const float4 *>(es.bias + col);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            const float4 b = __ldg(b4 + q);
-            v[4 * q] = __uint_as_float(r[4 * q]) + b.x;
-            v[4 * q + 1] = __uint_as_float(r[4 * q + 1]) + b.y;
-            v[4 * q + 2] = __uint_as_float(r[4 * q + 2]) + b.z;
-            v[4 * q + 3] = __uint_as_float(r[4 * q + 3]) + b.w;
+            const float4 b = b4[q];
+            v[4 * q] += b.x;
+            v[4 * q + 1] += b.y;
+            v[4 * q + 2] += b.z;
+            v[4 * q + 3] += b.w;
         }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
     }
     if (g.relu) {
 #pragma unroll
@@ -200,42 +229,70 @@ __device__ __forceinline__ void emit32(const UmmaArgs &g, void *C, int row, int 
             const uint32_t mw[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162 *>(&mw[e]);
-                if (!(__low2float(h) > 0.f)) v[q * 8 + 2 * e] = 0.f;
-                if (!(__high2float(h) > 0.f)) v[q * 8 + 2 * e + 1] = 0.f;
+                const float2 h = unpack(mw[e]);
+                if (!(h.x > 0.f)) v[q * 8 + 2 * e] = 0.f;
+                if (!(h.y > 0.f)) v[q * 8 + 2 * e + 1] = 0.f;
             }
         }
     }
-    if (g.w3) head32(g, col, v, a0, a1);
-    if (g.store && in) {
-        if (g.out_bf16) {
-            uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(C) + (size_t)row * g.ldc + col);
+    if (g.store && !g.out_bf16 && in) {
+        float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(C) + (size_t)row * g.ldc + col);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t w[4];
+        for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+    uint32_t w[16];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const __nv_bfloat162 h = __floats2bfloat162_rn(v[q * 8 + 2 * e], v[q * 8 + 2 * e + 1]);
-                    w[e] = *reinterpret_cast<const uint32_t *>(&h);
-                }
-                dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        } else {
-            float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(C) + (size_t)row * g.ldc + col);
+    for (int j = 0; j < 16; ++j) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+        w[j] = *reinterpret_cast<const uint32_t *>(&h);
+    }
+    if (g.store && g.out_bf16) {
+        // the warp's last outputs have been read
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        __syncwarp();
+        const uint32_t at = es.out + 64u * lane, x = lane >> 1 & 3u;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (uint32_t q = 0; q < 4; ++q)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + ((q ^ x) << 4)), "r"(w[4 * q]),
+                         "r"(w[4 * q + 1]), "r"(w[4 * q + 2]), "r"(w[4 * q + 3])
+                         : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0 && in) {   // rows past M are cut off
+            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                             reinterpret_cast<uint64_t>(tc)),
+                         "r"(col), "r"(row), "r"(es.out)
+                         : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+    }
+    if (g.w3) {
+        const float4 *x4 = reinterpret_cast<const float4 *>(es.w3 + col);
+        const float4 *y4 = reinterpret_cast<const float4 *>(es.w3 + g.N + col);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float2 h0 = unpack(w[2 * q]), h1 = unpack(w[2 * q + 1]);
+            const float4 x = x4[q], y = y4[q];
+            fma2(a0[0], h0, make_float2(x.x, x.y));
+            fma2(a1[0], h0, make_float2(y.x, y.y));
+            fma2(a0[1], h1, make_float2(x.z, x.w));
+            fma2(a1[1], h1, make_float2(y.z, y.w));
         }
     }
     if (cs) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = in ? __bfloat162float(__float2bfloat16_rn(v[j])) : 0.f;
+        for (int j = 0; j < 16; ++j) {
+            const float2 h = unpack(w[j]);
+            v[2 * j] = in ? h.x : 0.f;
+            v[2 * j + 1] = in ? h.y : 0.f;
+        }
         cs[lane] = colsum32(v, lane);
     }
 }
 
 // One or two products of one launch; product 1's items follow product 0's.
 struct Batch {
-    CUtensorMap ta[2], tb[2];
+    CUtensorMap ta[2], tb[2], tc[2];   // tc: bf16 outputs
     UmmaArgs g[2];
     int items0, items;
 };
@@ -284,7 +341,7 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
         }
         for (int i = 0; i < 2; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tfull0 + 8u * i) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(tempty0 + 8u * i) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(tempty0 + 8u * i) : "memory");
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *okp = 1u;
@@ -379,8 +436,21 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
                          : "memory");
         }
     } else if (warp >= 2) {
-        // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, the tile rows of that quarter
-        const uint32_t q = warp & 3u;
+        // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, the tile rows of that quarter, and one half of the columns
+        constexpr int HC = UN / 2;
+        const uint32_t q = warp & 3u, half = (warp - 2u) >> 2;
+        const int et = (int)threadIdx.x - 64;
+        float *bias = reinterpret_cast<float *>(base + S::BIAS_OFF), *w3 = reinterpret_cast<float *>(base + S::W3_OFF);
+        const EpiSmem es{bias, w3, s0 + S::OUT_OFF + (warp - 2u) * OUT_BYTES};
+        if (b.g[0].bias || b.g[0].w3) {   // one product
+            const UmmaArgs &g = b.g[0];
+            if (g.bias)
+                for (int i = et; i < g.N; i += EPI) bias[i] = g.bias[i];
+            if (g.w3)
+                for (int i = et; i < 2 * g.N; i += EPI)
+                    w3[i] = __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(g.w3)[i]);
+            asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
+        }
         uint32_t j = 0;
         for (int t = blockIdx.x; t < b.items; t += gridDim.x, ++j) {
             const Item<UN, TWO> it(b, t);
@@ -389,44 +459,57 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
             uint32_t ok = 1u;
             if (lane == 0) ok = mbar_wait(tfull0 + 8u * bf, (j >> 1) & 1u, okp) ? 1u : 0u;
             ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
-            if (g.colsum)   // the four warps meet at barriers below: they go on, or give up, together
-                asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %0, 0;\n bar.red.and.pred q, 1, 128, p;\n"
+            if (g.colsum || g.w3)   // the warps meet at barriers below: they go on, or give up, together
+                asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %0, 0;\n bar.red.and.pred q, 1, %1, p;\n"
                              " selp.u32 %0, 1, 0, q;\n}\n"
-                             : "+r"(ok)::"memory");
+                             : "+r"(ok)
+                             : "n"(EPI)
+                             : "memory");
             if (!ok) {
                 if (lane == 0) *okp = 0u;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int row = it.m0 + (int)(q * 32 + lane);
+            const int n0 = it.n0 + (int)half * HC;
             void *C = reinterpret_cast<uint8_t *>(g.C) + (size_t)it.split * g.c_split * (g.out_bf16 ? 2 : 4);
-            float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};   // the fused output layer
-            for (int c0 = 0; c0 < UN; c0 += 64) {   // two 32-column loads in flight per wait
-                uint32_t ra[32], rb[32];
-                const uint32_t ta = taddr + ((q * 32u) << 16) + bf * UN + (uint32_t)c0;
-                tmem_ld32(ta, ra);
-                tmem_ld32(ta + 32u, rb);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                float *cs = g.colsum ? csum + q * UN + c0 : nullptr;
-                emit32(g, C, row, it.n0 + c0, ra, a0, a1, cs, lane);
-                emit32(g, C, row, it.n0 + c0 + 32, rb, a0, a1, cs ? cs + 32 : nullptr, lane);
+            float2 a0[2] = {}, a1[2] = {};   // the fused output layer
+            uint32_t r[2][32];
+            const uint32_t ta = taddr + ((q * 32u) << 16) + bf * UN + half * HC;
+            tmem_ld32(ta, r[0]);
+#pragma unroll
+            for (int k = 0; k < HC / 32; ++k) {   // the next 32 columns load while these are worked on
+                tmem_wait(r[k & 1]);
+                if (k + 1 < HC / 32) {
+                    tmem_ld32(ta + 32u * (k + 1), r[(k + 1) & 1]);
+                } else {   // the accumulator may be overwritten from here on
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * bf) : "memory");
+                }
+                emit32(g, &b.tc[it.p], C, row, n0 + 32 * k, r[k & 1], es, a0, a1,
+                       g.colsum ? csum + q * UN + half * HC + 32 * k : nullptr, lane);
             }
-            // the accumulator may be overwritten from here on
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * bf) : "memory");
-            if (g.w3 && row < g.M)
-                reinterpret_cast<float2 *>(g.y)[(size_t)(it.n0 / UN) * g.M + row] =
-                    make_float2((a0[0] + a0[1]) + (a0[2] + a0[3]), (a1[0] + a1[1]) + (a1[2] + a1[3]));
-            if (g.colsum) {   // the four warps' sums, added by the 128 epilogue threads
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                for (int c = (int)threadIdx.x - 64; c < UN; c += 128)
+            if (g.w3) {   // the first half's warp adds the second's sums (two places: one barrier an item is enough)
+                float2 *hs = reinterpret_cast<float2 *>(base + S::HS_OFF) + bf * UM + q * 32 + lane;
+                const float2 sum = make_float2((a0[0].x + a0[0].y) + (a0[1].x + a0[1].y),
+                                               (a1[0].x + a1[0].y) + (a1[1].x + a1[1].y));
+                if (half) *hs = sum;
+                asm volatile("bar.sync %0, 64;" ::"r"(2u + q) : "memory");
+                if (!half && row < g.M)
+                    reinterpret_cast<float2 *>(g.y)[(size_t)(it.n0 / UN) * g.M + row] =
+                        make_float2(sum.x + hs->x, sum.y + hs->y);
+            }
+            if (g.colsum) {   // the four quarters' sums, added by the epilogue's threads
+                asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
+                for (int c = et; c < UN; c += EPI)
                     g.colsum[(size_t)(it.m0 / UM) * g.N + it.n0 + c] =
                         (csum[c] + csum[UN + c]) + (csum[2 * UN + c] + csum[3 * UN + c]);
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+                asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
             }
         }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     __syncwarp();
     __syncthreads();
@@ -447,6 +530,7 @@ bool umma_shape_ok(const UmmaArgs &a) {
            a.splits <= (a.K + UK - 1) / UK && a.ldc % (a.out_bf16 ? 8 : 4) == 0 && ((uintptr_t)a.A & 15) == 0 &&
            ((uintptr_t)a.B & 15) == 0 && ((uintptr_t)a.C & 15) == 0 && ((uintptr_t)a.bias & 15) == 0 &&
            (!a.mask || (a.ldc % 8 == 0 && ((uintptr_t)a.mask & 15) == 0)) &&
+           (!(a.bias || a.w3) || a.N <= HEAD_N) &&
            (!a.w3 || (a.y && ((uintptr_t)a.w3 & 15) == 0 && ((uintptr_t)a.y & 7) == 0));
 }
 
@@ -470,16 +554,18 @@ EncodeTiled encode_fn() {
 }
 
 // Tensor map of a row-major bf16 matrix [rows][ld] (cols used): 64-column x box_rows
-// boxes in the 128-byte swizzle, rows past the end read as zeros.
-bool make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows) {
+// boxes in the 128-byte swizzle, rows past the end read as zeros; or 32-column
+// boxes in the 64-byte one.
+bool make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows, int box_cols = UK) {
     EncodeTiled fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)UK, (cuuint32_t)box_rows};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE,
+              box_cols == UK ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -505,7 +591,8 @@ int launch(const UmmaArgs *a, int count, cudaStream_t s) {
         const bool ok = (a[p].a_mn ? make_map(&b.ta[p], a[p].A, a[p].K, a[p].M, a[p].lda, UK)
                                    : make_map(&b.ta[p], a[p].A, a[p].M, a[p].K, a[p].lda, UM)) &&
                         (a[p].b_mn ? make_map(&b.tb[p], a[p].B, a[p].K, a[p].N, a[p].ldb, UK)
-                                   : make_map(&b.tb[p], a[p].B, a[p].N, a[p].K, a[p].ldb, UN));
+                                   : make_map(&b.tb[p], a[p].B, a[p].N, a[p].K, a[p].ldb, UN)) &&
+                        (!a[p].store || !a[p].out_bf16 || make_map(&b.tc[p], a[p].C, a[p].M, a[p].N, a[p].ldc, 32, 32));
         if (!ok) return (int)cudaErrorInvalidValue;
     }
     b.items0 = (int)item_count(a[0], UN);
@@ -531,7 +618,7 @@ int umma_tile_n(const UmmaArgs *a, int count) {
 int umma_gemm(const UmmaArgs *a, int count, void *stream) {
     if (count < 1 || count > 2) return (int)cudaErrorInvalidValue;
     for (int p = 0; p < count; ++p) {
-        if (!umma_shape_ok(a[p])) return (int)cudaErrorInvalidValue;
+        if (!umma_shape_ok(a[p]) || (count > 1 && (a[p].bias || a[p].w3))) return (int)cudaErrorInvalidValue;
         if (a[p].M <= 0) return 0;
     }
     const int un = umma_tile_n(a, count);

@@ -51,6 +51,25 @@ def test_gradients_of_ragged_batches_on_tcgen05(env, B):
         assert abs(float(loss.item()) - ref_loss) <= 1e-3 * abs(ref_loss)
 
 
+# tiles of 64, 128 and 256 columns, their first and last sizes; a row tile that ends in its first or a later warp
+@pytest.mark.parametrize("B", [1, 31, 33, 129, 3584, 3585, 7168, 7169, 7267, 20001])
+def test_forward_of_every_tile_shape(env, B):
+    """Predictions within test_gpu_surrogate.py's bf16 bounds of the oracle, also for a batch's last rows alone."""
+    torch, H, sg = env
+    X, _ = _batch(B, 7)
+    p = sg.init_params(4)
+    s = sg.Surrogate(p)
+    Xd = torch.from_numpy(X).to("cuda").to(torch.bfloat16)
+    Y = s.predict(Xd).cpu().numpy()
+    H.hedl_mlp_status(s.mlp)
+    ref, _ = S.forward(sg.split_params(p), X, rounding=True)
+    scale = max(1.0, np.abs(ref).max())
+    assert np.abs(Y - ref).max() <= 2e-2 * scale
+    assert np.abs(Y - ref).mean() <= 2e-3 * max(1.0, np.abs(ref).mean())
+    few = s.predict(Xd[-64:].contiguous()).cpu().numpy()
+    assert np.abs(Y[-64:] - few).max() <= 2e-2 * scale
+
+
 # one cluster block's share of 8,192 keys and its neighbours; several tiles a block; all, one and half wanted
 @pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 1023, 8192, 65535, 65536, 65537, 200001])
 @pytest.mark.parametrize("kind", ["ties", "distinct", "equal", "wild"])
