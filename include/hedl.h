@@ -250,7 +250,8 @@ typedef struct {
     uint32_t n_segments;
     uint32_t n_slots;        /* materialized intermediate bitsets */
     uint32_t n_levels;
-    uint32_t n_items;        /* (segment, tile) work items */
+    uint32_t n_items;        /* (task, tile) pairs, a tile having tile_words words; the interpreter
+                                works on several segments at once and on narrower tiles of walks */
     uint32_t tile_words;
     uint32_t n_role_ops;     /* role restrictions evaluated (after sharing) */
     uint32_t n_role_groups;  /* shared CSR walks of bit-sliced role restrictions */
@@ -412,7 +413,7 @@ int hedl_autotune_workspace_size(hedl_kb *kb, const uint64_t *progs, const uint3
                                  size_t *bytes);
 
 /* Autotuner for the launch shape (warps per CTA, words per lane, rounds per
- * work item, chunks per role-walk step, filler staging).  No counterpart in
+ * work item, filler staging).  No counterpart in
  * the paper.  Each candidate shape plans the probe batch (HOST progs / offs as
  * in hedl_plan_batch, scored against the handle's examples), runs it once,
  * then times three replays with CUDA events on s; the fastest becomes the

@@ -455,8 +455,8 @@ struct ValueTest {
 // vals[rp[i] .. rp[i+1]) passes the test.  The warp's 32*WPL words are
 // 1024*WPL consecutive individuals, so their values form one contiguous run,
 // which the warp streams once, in windows of EX_WIN values that asynchronous
-// 16-byte copies bring into a ring of EX_STAGES windows in shared memory (32
-// warps an SM keep 64 KB in flight and hold no registers for it).  Lane l tests
+// 16-byte copies bring into one of two places in shared memory, the next
+// window while one is tested (no registers hold what is in flight).  Lane l tests
 // value 32u + l of a window, and a ballot packs 32 tests into a mask word in
 // the order of the values, which lane 0 puts into a ring of masks.  The row
 // pointers come the same way, a batch of four words (128 individuals) ahead.  A
@@ -475,7 +475,7 @@ struct ValueTest {
 // 138, and with a function a kind of test and the row batches in two register
 // sets warps waited 47 % of their time for instructions.  24 restrictions on 8
 // roles at 10^7 individuals (3.8 GB by the model, each role read three times):
-// 1.96 ms -> 1.26 ms.
+// 1.96 ms -> 1.26 ms, with rings half as large 1.10 ms.
 static_assert(EX_RING % EX_LOADS == 0 && EX_LOADS % 4 == 0, "a window's masks are whole 16-byte stores");
 
 // Asynchronous copy of src[at .. at + COUNT) to dst, the elements below end
@@ -601,12 +601,12 @@ __device__ __noinline__ RowWords<WPL> exist_run(const uint32_t *rp, const uint32
         }
         return commit();
     };
-    uint32_t slot = 0;   // window c's place of the ring; the next two follow
+    uint32_t slot = 0;   // window c's place of the two
     auto copy_window = [&](uint32_t at, uint32_t to) {
-        if (at < end) ex_copy<EX_WIN>(stages + (to >= EX_STAGES ? to - EX_STAGES : to) * EX_WIN, vals, at, end, vec, lane);
+        if (at < end) ex_copy<EX_WIN>(stages + to * EX_WIN, vals, at, end, vec, lane);
         return commit();
     };
-    static_assert(EX_STAGES == 3, "two windows in flight beside the one that is read");
+    static_assert(EX_STAGES == 2, "the window that is read and the next one");
     if (rvec) prefetch_range(rp, 32u * wb, i1 + 1u, lane);
     uint32_t half = 0, r = copy_rows(wb, 0u);                            // the next batch's group
     uint32_t v0 = copy_window(c, 0u), v1 = copy_window(c + EX_WIN, 1u);   // window c's and the next one's
@@ -638,8 +638,8 @@ __device__ __noinline__ RowWords<WPL> exist_run(const uint32_t *rp, const uint32
                 ex_wait(groups - 1u - v0);
                 ex_masks(stages + slot * EX_WIN, c, end, lane, test, ring + (c >> 5) % EX_RING);
                 __syncwarp();   // the window has been read, its masks are there
-                v0 = v1, v1 = copy_window(c + 2u * EX_WIN, slot + 2u);   // into the place of the window before c
-                slot = slot + 1u == EX_STAGES ? 0u : slot + 1u;
+                v0 = v1, v1 = copy_window(c + 2u * EX_WIN, slot);   // into the place of window c
+                slot ^= 1u;
                 c += EX_WIN;
             }
 #pragma unroll

@@ -1,16 +1,17 @@
 // Batched evaluation: one persistent interpreter kernel over a work queue of
 // (task, tile) items (see plan.cpp for how a batch becomes tasks).
 //
-// Each CTA pops an item, waits (bounded) until every task it reads is
-// complete, then its warps run the task over the tile.  A segment task is a
+// Each CTA pops an item (one task over a tile, or up to SEG_BATCH segments
+// over one), waits (bounded) until every task it reads is complete, then its
+// warps run it.  A segment task is a
 // stack machine whose values are bitset words (one register set per lane,
 // deeper stack entries in shared memory), whose leaves load concept rows /
 // slots, evaluate data ranges by ballot, or evaluate a lone role restriction
 // by the warp's edge-stream CSR walk (role_stream).  A segment's result is
 // written to its slot, or, for a hypothesis root, reduced against the example
 // sets by popcount (the paper's coverage count, Algorithm 15) with one atomic
-// per warp.  A role group (up to 64 restrictions sharing a role, direction
-// and role depth) runs as two tasks: a transpose of its fillers into one or
+// per warp.  A role group (up to 64 restrictions sharing a role and
+// direction) runs as two tasks: a transpose of its fillers into one or
 // two 32-bit words per individual, and one bit-sliced walk that evaluates all
 // of them.
 //

@@ -147,8 +147,7 @@ struct PlanHeader {
 struct Counters {
     uint32_t head;     // next work item
     uint32_t abort;    // set when a wait gave up
-    uint32_t err;
-    uint32_t pad;
+    uint32_t pad[2];
     // followed by done[n_segs] (tiles finished) and acc[n_hyps][2] (TP, FP)
 };
 
@@ -175,9 +174,13 @@ constexpr int PLAN_ONLY_SMS = 152;               // planning-only handles plan f
 constexpr int PF_SLOTS = 8;
 
 // A concrete-role walk's rings, per warp: mask words, two batches of row
-// pointers (128 and the one after them), EX_STAGES windows of values (4.4 KB,
-// so that 32 warps of a CTA fit beside their stacks).
-constexpr uint32_t EX_RING = 64, EX_ROWS = 132, EX_LOADS = 8, EX_WIN = 32 * EX_LOADS, EX_STAGES = 3;
+// pointers (128 and the one after them), EX_STAGES windows of values.  Kept
+// small (2.3 KB): what they leave of an SM's memory is the L1 cache of the
+// containment rows that string tests gather from (12.5 KB a pattern for 10^5
+// strings).  24 restrictions at 10^7 individuals, a third of them such tests:
+// three windows of 256 values (4.4 KB) 1,257 us, four of 128 1,206, three of
+// 128 1,143, two of 128 1,102.
+constexpr uint32_t EX_RING = 64, EX_ROWS = 132, EX_LOADS = 4, EX_WIN = 32 * EX_LOADS, EX_STAGES = 2;
 constexpr uint32_t EX_SMEM_WORDS = EX_RING + 2 * EX_ROWS + EX_STAGES * EX_WIN;
 
 // Segments a CTA prepares together (one work item), and the instructions of
