@@ -433,7 +433,9 @@ int execute(hedl_kb *kb, const PlanImpl *pc, uint32_t *counts, uint32_t *out_bit
         int le = launch_exec(kb, p, counts, out_bits, ws, st);
         return le ? cuda_fail(le, "exec launch") : HEDL_OK;
     }
-    if (!p->graph_exec || p->graph_ws != ws || p->graph_counts != counts || p->graph_out != out_bits) {
+    const KBView view = kb->view();
+    if (!p->graph_exec || p->graph_ws != ws || p->graph_counts != counts || p->graph_out != out_bits ||
+        memcmp(&p->graph_view, &view, sizeof view) != 0) {
         destroy_graph(p);
         // captured on the handle's own stream (the legacy default stream
         // cannot be captured), launched on the caller's
@@ -456,6 +458,7 @@ int execute(hedl_kb *kb, const PlanImpl *pc, uint32_t *counts, uint32_t *out_bit
         cudaGraphDestroy(g);
         if (e) return cuda_fail(e, "graph instantiate");
         p->graph_exec = ge;
+        p->graph_view = view;
         p->graph_ws = ws;
         p->graph_counts = counts;
         p->graph_out = out_bits;

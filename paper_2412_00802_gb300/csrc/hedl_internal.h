@@ -50,6 +50,7 @@ struct KBView {
     uint32_t *status;            // device status word owned by the handle
     uint32_t n, w, wp;           // individuals, valid words, row words
     uint32_t n_pos, n_neg;
+    uint32_t pad;                // views are compared byte for byte
 };
 
 // status word bits (device)
@@ -307,9 +308,12 @@ struct PlanImpl {
     std::vector<uint32_t> offs;
     uint32_t plain_depth = 0;
     // graph cache (a plan is captured at its second execution: a one-shot
-    // plan launches directly and pays no capture)
+    // plan launches directly and pays no capture).  The graph's kernels hold
+    // the KB's view by value, so it is good for an equal view only: new
+    // examples are captured anew.
     uint32_t runs = 0;
     void *graph_exec = nullptr;
+    KBView graph_view{};
     void *graph_ws = nullptr;
     uint32_t *graph_counts = nullptr;
     uint32_t *graph_out = nullptr;

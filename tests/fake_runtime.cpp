@@ -1,0 +1,170 @@
+// A stand-in for the CUDA runtime, linked with the library's own objects: it
+// launches nothing, keeps "device" memory on the host, and checks or records
+// what the library asks of it.  main runs one scenario, named by its argument.
+#include <cuda_runtime_api.h>
+
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <string>
+#include <utility>
+#include <vector>
+
+#include "hedl_internal.h"
+
+namespace {
+struct Launch {
+    const void *fn;
+    unsigned grid;
+    const uint32_t *pos;   // captured launches: the positive examples in the kernel's view of the KB
+};
+int device = 0;
+bool capturing = false;
+cudaError_t last = cudaSuccess;
+int instantiated = 0;
+std::vector<Launch> captured;
+
+cudaError_t launch(const void *fn, dim3 grid, void **args) {
+    // the interpreter's and the final kernel's first argument begins with the KBView
+    if (capturing) captured.push_back({fn, grid.x, static_cast<const hedl::KBView *>(args[0])->pos});
+    return cudaSuccess;
+}
+struct Config {
+    dim3 grid, block;
+    size_t smem;
+    void *stream;
+} config;
+}  // namespace
+
+extern "C" {
+cudaError_t cudaMalloc(void **p, size_t n) { return (*p = calloc(n ? n : 1, 1)) ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaFree(void *p) { free(p); return cudaSuccess; }
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) { memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemset(void *d, int v, size_t n) { memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaGetLastError() { return std::exchange(last, cudaSuccess); }
+const char *cudaGetErrorString(cudaError_t) { return "fake error"; }
+cudaError_t cudaGetDevice(int *d) { *d = device; return cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { device = d; return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
+    *v = a == cudaDevAttrMultiProcessorCount ? 152 : a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 232448 : 0;
+    return cudaSuccess;
+}
+cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int) { memset(p, 0, sizeof *p); return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = reinterpret_cast<cudaStream_t>(&device); return cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) {
+    capturing = true;
+    captured.clear();
+    return cudaSuccess;
+}
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) {
+    capturing = false;
+    *g = reinterpret_cast<cudaGraph_t>(&device);
+    return cudaSuccess;
+}
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t, unsigned long long) {
+    ++instantiated;
+    *e = reinterpret_cast<cudaGraphExec_t>(&device);
+    return cudaSuccess;
+}
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = nullptr; return cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 1.f; return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) { *n = 3; return cudaSuccess; }
+cudaError_t cudaGetSymbolAddress(void **p, const void *) { *p = nullptr; return cudaErrorInvalidSymbol; }
+static int encode_tiled(...) { return 0; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **fn, unsigned, unsigned long long, cudaDriverEntryPointQueryResult *r) {
+    *fn = reinterpret_cast<void *>(&encode_tiled);
+    if (r) *r = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, void **args) { return launch(fn, c->gridDim, args); }
+unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, CUstream_st *s) { config = {g, b, smem, s}; return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *smem, void *s) {
+    *g = config.grid, *b = config.block, *smem = config.smem;
+    *static_cast<void **>(s) = config.stream;
+    return cudaSuccess;
+}
+cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *fn) {
+    *k = reinterpret_cast<cudaKernel_t>(const_cast<void *>(fn));
+    return cudaSuccess;
+}
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void **args, size_t, cudaStream_t) {
+    return last = launch(k, grid, args);
+}
+void **__cudaRegisterFatBinary(void *) { return nullptr; }
+void __cudaRegisterFatBinaryEnd(void **) {}
+void __cudaUnregisterFatBinary(void **) {}
+void __cudaRegisterFunction(void **, const char *, char *, const char *, int, uint3 *, uint3 *, dim3 *, dim3 *, int *) {}
+void __cudaRegisterVar(void **, char *, char *, const char *, int, size_t, int, int) {}
+}
+
+#define REQUIRE(x)                                                                              \
+    do {                                                                                        \
+        if (!(x)) return printf("line %d: %s (%s)\n", __LINE__, #x, hedl_last_error()), 1;      \
+    } while (0)
+
+namespace {
+constexpr uint32_t N = 1000, WP = 32;
+struct alignas(256) Row { uint32_t w[WP]; };
+
+hedl_kb *load(const Row &concept_row) {
+    hedl_kb_desc d{};
+    d.n_indiv = N;
+    d.n_concepts = 1;
+    d.concept_bits = concept_row.w;
+    hedl_kb *kb = nullptr;
+    hedl_kb_load(&d, HEDL_KB_NO_VALIDATE, nullptr, &kb);
+    return kb;
+}
+
+// A captured graph holds the examples that it was captured with: after
+// hedl_examples_set the next scoring call has to capture anew.
+int examples_after_capture(bool one_shot) {
+    static Row bits, ex[4];
+    hedl_kb *kb = load(bits);
+    REQUIRE(kb);
+    REQUIRE(hedl_examples_set(kb, ex[0].w, ex[1].w, nullptr) == HEDL_OK);
+    const uint64_t prog = HEDL_OP_ATOM;
+    const uint32_t offs[2] = {0, 1};
+    hedl_plan *plan = nullptr;
+    REQUIRE(hedl_plan_batch(kb, &prog, offs, 1, 0, &plan) == HEDL_OK);
+    hedl_plan_info info;
+    REQUIRE(hedl_plan_info_get(plan, &info) == HEDL_OK);
+    void *ws = aligned_alloc(256, (info.workspace_bytes + 255) / 256 * 256);
+    alignas(16) static uint32_t counts[4];
+    auto score = [&]() {
+        return one_shot ? hedl_score_batch(kb, &prog, offs, 1, counts, ws, info.workspace_bytes, 0, nullptr)
+                        : hedl_plan_execute(kb, plan, counts, nullptr, ws, info.workspace_bytes, nullptr);
+    };
+    for (int k = 0; k < 3; ++k) REQUIRE(score() == HEDL_OK);
+    REQUIRE(instantiated == 1 && captured.size() == 2 && captured[0].pos == ex[0].w);
+    REQUIRE(hedl_examples_set(kb, ex[2].w, ex[3].w, nullptr) == HEDL_OK);
+    REQUIRE(score() == HEDL_OK);
+    REQUIRE(instantiated == 2 && captured[0].pos == ex[2].w && captured[1].pos == ex[2].w);
+    REQUIRE(score() == HEDL_OK && instantiated == 2);   // unchanged: the graph is launched again
+    if (!one_shot) REQUIRE(hedl_plan_replay(kb, plan, counts, nullptr, ws, info.workspace_bytes, nullptr) == HEDL_OK && instantiated == 2);
+    hedl_plan_free(plan);
+    hedl_kb_free(kb);
+    free(ws);
+    return 0;
+}
+}  // namespace
+
+int main(int argc, char **argv) {
+    const std::string s = argc > 1 ? argv[1] : "";
+    if (s == "examples_plan") return examples_after_capture(false);
+    if (s == "examples_one_shot") return examples_after_capture(true);
+    return 2;
+}
