@@ -2,6 +2,7 @@
 // C-ABI layer (api.cu) and the device kernels (exec.cu, plain.cu, kb.cu).
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <string>
@@ -277,10 +278,16 @@ struct UmmaArgs {
 };
 constexpr int UMMA_MAX_HEAD_TILES = 8;   // column tiles of a 512-wide layer at the narrowest tile
 bool umma_shape_ok(const UmmaArgs &a);
+// What the products need of the device they run on; kept by a handle of that device.
+struct UmmaDevice {
+    int sms = 0;
+    std::atomic<uint32_t> allowed{0};   // kernels that may use their shared memory (a bit each)
+};
+int umma_device(UmmaDevice *d);         // of the current device
 // Width of the column tiles that umma_gemm takes for these products.
-int umma_tile_n(const UmmaArgs *a, int count);
+int umma_tile_n(const UmmaArgs *a, int count, const UmmaDevice &dev);
 // One launch over one or two independent products.
-int umma_gemm(const UmmaArgs *a, int count, void *stream);
+int umma_gemm(const UmmaArgs *a, int count, UmmaDevice &dev, void *stream);
 
 int fail(int code, const std::string &msg);
 int cuda_fail(int cuda_err, const char *what);

@@ -34,4 +34,13 @@ cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size
     return cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 
+// Lets a kernel launch with `smem` bytes of dynamic shared memory, beyond the
+// 48 KB that need no leave.  The leave belongs to the kernel on the current
+// device and ends with its context: it may be remembered with what lives there
+// (a handle), not for the process, and a failure not at all.
+template <class... P>
+cudaError_t allow_smem(void (*kernel)(P...), size_t smem) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 }  // namespace hedl

@@ -996,6 +996,7 @@ struct hedl_mlp {
     // the target map (mean0, mean1, scale0, scale1, tail weight)
     float *w = nullptr, *m = nullptr, *v = nullptr, *g = nullptr, *map = nullptr;
     uint32_t *err = nullptr;                  // device: bit 0 = a tensor-core wait timed out
+    hedl::UmmaDevice dev;                     // the device that all of these live on
     unsigned gemm = HEDL_GEMM_TCGEN05;        // engine of the dense layers' forward GEMMs
     __nv_bfloat16 *wb = nullptr;
     size_t n = 0;
@@ -1072,14 +1073,14 @@ int forward_impl(hedl_mlp *mlp, const __nv_bfloat16 *X, uint32_t B, const MlpWs 
     int e;
     if (mlp->gemm == HEDL_GEMM_TCGEN05) {
         UmmaArgs u{X, mlp->wb + OFF_W1, w.h1, mlp->w + OFF_B1, (int)B, DH, DI, DI, DI, DH, 1, 1, mlp->err, nullptr};
-        e = umma_gemm(&u, 1, s);
+        e = umma_gemm(&u, 1, mlp->dev, s);
         if (e) return e;
         UmmaArgs v{w.h1, mlp->wb + OFF_W2, w.h2, mlp->w + OFF_B2, (int)B, DH, DH, DH, DH, DH, 1, 1, mlp->err, nullptr};
         v.w3 = mlp->wb + OFF_W3;
         v.y = w.y;
         v.store = need_h2;
-        *parts = DH / umma_tile_n(&v, 1);
-        return umma_gemm(&v, 1, s);
+        *parts = DH / umma_tile_n(&v, 1, mlp->dev);
+        return umma_gemm(&v, 1, mlp->dev, s);
     }
     e = dense_relu(X, mlp->wb + OFF_W1, mlp->w + OFF_B1, w.h1, (int)B, DI, s);
     if (!e) e = dense_relu(w.h1, mlp->wb + OFF_W2, mlp->w + OFF_B2, w.h2, (int)B, DH, s);
@@ -1115,13 +1116,13 @@ int grads_impl(hedl_mlp *mlp, const __nv_bfloat16 *X, const float *T, uint32_t B
         UmmaArgs d{w.dh2, mlp->wb + OFF_W2, w.dh1, nullptr, M, DH, DH, DH, DH, DH, 0, 1, mlp->err, w.h1};
         d.b_mn = 1;
         d.colsum = w.b1;
-        e = umma_gemm(&d, 1, s);
+        e = umma_gemm(&d, 1, mlp->dev, s);
         if (e) return e;
         // dW1 = dH1^T . X and dW2 = dH2^T . H1: contractions over the batch, both operands MN-major
         UmmaArgs g[2] = {{w.dh1, X, w.w1, nullptr, DH, DI, M, DH, DI, DI, 0, 0, mlp->err, nullptr},
                          {w.dh2, w.h1, w.w2, nullptr, DH, DH, M, DH, DH, DH, 0, 0, mlp->err, nullptr}};
         for (UmmaArgs &a : g) a.a_mn = a.b_mn = 1, a.splits = splits, a.c_split = (size_t)DH * DH;
-        return umma_gemm(g, 2, s);
+        return umma_gemm(g, 2, mlp->dev, s);
     }
     out->splits = 1;   // the atomics add every K range into the first part
     e = cudaMemsetAsync(w.w1, 0, (size_t)DH * DI * 4, s);
@@ -1165,7 +1166,8 @@ int hedl_mlp_create(const float *params, hedl_mlp **out) {
     *out = nullptr;
     auto *m = new hedl_mlp();
     m->n = N_PARAMS;
-    cudaError_t e = cudaMalloc(&m->w, N_PARAMS * 4);
+    cudaError_t e = (cudaError_t)umma_device(&m->dev);
+    if (!e) e = cudaMalloc(&m->w, N_PARAMS * 4);
     if (!e) e = cudaMalloc(&m->m, N_PARAMS * 4);
     if (!e) e = cudaMalloc(&m->v, N_PARAMS * 4);
     if (!e) e = cudaMalloc(&m->g, N_PARAMS * 4);
@@ -1361,11 +1363,10 @@ int hedl_select_top(const float *Y, uint32_t H, uint32_t k, uint32_t *idx, void 
     if (!Y || !idx) return fail(HEDL_ERR_INVALID_ARG, "NULL argument");
     if (k == 0 || k > H) return fail(HEDL_ERR_INVALID_ARG, "k must be in 1..H");
     if (!ws || ws_bytes < 8ull * H + 4096 + 256) return fail(HEDL_ERR_WORKSPACE_TOO_SMALL, "select workspace too small");
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SelSmem));
-    if (attr) return cuda_fail(attr, "select setup");
+    cudaError_t e = allow_smem(select_kernel, sizeof(SelSmem));
+    if (e) return cuda_fail(e, "select setup");
     select_kernel<<<SEL_CTAS, SEL_THREADS, sizeof(SelSmem), (cudaStream_t)s>>>(Y, H, k, idx);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     return e ? cuda_fail(e, "select launch") : HEDL_OK;
 }
 

@@ -569,22 +569,16 @@ bool make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int b
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int sm_count() {
-    static const int sms = [] {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) || n < 1 ? 1 : n;
-    }();
-    return sms;
-}
-
 long item_count(const UmmaArgs &a, int un) { return (long)((a.M + UM - 1) / UM) * (a.N / un) * a.splits; }
 
 template <int UN, bool TWO>
-int launch(const UmmaArgs *a, int count, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        umma_kernel<UN, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Shape<UN>::SMEM);
-    if (attr) return (int)attr;
+int launch(const UmmaArgs *a, int count, UmmaDevice &dev, cudaStream_t s) {
+    constexpr uint32_t bit = (UN == 256 ? 1u : UN == 128 ? 2u : 4u) << (TWO ? 3 : 0);
+    if (!(dev.allowed.load(std::memory_order_relaxed) & bit)) {
+        const cudaError_t e = allow_smem(umma_kernel<UN, TWO>, Shape<UN>::SMEM);
+        if (e) return (int)e;
+        dev.allowed.fetch_or(bit, std::memory_order_relaxed);
+    }
     Batch b{};
     for (int p = 0; p < count; ++p) {
         b.g[p] = a[p];
@@ -597,12 +591,18 @@ int launch(const UmmaArgs *a, int count, cudaStream_t s) {
     }
     b.items0 = (int)item_count(a[0], UN);
     b.items = b.items0 + (count > 1 ? (int)item_count(a[1], UN) : 0);
-    return (int)launch_pdl(umma_kernel<UN, TWO>, (unsigned)std::min(b.items, sm_count()), THREADS, Shape<UN>::SMEM, s, b);
+    return (int)launch_pdl(umma_kernel<UN, TWO>, (unsigned)std::min(b.items, dev.sms), THREADS, Shape<UN>::SMEM, s, b);
 }
 
 }  // namespace
 
-int umma_tile_n(const UmmaArgs *a, int count) {
+int umma_device(UmmaDevice *d) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return (int)(e ? e : cudaDeviceGetAttribute(&d->sms, cudaDevAttrMultiProcessorCount, dev));
+}
+
+int umma_tile_n(const UmmaArgs *a, int count, const UmmaDevice &dev) {
     for (int un : {256, 128}) {
         long items = 0;
         bool fits = true;
@@ -610,22 +610,26 @@ int umma_tile_n(const UmmaArgs *a, int count) {
             items += item_count(a[p], un);
             fits = fits && a[p].N % un == 0;
         }
-        if (fits && 4 * items >= 3l * sm_count()) return un;
+        if (fits && 4 * items >= 3l * dev.sms) return un;
     }
     return 64;
 }
 
-int umma_gemm(const UmmaArgs *a, int count, void *stream) {
+int umma_gemm(const UmmaArgs *a, int count, UmmaDevice &dev, void *stream) {
     if (count < 1 || count > 2) return (int)cudaErrorInvalidValue;
     for (int p = 0; p < count; ++p) {
         if (!umma_shape_ok(a[p]) || (count > 1 && (a[p].bias || a[p].w3))) return (int)cudaErrorInvalidValue;
         if (a[p].M <= 0) return 0;
     }
-    const int un = umma_tile_n(a, count);
+    const int un = umma_tile_n(a, count, dev);
     cudaStream_t s = (cudaStream_t)stream;
     if (count == 1)
-        return un == 256 ? launch<256, false>(a, 1, s) : un == 128 ? launch<128, false>(a, 1, s) : launch<64, false>(a, 1, s);
-    return un == 256 ? launch<256, true>(a, 2, s) : un == 128 ? launch<128, true>(a, 2, s) : launch<64, true>(a, 2, s);
+        return un == 256   ? launch<256, false>(a, 1, dev, s)
+               : un == 128 ? launch<128, false>(a, 1, dev, s)
+                           : launch<64, false>(a, 1, dev, s);
+    return un == 256   ? launch<256, true>(a, 2, dev, s)
+           : un == 128 ? launch<128, true>(a, 2, dev, s)
+                       : launch<64, true>(a, 2, dev, s);
 }
 
 }  // namespace hedl

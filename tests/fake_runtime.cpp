@@ -19,13 +19,19 @@ struct Launch {
     unsigned grid;
     const uint32_t *pos;   // captured launches: the positive examples in the kernel's view of the KB
 };
-int device = 0;
+int device = 0;                    // devices 0 and 1, with different numbers of SMs
+constexpr int SMS[] = {152, 16};
+std::map<std::pair<int, const void *>, size_t> opted;   // (device, kernel) -> shared memory it may use
+bool refuse_opt_in = false;        // the next opt-in fails
+unsigned last_grid = 0;
 bool capturing = false;
 cudaError_t last = cudaSuccess;
 int instantiated = 0;
 std::vector<Launch> captured;
 
-cudaError_t launch(const void *fn, dim3 grid, void **args) {
+cudaError_t launch(const void *fn, dim3 grid, size_t smem, void **args) {
+    if (smem > 49152 && smem > opted[{device, fn}]) return cudaErrorInvalidValue;
+    last_grid = grid.x;
     // the interpreter's and the final kernel's first argument begins with the KBView
     if (capturing) captured.push_back({fn, grid.x, static_cast<const hedl::KBView *>(args[0])->pos});
     return cudaSuccess;
@@ -49,8 +55,8 @@ const char *cudaGetErrorString(cudaError_t) { return "fake error"; }
 cudaError_t cudaGetDevice(int *d) { *d = device; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { device = d; return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
-cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
-    *v = a == cudaDevAttrMultiProcessorCount ? 152 : a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 232448 : 0;
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int d) {
+    *v = a == cudaDevAttrMultiProcessorCount ? SMS[d] : a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 232448 : 0;
     return cudaSuccess;
 }
 cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int) { memset(p, 0, sizeof *p); return cudaSuccess; }
@@ -80,7 +86,11 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 1.f; return cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute a, int v) {
+    if (std::exchange(refuse_opt_in, false)) return cudaErrorMemoryAllocation;
+    if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) opted[{device, fn}] = (size_t)v;
+    return cudaSuccess;
+}
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) { *n = 3; return cudaSuccess; }
 cudaError_t cudaGetSymbolAddress(void **p, const void *) { *p = nullptr; return cudaErrorInvalidSymbol; }
 static int encode_tiled(...) { return 0; }
@@ -89,7 +99,7 @@ cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **fn, unsigned, 
     if (r) *r = cudaDriverEntryPointSuccess;
     return cudaSuccess;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, void **args) { return launch(fn, c->gridDim, args); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, void **args) { return launch(fn, c->gridDim, c->dynamicSmemBytes, args); }
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, CUstream_st *s) { config = {g, b, smem, s}; return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *smem, void *s) {
     *g = config.grid, *b = config.block, *smem = config.smem;
@@ -100,8 +110,8 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *fn) {
     *k = reinterpret_cast<cudaKernel_t>(const_cast<void *>(fn));
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void **args, size_t, cudaStream_t) {
-    return last = launch(k, grid, args);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void **args, size_t smem, cudaStream_t) {
+    return last = launch(k, grid, smem, args);
 }
 void **__cudaRegisterFatBinary(void *) { return nullptr; }
 void __cudaRegisterFatBinaryEnd(void **) {}
@@ -160,11 +170,48 @@ int examples_after_capture(bool one_shot) {
     free(ws);
     return 0;
 }
+
+// The shared memory that a kernel needs is allowed on every device that it
+// launches on, and a failure is not kept; grids follow the current device.
+int second_device() {
+    for (int d : {0, 1, 0}) {
+        cudaSetDevice(d);
+        alignas(16) static float y[2 * 64];
+        static uint32_t idx[4];
+        static uint8_t ws[8192];
+        refuse_opt_in = true;
+        REQUIRE(hedl_select_top(y, 64, 4, idx, ws, sizeof ws, nullptr) == HEDL_ERR_CUDA);
+        REQUIRE(hedl_select_top(y, 64, 4, idx, ws, sizeof ws, nullptr) == HEDL_OK);
+        std::vector<float> params(hedl_mlp_param_count());
+        hedl_mlp *mlp = nullptr;
+        REQUIRE(hedl_mlp_create(params.data(), &mlp) == HEDL_OK);
+        for (uint32_t rows : {100u, 4096u, 20000u}) {   // tiles of 64, 128 and 256 columns on device 0
+            size_t bytes = 0;
+            REQUIRE(hedl_mlp_workspace_size(rows, &bytes) == HEDL_OK);
+            void *w = malloc(bytes), *x = aligned_alloc(16, 1024ull * rows), *t = malloc(8ull * rows);
+            refuse_opt_in = rows == 100u;
+            if (refuse_opt_in)
+                REQUIRE(hedl_mlp_forward(mlp, (uint16_t *)x, rows, (float *)t, w, bytes, nullptr) == HEDL_ERR_CUDA);
+            REQUIRE(hedl_mlp_forward(mlp, (uint16_t *)x, rows, (float *)t, w, bytes, nullptr) == HEDL_OK);
+            REQUIRE(hedl_mlp_gradients(mlp, (uint16_t *)x, (float *)t, rows, nullptr, w, bytes, nullptr) == HEDL_OK);
+            free(w), free(x), free(t);
+        }
+        hedl::UmmaDevice dev;
+        hedl::UmmaArgs a{};   // a product of many tiles: one block an SM
+        alignas(16) static uint8_t operand[16];
+        a.A = a.B = a.C = operand;
+        a.M = 1 << 16, a.N = a.K = a.lda = a.ldb = a.ldc = 512, a.out_bf16 = 1;
+        REQUIRE(hedl::umma_device(&dev) == 0 && hedl::umma_gemm(&a, 1, dev, nullptr) == 0 && last_grid == (unsigned)SMS[d]);
+        hedl_mlp_free(mlp);
+    }
+    return 0;
+}
 }  // namespace
 
 int main(int argc, char **argv) {
     const std::string s = argc > 1 ? argv[1] : "";
     if (s == "examples_plan") return examples_after_capture(false);
     if (s == "examples_one_shot") return examples_after_capture(true);
+    if (s == "second_device") return second_device();
     return 2;
 }
