@@ -271,7 +271,7 @@ struct UmmaArgs {
     float *y = nullptr;
     int store = 1;
     int a_mn = 0, b_mn = 0;
-    // K in `splits` equal ranges (whole blocks of 64), range s into C + s * c_split elements
+    // K in `splits` equal ranges (whole blocks of 64), range s into C + s * c_split floats (FP32 outputs alone)
     int splits = 1;
     size_t c_split = 0;
     float *colsum = nullptr;   // or float [ceil(M/128)][N]: column sums of the bf16 outputs of each 128-row tile

@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(THREADS, 1) umma_kernel(const __grid_constant_
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int row = it.m0 + (int)(q * 32 + lane);
             const int n0 = it.n0 + (int)half * HC;
-            void *C = reinterpret_cast<uint8_t *>(g.C) + (size_t)it.split * g.c_split * (g.out_bf16 ? 2 : 4);
+            void *C = reinterpret_cast<float *>(g.C) + (size_t)it.split * g.c_split;   // FP32 outputs
             float2 a0[2] = {}, a1[2] = {};   // the fused output layer
             uint32_t r[2][32];
             const uint32_t ta = taddr + ((q * 32u) << 16) + bf * UN + half * HC;
@@ -527,7 +527,13 @@ bool umma_shape_ok(const UmmaArgs &a) {
     // has 64-row boxes along M or N and any K (rows past it read as zeros)
     return a.N % 64 == 0 && a.N > 0 && a.K > 0 && (a.a_mn ? a.M % 64 == 0 : a.K % UK == 0) &&
            (a.b_mn || a.K % UK == 0) && a.lda % 8 == 0 && a.ldb % 8 == 0 && a.splits >= 1 &&
-           a.splits <= (a.K + UK - 1) / UK && a.ldc % (a.out_bf16 ? 8 : 4) == 0 && ((uintptr_t)a.A & 15) == 0 &&
+           a.splits <= (a.K + UK - 1) / UK &&
+           // a K range has a place of its own in FP32 outputs only: bf16 ones leave through one
+           // tensor map, and column sums and the output layer's have one place a tile; bias, ReLU
+           // and mask would apply to every range
+           (a.splits == 1 ||
+            (!a.out_bf16 && !a.colsum && !a.w3 && !a.bias && !a.relu && !a.mask && a.c_split % 4 == 0)) &&
+           a.ldc % (a.out_bf16 ? 8 : 4) == 0 && ((uintptr_t)a.A & 15) == 0 &&
            ((uintptr_t)a.B & 15) == 0 && ((uintptr_t)a.C & 15) == 0 && ((uintptr_t)a.bias & 15) == 0 &&
            (!a.mask || (a.ldc % 8 == 0 && ((uintptr_t)a.mask & 15) == 0)) &&
            (!(a.bias || a.w3) || a.N <= HEAD_N) &&

@@ -206,6 +206,31 @@ int second_device() {
     }
     return 0;
 }
+
+// Products split over K have a place for each range in plain FP32 outputs only.
+int split_products() {
+    alignas(16) static uint8_t operand[16];
+    hedl::UmmaArgs a{};
+    a.A = a.B = a.C = operand;
+    a.M = a.N = a.K = a.lda = a.ldb = a.ldc = 512, a.splits = 4, a.c_split = 512 * 512;
+    REQUIRE(hedl::umma_shape_ok(a));
+    auto refused = [&](auto change) {
+        hedl::UmmaArgs b = a;
+        change(b);
+        const bool split = hedl::umma_shape_ok(b);
+        b.splits = 1;
+        return !split && hedl::umma_shape_ok(b);
+    };
+    auto *f = reinterpret_cast<float *>(operand);
+    REQUIRE(refused([&](hedl::UmmaArgs &b) { b.out_bf16 = 1; }));
+    REQUIRE(refused([&](hedl::UmmaArgs &b) { b.colsum = f; }));
+    REQUIRE(refused([&](hedl::UmmaArgs &b) { b.w3 = operand, b.y = f; }));
+    REQUIRE(refused([&](hedl::UmmaArgs &b) { b.bias = f; }));
+    REQUIRE(refused([&](hedl::UmmaArgs &b) { b.relu = 1; }));
+    REQUIRE(refused([&](hedl::UmmaArgs &b) { b.mask = operand; }));
+    REQUIRE(refused([&](hedl::UmmaArgs &b) { b.c_split = 6; }));
+    return 0;
+}
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -213,5 +238,6 @@ int main(int argc, char **argv) {
     if (s == "examples_plan") return examples_after_capture(false);
     if (s == "examples_one_shot") return examples_after_capture(true);
     if (s == "second_device") return second_device();
+    if (s == "split_products") return split_products();
     return 2;
 }
