@@ -859,7 +859,8 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
         k = k2;
     }
     for (uint32_t l = 1; l <= n_levels; ++l) level_items[l] = std::max(level_items[l], level_items[l - 1]);
-    if (items >= 0xFFFFFFFFull) {
+    // the (task, tile) pairs that the plan reports, and the items made of them
+    if (items >= 0xFFFFFFFFull || (uint64_t)NS * n_tiles >= 0xFFFFFFFFull) {
         delete p;
         return fail(HEDL_ERR_INVALID_ARG, "batch too large: more than 2^32 work items");
     }

@@ -535,3 +535,17 @@ def test_plan_byte_model_equals_the_oracles_count(n):
         assert H.hedl_plan_info_get(par)["model_bytes"] == want
         for f in (0, H.HEDL_NO_SLICE, H.HEDL_SLICE_ALL):
             assert H.hedl_plan_info_get(H.hedl_plan_batch(hk, flat, offs, f))["model_bytes"] <= want, (it, f)
+
+
+def test_batches_past_the_item_limit_are_refused():
+    """A plan reports its (task, tile) pairs in 32 bits: a batch of more is refused, whatever the work items that the
+    interpreter makes of them (131,072 tiles a segment here, eight segments an item)."""
+    hk = H.hedl_kb_plan_only(0x7FFFFF00, 4, [100], 0)
+    progs = [P.compile_text("(some r0 A1)"), P.compile_text("(all r0 A2)")] + [P.compile_text("(and A0 A1)")] * 33_000
+    few = H.hedl_plan_info_get(H.hedl_plan_batch(hk, *P.pack_batch(progs[:32_000])))
+    assert few["n_role_groups"] == 1
+    assert few["n_items"] == few["n_segments"] * -(-H.hedl_row_words(0x7FFFFF00) // few["tile_words"])
+    assert few["n_segments"] * 131_072 < 2 ** 32 <= (few["n_segments"] + len(progs) - 32_000) * 131_072
+    with pytest.raises(H.HedlError) as e:
+        H.hedl_plan_batch(hk, *P.pack_batch(progs))
+    assert e.value.code == -1 and "work items" in str(e.value)
