@@ -29,6 +29,7 @@
 //      level that walks a role holds too few tasks to fill the GPU.
 #include <algorithm>
 #include <cstring>
+#include <utility>
 
 #include "hedl_internal.h"
 
@@ -193,75 +194,138 @@ uint64_t put(std::vector<uint8_t> &img, const std::vector<T> &v) {
 }
 
 // The stage (1, 2, ...) at which each bit-sliceable role restriction walks;
-// 0 for every other node.  A restriction may walk once those nested in its
-// filler have (a stage later than all of them), and has to by the stage that
-// leaves one stage for each restriction around it, in a plan of as many stages
-// as the deepest nesting.  At each stage a role and direction walks if one of
-// its ready restrictions cannot wait; then all its ready ones walk with it.
-// Otherwise only whole groups of SLICES * MAX_PARTS walk (waiting could not
-// save their walk), the ones with the least time left first.  A role and
-// direction of one or two restrictions does not wait: two lone walks over
+// 0 for every other node, and for all of them if none could share a walk (and
+// all is false: lone ones are not sliced then).  A restriction may walk once
+// those nested in its filler have (a stage later than all of them), and has to
+// by the stage that leaves one stage for each restriction around it, in a plan
+// of as many stages as the deepest nesting.  At each stage a role and direction
+// walks if one of its ready restrictions cannot wait; then all its ready ones
+// walk with it.  Otherwise only whole groups of SLICES * MAX_PARTS walk (waiting
+// could not save their walk), the ones with the least time left first.  A role
+// and direction of one or two restrictions does not wait: two lone walks over
 // bitset fillers cost about as much as a shared one with its transpose.
 // Walking every restriction as soon as it is ready (one group per role,
 // direction and nesting depth) took 261 walks for 2,048 refinements over 64
 // roles and directions and 244 for a batch of 4,096 over 32; this takes 134
 // and 186 (2,048 refinements at 4 * 10^6 individuals 57.3 -> 35.4 ms).
 // key_of numbers the (stage, role, direction) triples 0, 1, ... by stage; key_size counts their restrictions.
-void walk_stages(const std::vector<PNode> &nodes, uint32_t n_roles, std::vector<uint32_t> &stage,
+//
+// Each node is finished once, when its last operand is, and each role and
+// direction is looked at only at the stages where a restriction of it becomes
+// ready or due: the time grows with the batch, not with its depth or the KB's roles.
+void walk_stages(const std::vector<PNode> &nodes, uint32_t n_roles, bool all, std::vector<uint32_t> &stage,
                  std::vector<uint32_t> &key_of, std::vector<uint32_t> &key_size) {
-    const uint32_t NN = (uint32_t)nodes.size(), NEVER = 0xFFFFFFFFu;
+    const uint32_t NN = (uint32_t)nodes.size(), WHOLE = SLICES * MAX_PARTS;
     auto eligible = [&](const PNode &n) {
         return is_role(n.op) && (n.op == HEDL_OP_EXISTS || n.op == HEDL_OP_FORALL || n.b <= SLICE_MAX_N);
     };
-    std::vector<uint32_t> done(NN, 0);      // the stage that completes the restrictions in a node's expression
-    std::vector<uint32_t> inner;            // nodes with a restriction in their expression, children first
+    // nesting depths; the nodes with a restriction in their expression, children first
+    std::vector<uint32_t> depth(NN, 0), inner, sliceable;
     uint32_t last = 0;
     for (uint32_t i = 0; i < NN; ++i) {
         const PNode &n = nodes[i];
-        const uint32_t d = std::max(n.k0 >= 0 ? done[n.k0] : 0u, n.k1 >= 0 ? done[n.k1] : 0u);
-        done[i] = d + (is_role(n.op) ? 1u : 0u);
-        if (done[i]) inner.push_back(i);
-        last = std::max(last, done[i]);
+        const uint32_t d = std::max(n.k0 >= 0 ? depth[n.k0] : 0u, n.k1 >= 0 ? depth[n.k1] : 0u);
+        depth[i] = d + (is_role(n.op) ? 1u : 0u);
+        if (depth[i]) inner.push_back(i);
+        if (eligible(n)) sliceable.push_back(i);
+        last = std::max(last, depth[i]);
     }
-    std::vector<uint32_t> limit(NN, last);
+    // the roles and directions that have sliceable restrictions, in a dense
+    // numbering: by a table of the KB's, unless the batch has far fewer restrictions
+    std::vector<uint32_t> role(NN, 0), total;
+    {
+        std::vector<uint32_t> ids;
+        if (2ull * n_roles <= 4ull * sliceable.size() + 64) {
+            ids.assign(2 * (size_t)n_roles, 0);
+            for (uint32_t i : sliceable) ids[2 * nodes[i].a + nodes[i].inv] = 1;
+            uint32_t k = 0;
+            for (uint32_t &id : ids) k += std::exchange(id, k);
+            total.assign(k, 0);
+            for (uint32_t i : sliceable) total[role[i] = ids[2 * nodes[i].a + nodes[i].inv]]++;
+        } else {
+            for (uint32_t i : sliceable) ids.push_back(2 * nodes[i].a + nodes[i].inv);
+            std::sort(ids.begin(), ids.end());
+            ids.erase(std::unique(ids.begin(), ids.end()), ids.end());
+            total.assign(ids.size(), 0);
+            for (uint32_t i : sliceable)
+                total[role[i] = (uint32_t)(std::lower_bound(ids.begin(), ids.end(), 2 * nodes[i].a + nodes[i].inv) - ids.begin())]++;
+        }
+    }
+    if (!all && std::none_of(total.begin(), total.end(), [](uint32_t n) { return n > 1; })) return;
+    // the stage by which a node has to be complete; how many of its operands still wait
+    std::vector<uint32_t> limit(NN, last), waits(NN, 0);
     for (auto it = inner.rbegin(); it != inner.rend(); ++it) {
         const PNode &n = nodes[*it];
         const uint32_t l = limit[*it] - (is_role(n.op) ? 1u : 0u);
         if (n.k0 >= 0) limit[n.k0] = std::min(limit[n.k0], l);
         if (n.k1 >= 0) limit[n.k1] = std::min(limit[n.k1], l);
     }
-    std::vector<std::vector<uint32_t>> ready(2 * (size_t)n_roles);
-    std::vector<uint32_t> total(2 * (size_t)n_roles, 0);
+    // the nodes that read node i: users[first[i] .. first[i + 1])
+    std::vector<uint32_t> first(NN + 1, 0), users;
     for (uint32_t i : inner)
-        if (eligible(nodes[i])) total[2 * nodes[i].a + nodes[i].inv]++;
-    std::vector<uint32_t> open(inner);   // nodes that a restriction still keeps waiting, children first
-    for (uint32_t s = 1; s <= last; ++s) {
-        size_t kept = 0;
-        for (uint32_t i : open) {
-            const PNode &n = nodes[i];
-            uint32_t d = std::max(n.k0 >= 0 ? done[n.k0] : 0u, n.k1 >= 0 ? done[n.k1] : 0u);
-            if (stage[i]) d = stage[i];
-            else if (eligible(n)) {
-                if (d < s) ready[2 * n.a + n.inv].push_back(i);   // d is NEVER while something nested waits
-                d = NEVER;
-            } else if (is_role(n.op) && d != NEVER) ++d;
-            done[i] = d;
-            if (d == NEVER) open[kept++] = i;
-        }
-        open.resize(kept);
-        for (size_t key = 0; key < ready.size(); ++key) {
-            std::vector<uint32_t> &r = ready[key];
-            bool urgent = total[key] < 3;
-            for (uint32_t i : r) urgent = urgent || limit[i] <= s;
-            if (!urgent) {
-                std::stable_sort(r.begin(), r.end(), [&](uint32_t x, uint32_t y) { return limit[x] < limit[y]; });
-                r.resize(r.size() / (SLICES * MAX_PARTS) * (SLICES * MAX_PARTS));
+        for (int32_t k : {nodes[i].k0, nodes[i].k1})
+            if (k >= 0 && depth[k]) first[k + 1]++, waits[i]++;
+    for (uint32_t i = 0; i < NN; ++i) first[i + 1] += first[i];
+    users.resize(first[NN]);
+    {
+        std::vector<uint32_t> at(first.begin(), first.end() - 1);
+        for (uint32_t i : inner)
+            for (int32_t k : {nodes[i].k0, nodes[i].k1})
+                if (k >= 0 && depth[k]) users[at[k]++] = i;
+    }
+    std::vector<uint32_t> done(NN, 0);   // the stage that completes a node, once it is known
+    // stage s: the restrictions that become ready, and the roles and directions of which one is due
+    std::vector<std::vector<uint32_t>> ready(last + 2), due(last + 1);
+    std::vector<uint32_t> stack;
+    // node i's operands are complete by stage d
+    auto operands_done = [&](uint32_t i, uint32_t d) {
+        if (eligible(nodes[i])) ready[d + 1].push_back(i);
+        else done[i] = d + (is_role(nodes[i].op) ? 1u : 0u), stack.push_back(i);
+    };
+    auto spread = [&]() {
+        while (!stack.empty()) {
+            const uint32_t i = stack.back();
+            stack.pop_back();
+            for (uint32_t q = first[i]; q < first[i + 1]; ++q) {
+                const uint32_t u = users[q];
+                const PNode &n = nodes[u];
+                if (--waits[u] == 0) operands_done(u, std::max(n.k0 >= 0 ? done[n.k0] : 0u, n.k1 >= 0 ? done[n.k1] : 0u));
             }
-            if (r.empty()) continue;
-            for (uint32_t i : r) stage[i] = s, key_of[i] = (uint32_t)key_size.size();
-            key_size.push_back((uint32_t)r.size());
-            r.clear();
         }
+    };
+    for (uint32_t i : inner)
+        if (depth[i] == 1 && waits[i] == 0) operands_done(i, 0);
+    spread();
+    std::vector<std::vector<uint32_t>> pending(total.size());   // ready restrictions that wait
+    std::vector<uint32_t> looked;
+    for (uint32_t s = 1; s <= last; ++s) {
+        looked.swap(due[s]);
+        for (uint32_t i : ready[s]) {
+            std::vector<uint32_t> &p = pending[role[i]];
+            if (total[role[i]] < 3 || limit[i] <= s || p.size() + 1 >= WHOLE) looked.push_back(role[i]);
+            p.push_back(i);
+            if (limit[i] > s) due[limit[i]].push_back(role[i]);
+        }
+        std::sort(looked.begin(), looked.end());
+        looked.erase(std::unique(looked.begin(), looked.end()), looked.end());
+        for (uint32_t k : looked) {
+            std::vector<uint32_t> &p = pending[k];
+            size_t n = p.size();   // how many walk now
+            if (total[k] >= 3 && std::none_of(p.begin(), p.end(), [&](uint32_t i) { return limit[i] <= s; })) {
+                n = n / WHOLE * WHOLE;
+                if (n) std::sort(p.begin(), p.end(), [&](uint32_t x, uint32_t y) { return limit[x] != limit[y] ? limit[x] < limit[y] : x < y; });
+            }
+            if (n == 0) continue;
+            for (size_t q = 0; q < n; ++q) {
+                const uint32_t i = p[q];
+                done[i] = stage[i] = s, key_of[i] = (uint32_t)key_size.size();
+                stack.push_back(i);
+            }
+            key_size.push_back((uint32_t)n);
+            p.erase(p.begin(), p.begin() + (ptrdiff_t)n);
+        }
+        looked.clear();
+        spread();
     }
 }
 
@@ -390,7 +454,7 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     std::vector<uint8_t> sl(NN, 0);
     std::vector<uint32_t> stage(NN, 0), key_of(NN, 0), key_size;
     if (sliced) {
-        walk_stages(nodes, kb->n_roles, stage, key_of, key_size);
+        walk_stages(nodes, kb->n_roles, (flags & HEDL_SLICE_ALL) != 0, stage, key_of, key_size);
         for (uint32_t i = 0; i < NN; ++i)
             if (stage[i] && ((flags & HEDL_SLICE_ALL) || key_size[key_of[i]] >= 2)) sl[i] = mat[i] = 1;
     }
