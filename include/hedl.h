@@ -397,7 +397,7 @@ typedef struct {
     uint32_t stage_fillers;    /* 1: copy a role restriction's filler row into shared memory once per
                                   work item when it fits (then a segment reads at most one role
                                   restriction); 0: gather filler bits from global memory */
-    uint32_t role_block;       /* 4 or 8: kept for callers that set it; the role walk's windows have one size */
+    uint32_t role_block;       /* 4 or 8: 32-edge chunks a lone role walk loads per step */
     uint32_t full_occupancy;   /* 1: with 8 warps, 1 word per lane and no staging, use the build
                                   limited to 32 registers so 8 CTAs fit per SM */
 } hedl_tuning;
@@ -413,7 +413,7 @@ int hedl_autotune_workspace_size(hedl_kb *kb, const uint64_t *progs, const uint3
                                  size_t *bytes);
 
 /* Autotuner for the launch shape (warps per CTA, words per lane, rounds per
- * work item, filler staging).  No counterpart in
+ * work item, chunks per role-walk step, filler staging).  No counterpart in
  * the paper.  Each candidate shape plans the probe batch (HOST progs / offs as
  * in hedl_plan_batch, scored against the handle's examples), runs it once,
  * then times three replays with CUDA events on s; the fastest becomes the

@@ -249,17 +249,27 @@ __device__ __forceinline__ void role_words(const DevCSR g, const uint32_t *fille
 // A word whose every lane is decided (cap reached or row ended) makes the
 // stream jump to the next word's first edge.  Word k of the warp goes to lane
 // k / WPL, slot k % WPL.  n_words bounds the warp's words; lanes of
-// individuals >= n hold empty rows and emit 0.  A function of its own, with
-// registers of its own: inlined, the stack machine around it spilled.
+// individuals >= n hold empty rows and emit 0.  SMEM: the filler row is staged
+// in shared memory.  A function of its own, with registers of its own: inlined,
+// the stack machine around it spilled.
+//
+// Bound: latency and the filler's gathers.  Which block is faster depends on
+// the rows, which the plan does not know: on heavy-tailed ones a block of 8
+// chunks keeps more in flight (a lone hypothesis on 10^7 individuals, Zipf
+// degrees of mean 8: 1,416 us with 4, 1,369 with 8; on 10^6: 265 and 218), on
+// even ones its emptier blocks cost more (Poisson degrees of mean 4, 10^6
+// individuals: 127 and 134).  So it is part of the launch shape (role_block),
+// 4 unless the tuner has timed it.
 template <int WPL>
 struct RowWords {
     uint32_t v[WPL];
 };
-template <int WPL>
+template <int WPL, uint32_t BLK, bool SMEM>
 __device__ __noinline__ RowWords<WPL> role_stream(const uint32_t *rp, const uint32_t *col, const uint32_t *filler,
                                                   uint32_t kind, uint32_t n_arg, uint32_t n, uint32_t n_words,
                                                   uint32_t wb, bool filler_inverted) {
-    constexpr uint32_t BLK = 4, BE = 32u * BLK;     // chunks and edges per block
+    if constexpr (BLK == 8u && !SMEM) __builtin_assume(__isGlobal(filler));   // loads of blocks of 4 got 1 % slower
+    constexpr uint32_t BE = 32u * BLK;              // edges per block
     const uint32_t lane = threadIdx.x & 31u;
     RowWords<WPL> out;
     uint32_t (&v)[WPL] = out.v;

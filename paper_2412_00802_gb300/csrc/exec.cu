@@ -162,7 +162,7 @@ __device__ bool prepare_task(const ExecArgs &A, const PlanHeader &hd, Smem<NW, W
     return __all_sync(FULL, ok);
 }
 
-template <int NW, int WPL, bool STAGE, bool CONCRETE>
+template <int NW, int WPL, bool STAGE, int BLK, bool CONCRETE>
 __device__ void run_tile(const ExecArgs &A, const PlanHeader &hd, uint32_t b, uint32_t tile, Smem<NW, WPL> &sm,
                          uint32_t *slots, uint32_t *acc) {
     const KBView &kb = A.kb;
@@ -284,7 +284,7 @@ __device__ void run_tile(const ExecArgs &A, const PlanHeader &hd, uint32_t b, ui
                 const uint32_t *filler = STAGE ? sm.tail + A.ring_words
                                          : (d.ref & REF_SLOT) ? slots + (uint64_t)(d.ref & ~REF_SLOT) * kb.wp
                                                               : kb.concepts + (uint64_t)d.ref * kb.wp;
-                const RowWords<WPL> o = role_stream<WPL>(g.rp, g.col, filler, kind, d.b, kb.n, lim_w, wb,
+                const RowWords<WPL> o = role_stream<WPL, BLK, STAGE>(g.rp, g.col, filler, kind, d.b, kb.n, lim_w, wb,
                                                          STAGE && kind == HEDL_OP_FORALL);
 #pragma unroll
                 for (int s = 0; s < WPL; ++s) top[s] = o.v[s];
@@ -670,7 +670,7 @@ __device__ __forceinline__ void stage_filler(const KBView &kb, const uint32_t *s
 // CONCRETE = false leaves the concrete-role value walk out, for KBs that have
 // no concrete roles: its registers would otherwise raise the spills of the
 // whole stack machine.
-template <int NW, int WPL, bool STAGE, bool FULL = false, bool GROUPS = true, bool CONCRETE = true>
+template <int NW, int WPL, bool STAGE, int BLK, bool FULL = false, bool GROUPS = true, bool CONCRETE = true>
 __global__ void __launch_bounds__(NW * 32, (FULL ? 64 : (GROUPS ? 24 : 32)) / NW) exec_kernel(ExecArgs A) {
     // the host sizes the dynamic shared memory (smem_bytes)
     using SmemT = Smem<NW, WPL>;
@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(NW * 32, (FULL ? 64 : (GROUPS ? 24 : 32)) / NW
             }
 #pragma unroll 1
             for (uint32_t b = 0; b < n_tasks; ++b)
-                run_tile<NW, WPL, STAGE, CONCRETE>(A, hd, b, tile, sm, slots, acc);
+                run_tile<NW, WPL, STAGE, BLK, CONCRETE>(A, hd, b, tile, sm, slots, acc);
         }
         __syncthreads();
         if (A.use_queue) {
@@ -805,33 +805,39 @@ __global__ void upload_kernel(const __grid_constant__ SmallImage img, uint4 *ws,
 
 using KernelFn = void (*)(ExecArgs);
 
-// Instantiated launch shapes: warps x words per lane x staging (1- and 2-warp
-// CTAs only with one word per lane and no staging).  The tuning's role_block
-// shapes no code any more (the lone walk's block of 4 chunks was never slower).
-template <bool STAGE>
+// Instantiated launch shapes: warps x words per lane x staging x chunks per
+// block of the lone walk (1- and 2-warp CTAs only with one word per lane and no
+// staging).
+template <bool STAGE, int BLK>
 KernelFn pick_t(uint32_t warps, uint32_t wpl) {
     if (wpl == 4) {
-        if (warps == 4) return exec_kernel<4, 4, STAGE>;
-        if (warps == 16) return exec_kernel<16, 4, STAGE>;
-        return exec_kernel<8, 4, STAGE>;
+        if (warps == 4) return exec_kernel<4, 4, STAGE, BLK>;
+        if (warps == 16) return exec_kernel<16, 4, STAGE, BLK>;
+        return exec_kernel<8, 4, STAGE, BLK>;
     }
     if constexpr (!STAGE) {
-        if (warps == 1) return exec_kernel<1, 1, false>;
-        if (warps == 2) return exec_kernel<2, 1, false>;
+        if (warps == 1) return exec_kernel<1, 1, false, BLK>;
+        if (warps == 2) return exec_kernel<2, 1, false, BLK>;
     }
-    if (warps == 4) return exec_kernel<4, 1, STAGE>;
-    if (warps == 16) return exec_kernel<16, 1, STAGE>;
-    if (warps == 32) return exec_kernel<32, 1, STAGE>;
-    return exec_kernel<8, 1, STAGE>;
+    if (warps == 4) return exec_kernel<4, 1, STAGE, BLK>;
+    if (warps == 16) return exec_kernel<16, 1, STAGE, BLK>;
+    if (warps == 32) return exec_kernel<32, 1, STAGE, BLK>;
+    return exec_kernel<8, 1, STAGE, BLK>;
+}
+
+template <int BLK>
+KernelFn pick_b(const Tuning &t, bool stage, bool groups, bool concrete) {
+    if (t.warps == 8 && t.wpl == 1 && !stage) {   // the common shapes
+        if (t.full_occupancy) return exec_kernel<8, 1, false, BLK, true>;
+        if (!groups)
+            return concrete ? exec_kernel<8, 1, false, BLK, false, false> : exec_kernel<8, 1, false, BLK, false, false, false>;
+        if (!concrete) return exec_kernel<8, 1, false, BLK, false, true, false>;
+    }
+    return stage ? pick_t<true, BLK>(t.warps, t.wpl) : pick_t<false, BLK>(t.warps, t.wpl);
 }
 
 KernelFn pick(const Tuning &t, bool stage, bool groups, bool concrete) {
-    if (t.warps == 8 && t.wpl == 1 && !stage) {   // the common shapes
-        if (t.full_occupancy) return exec_kernel<8, 1, false, true>;
-        if (!groups) return concrete ? exec_kernel<8, 1, false, false, false> : exec_kernel<8, 1, false, false, false, false>;
-        if (!concrete) return exec_kernel<8, 1, false, false, true, false>;
-    }
-    return stage ? pick_t<true>(t.warps, t.wpl) : pick_t<false>(t.warps, t.wpl);
+    return t.role_block == 8 ? pick_b<8>(t, stage, groups, concrete) : pick_b<4>(t, stage, groups, concrete);
 }
 
 uint32_t ring_words(const hedl_kb *kb, const Tuning &t) { return kb->has_concrete() ? t.warps * EX_SMEM_WORDS : 0u; }

@@ -21,8 +21,9 @@ bool same_shape(const Tuning &a, const Tuning &b) {
 
 std::vector<Tuning> candidates(const Tuning &base) {
     std::vector<Tuning> out;
-    auto add = [&](uint32_t stage, uint32_t warps, uint32_t wpl, uint32_t rounds, uint32_t full_occupancy) {
-        Tuning t = base;   // role_block included: it shapes no code
+    auto add = [&](uint32_t stage, uint32_t warps, uint32_t wpl, uint32_t rounds, uint32_t block, uint32_t full_occupancy) {
+        Tuning t = base;
+        t.role_block = block;
         t.stage = stage;
         t.warps = warps;
         t.wpl = wpl;
@@ -31,14 +32,15 @@ std::vector<Tuning> candidates(const Tuning &base) {
         t.full_occupancy = full_occupancy;
         out.push_back(t);
     };
+    for (uint32_t block : {4u, 8u})
+        for (uint32_t rounds : {1u, 2u, 4u}) {
+            for (uint32_t stage : {1u, 0u})
+                for (uint32_t warps : {8u, 16u, 32u}) add(stage, warps, 1, rounds, block, 0);
+            for (uint32_t warps : {1u, 2u}) add(0, warps, 1, rounds, block, 0);
+            add(0, 8, 1, rounds, block, 1);
+        }
     for (uint32_t stage : {1u, 0u})
-        for (uint32_t warps : {8u, 16u, 32u})
-            for (uint32_t rounds : {1u, 2u, 4u}) add(stage, warps, 1, rounds, 0);
-    for (uint32_t warps : {1u, 2u})
-        for (uint32_t rounds : {1u, 2u, 4u}) add(0, warps, 1, rounds, 0);
-    for (uint32_t rounds : {1u, 2u, 4u}) add(0, 8, 1, rounds, 1);
-    for (uint32_t stage : {1u, 0u})
-        for (uint32_t warps : {8u, 16u}) add(stage, warps, 4, 1, 0);
+        for (uint32_t warps : {8u, 16u}) add(stage, warps, 4, 1, 8, 0);
     return out;
 }
 

@@ -24,6 +24,7 @@ constexpr int SMS[] = {152, 16};
 std::map<std::pair<int, const void *>, size_t> opted;   // (device, kernel) -> shared memory it may use
 bool refuse_opt_in = false;        // the next opt-in fails
 unsigned last_grid = 0;
+const void *last_fn = nullptr;
 bool capturing = false;
 cudaError_t last = cudaSuccess;
 int instantiated = 0;
@@ -31,7 +32,7 @@ std::vector<Launch> captured;
 
 cudaError_t launch(const void *fn, dim3 grid, size_t smem, void **args) {
     if (smem > 49152 && smem > opted[{device, fn}]) return cudaErrorInvalidValue;
-    last_grid = grid.x;
+    last_grid = grid.x, last_fn = fn;
     // the interpreter's and the final kernel's first argument begins with the KBView
     if (capturing) captured.push_back({fn, grid.x, static_cast<const hedl::KBView *>(args[0])->pos});
     return cudaSuccess;
@@ -231,6 +232,41 @@ int split_products() {
     REQUIRE(refused([&](hedl::UmmaArgs &b) { b.c_split = 6; }));
     return 0;
 }
+
+// Every launch shape has an interpreter of its own for blocks of 4 and of 8 chunks.
+int role_block() {
+    static Row bits;
+    hedl_kb *kb = load(bits);
+    REQUIRE(kb);
+    const uint64_t prog = HEDL_OP_ATOM;
+    const uint32_t offs[2] = {0, 1};
+    static Row out;
+    void *ws = aligned_alloc(256, 1 << 20);
+    hedl_tuning t;
+    REQUIRE(hedl_tuning_get(kb, &t) == HEDL_OK && t.role_block == 4);
+    std::map<const void *, int> seen;
+    int shapes = 0;
+    for (uint32_t full : {0u, 1u})
+        for (uint32_t stage : {0u, 1u})
+            for (uint32_t wpl : {1u, 4u})
+                for (uint32_t warps : {1u, 2u, 4u, 8u, 16u, 32u}) {
+                    if ((wpl == 4 && (warps < 4 || warps == 32)) || (full && (warps != 8 || wpl != 1 || stage)) ||
+                        (stage && warps < 4))
+                        continue;
+                    ++shapes;
+                    for (uint32_t block : {4u, 8u}) {
+                        t.warps_per_cta = warps, t.words_per_lane = wpl, t.stage_fillers = stage;
+                        t.full_occupancy = full, t.role_block = block;
+                        REQUIRE(hedl_tuning_set(kb, &t) == HEDL_OK);
+                        REQUIRE(hedl_eval_concept(kb, &prog, 1, out.w, ws, 1 << 20, HEDL_NO_GRAPH, nullptr) == HEDL_OK);
+                        ++seen[last_fn];
+                    }
+                }
+    REQUIRE((int)seen.size() == 2 * shapes);
+    hedl_kb_free(kb);
+    free(ws);
+    return 0;
+}
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -239,5 +275,6 @@ int main(int argc, char **argv) {
     if (s == "examples_one_shot") return examples_after_capture(true);
     if (s == "second_device") return second_device();
     if (s == "split_products") return split_products();
+    if (s == "role_block") return role_block();
     return 2;
 }

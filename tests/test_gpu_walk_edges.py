@@ -96,3 +96,17 @@ def test_work_items_of_several_segments(n):
     base, _ = compare_batch(kb, dkb, progs, 0, sample=sample)
     for flags in (H.HEDL_LEVELS, H.HEDL_NO_SLICE, H.HEDL_PLAIN):
         assert np.array_equal(base, dkb.score(*P.pack_batch(progs), flags)), flags
+
+
+@pytest.mark.parametrize("stage", [0, 1])
+@pytest.mark.parametrize("n,spread", [(33, 1), (1000, 1), (6200, 40)])
+def test_lone_walks_in_blocks_of_eight_chunks(n, spread, stage):
+    """Blocks of 256 edges: rows of every length, a batch of lone walks and one restriction at a time."""
+    kb = _kb(n, 5 * n + spread, spread)
+    dkb = device_kb(kb)
+    H.hedl_tuning_set(dkb.handle, role_block=8, stage_fillers=stage)
+    r = Rng(n, 3 + spread)
+    compare_batch(kb, dkb, _restrictions(r, 60, True), H.HEDL_NO_SLICE)
+    compare_batch(kb, dkb, _restrictions(r, 24, True))
+    for p in _restrictions(r, 12, True):
+        compare_batch(kb, dkb, [p], 0)
