@@ -210,119 +210,138 @@ uint64_t put(std::vector<uint8_t> &img, const std::vector<T> &v) {
 // and 186 (2,048 refinements at 4 * 10^6 individuals 57.3 -> 35.4 ms).
 // key_of numbers the (stage, role, direction) triples 0, 1, ... by stage; key_size counts their restrictions.
 //
-// Each node is finished once, when its last operand is, and each role and
+// Each node is finished once, when its last operand is, and a role and
 // direction is looked at only at the stages where a restriction of it becomes
 // ready or due: the time grows with the batch, not with its depth or the KB's roles.
 void walk_stages(const std::vector<PNode> &nodes, uint32_t n_roles, bool all, std::vector<uint32_t> &stage,
                  std::vector<uint32_t> &key_of, std::vector<uint32_t> &key_size) {
-    const uint32_t NN = (uint32_t)nodes.size(), WHOLE = SLICES * MAX_PARTS;
-    auto eligible = [&](const PNode &n) {
-        return is_role(n.op) && (n.op == HEDL_OP_EXISTS || n.op == HEDL_OP_FORALL || n.b <= SLICE_MAX_N);
+    constexpr uint32_t NONE = 0xFFFFFFFFu, WHOLE = SLICES * MAX_PARTS;
+    const uint32_t NN = (uint32_t)nodes.size();
+    // the nodes with a restriction in their expression, children first
+    struct Inner {
+        uint32_t node, role;       // role: key into roles; NONE: no sliceable restriction
+        uint32_t kid[2];           // such nodes among the operands, or NONE
+        uint32_t users, next[2];   // the nodes that read this one: 2 * reader + operand, linked through next
+        uint16_t waits, step;      // operands that are not complete yet; 1 for a restriction
+        uint32_t ready;            // the stage that completed the others, then this one
+        uint32_t limit;            // the stage by which it has to be complete
+        uint32_t link;             // the next of the restrictions that become ready with this one
     };
-    // nesting depths; the nodes with a restriction in their expression, children first
-    std::vector<uint32_t> depth(NN, 0), inner, sliceable;
+    struct Role {
+        uint32_t total = 0, looked = 0, least = NONE;   // least: the smallest limit of the pending ones
+        std::vector<uint32_t> pending;                  // ready restrictions that wait
+    };
+    // roles and directions by their number, unless the KB has far more than the batch can name
+    const bool direct = 2ull * n_roles <= 4ull * NN + 64;
+    std::vector<uint32_t> named;
+    if (!direct) {
+        for (const PNode &n : nodes)
+            if (is_role(n.op)) named.push_back(2 * n.a + n.inv);
+        std::sort(named.begin(), named.end());
+        named.erase(std::unique(named.begin(), named.end()), named.end());
+    }
+    std::vector<Role> roles(direct ? 2 * (size_t)n_roles : named.size());
+    std::vector<Inner> inner;
+    std::vector<uint32_t> at(NN), depth;   // a node's place in inner or NONE; nesting depths by place
+    inner.reserve(NN);
+    depth.reserve(NN);
     uint32_t last = 0;
+    bool shared = all;
     for (uint32_t i = 0; i < NN; ++i) {
         const PNode &n = nodes[i];
-        const uint32_t d = std::max(n.k0 >= 0 ? depth[n.k0] : 0u, n.k1 >= 0 ? depth[n.k1] : 0u);
-        depth[i] = d + (is_role(n.op) ? 1u : 0u);
-        if (depth[i]) inner.push_back(i);
-        if (eligible(n)) sliceable.push_back(i);
-        last = std::max(last, depth[i]);
-    }
-    // the roles and directions that have sliceable restrictions, in a dense
-    // numbering: by a table of the KB's, unless the batch has far fewer restrictions
-    std::vector<uint32_t> role(NN, 0), total;
-    {
-        std::vector<uint32_t> ids;
-        if (2ull * n_roles <= 4ull * sliceable.size() + 64) {
-            ids.assign(2 * (size_t)n_roles, 0);
-            for (uint32_t i : sliceable) ids[2 * nodes[i].a + nodes[i].inv] = 1;
-            uint32_t k = 0;
-            for (uint32_t &id : ids) k += std::exchange(id, k);
-            total.assign(k, 0);
-            for (uint32_t i : sliceable) total[role[i] = ids[2 * nodes[i].a + nodes[i].inv]]++;
-        } else {
-            for (uint32_t i : sliceable) ids.push_back(2 * nodes[i].a + nodes[i].inv);
-            std::sort(ids.begin(), ids.end());
-            ids.erase(std::unique(ids.begin(), ids.end()), ids.end());
-            total.assign(ids.size(), 0);
-            for (uint32_t i : sliceable)
-                total[role[i] = (uint32_t)(std::lower_bound(ids.begin(), ids.end(), 2 * nodes[i].a + nodes[i].inv) - ids.begin())]++;
+        const bool role = is_role(n.op);
+        const uint32_t kid[2] = {n.k0 >= 0 ? at[n.k0] : NONE, n.k1 >= 0 ? at[n.k1] : NONE};
+        at[i] = NONE;
+        if (!role && kid[0] == NONE && kid[1] == NONE) continue;
+        const uint32_t me = at[i] = (uint32_t)inner.size();
+        Inner x{i, NONE, {kid[0], kid[1]}, NONE, {NONE, NONE}, 0, role, 0, 0, NONE};
+        uint32_t d = 0;
+        for (uint32_t k = 0; k < 2; ++k)
+            if (kid[k] != NONE) {
+                d = std::max(d, depth[kid[k]]);
+                x.next[k] = std::exchange(inner[kid[k]].users, 2 * me + k);
+                ++x.waits;
+            }
+        if (role && (n.op == HEDL_OP_EXISTS || n.op == HEDL_OP_FORALL || n.b <= SLICE_MAX_N)) {
+            const uint32_t key = 2 * n.a + n.inv;
+            x.role = direct ? key : (uint32_t)(std::lower_bound(named.begin(), named.end(), key) - named.begin());
+            shared |= ++roles[x.role].total > 1;
         }
+        depth.push_back(d + (role ? 1u : 0u));
+        last = std::max(last, depth.back());
+        inner.push_back(x);
     }
-    if (!all && std::none_of(total.begin(), total.end(), [](uint32_t n) { return n > 1; })) return;
-    // the stage by which a node has to be complete; how many of its operands still wait
-    std::vector<uint32_t> limit(NN, last), waits(NN, 0);
-    for (auto it = inner.rbegin(); it != inner.rend(); ++it) {
-        const PNode &n = nodes[*it];
-        const uint32_t l = limit[*it] - (is_role(n.op) ? 1u : 0u);
-        if (n.k0 >= 0) limit[n.k0] = std::min(limit[n.k0], l);
-        if (n.k1 >= 0) limit[n.k1] = std::min(limit[n.k1], l);
+    if (!shared) return;
+    for (Inner &x : inner) x.limit = last;
+    for (size_t q = inner.size(); q-- > 0;) {
+        const Inner &x = inner[q];
+        const uint32_t l = x.limit - x.step;
+        for (uint32_t k : x.kid)
+            if (k != NONE) inner[k].limit = std::min(inner[k].limit, l);
     }
-    // the nodes that read node i: users[first[i] .. first[i + 1])
-    std::vector<uint32_t> first(NN + 1, 0), users;
-    for (uint32_t i : inner)
-        for (int32_t k : {nodes[i].k0, nodes[i].k1})
-            if (k >= 0 && depth[k]) first[k + 1]++, waits[i]++;
-    for (uint32_t i = 0; i < NN; ++i) first[i + 1] += first[i];
-    users.resize(first[NN]);
-    {
-        std::vector<uint32_t> at(first.begin(), first.end() - 1);
-        for (uint32_t i : inner)
-            for (int32_t k : {nodes[i].k0, nodes[i].k1})
-                if (k >= 0 && depth[k]) users[at[k]++] = i;
-    }
-    std::vector<uint32_t> done(NN, 0);   // the stage that completes a node, once it is known
-    // stage s: the restrictions that become ready, and the roles and directions of which one is due
-    std::vector<std::vector<uint32_t>> ready(last + 2), due(last + 1);
-    std::vector<uint32_t> stack;
-    // node i's operands are complete by stage d
-    auto operands_done = [&](uint32_t i, uint32_t d) {
-        if (eligible(nodes[i])) ready[d + 1].push_back(i);
-        else done[i] = d + (is_role(nodes[i].op) ? 1u : 0u), stack.push_back(i);
+    std::vector<uint32_t> ready(last + 2, NONE);   // restrictions that become ready at a stage: the first one
+    struct Due {
+        uint32_t role, next;
     };
-    auto spread = [&]() {
-        while (!stack.empty()) {
-            const uint32_t i = stack.back();
-            stack.pop_back();
-            for (uint32_t q = first[i]; q < first[i + 1]; ++q) {
-                const uint32_t u = users[q];
-                const PNode &n = nodes[u];
-                if (--waits[u] == 0) operands_done(u, std::max(n.k0 >= 0 ? done[n.k0] : 0u, n.k1 >= 0 ? done[n.k1] : 0u));
+    std::vector<Due> dues;
+    std::vector<uint32_t> due(last + 1, NONE);     // roles and directions of which a restriction is due: the first one
+    std::vector<uint32_t> finished, looked;
+    auto operands_done = [&](uint32_t q) {
+        Inner &x = inner[q];
+        if (x.role != NONE) x.link = std::exchange(ready[x.ready + 1], q);
+        else x.ready += x.step, finished.push_back(q);
+    };
+    auto spread = [&]() {   // from the finished nodes to those that read them
+        while (!finished.empty()) {
+            const Inner &x = inner[finished.back()];
+            finished.pop_back();
+            for (uint32_t e = x.users; e != NONE; e = inner[e >> 1].next[e & 1]) {
+                Inner &u = inner[e >> 1];
+                u.ready = std::max(u.ready, x.ready);
+                if (--u.waits == 0) operands_done(e >> 1);
             }
         }
     };
-    for (uint32_t i : inner)
-        if (depth[i] == 1 && waits[i] == 0) operands_done(i, 0);
+    for (uint32_t q = 0; q < inner.size(); ++q)
+        if (inner[q].waits == 0) operands_done(q);
     spread();
-    std::vector<std::vector<uint32_t>> pending(total.size());   // ready restrictions that wait
-    std::vector<uint32_t> looked;
+    auto look = [&](uint32_t k, uint32_t s) {
+        if (std::exchange(roles[k].looked, s) != s) looked.push_back(k);
+    };
+    auto when_due = [&](uint32_t k, uint32_t limit) {   // limit: the new least one
+        roles[k].least = limit;
+        dues.push_back({k, due[limit]});
+        due[limit] = (uint32_t)dues.size() - 1;
+    };
     for (uint32_t s = 1; s <= last; ++s) {
-        looked.swap(due[s]);
-        for (uint32_t i : ready[s]) {
-            std::vector<uint32_t> &p = pending[role[i]];
-            if (total[role[i]] < 3 || limit[i] <= s || p.size() + 1 >= WHOLE) looked.push_back(role[i]);
-            p.push_back(i);
-            if (limit[i] > s) due[limit[i]].push_back(role[i]);
+        for (uint32_t e = due[s]; e != NONE; e = dues[e].next) look(dues[e].role, s);
+        for (uint32_t q = ready[s]; q != NONE; q = inner[q].link) {
+            Role &r = roles[inner[q].role];
+            r.pending.push_back(q);
+            if (inner[q].limit < r.least) when_due(inner[q].role, std::max(inner[q].limit, s));
+            if (r.total < 3 || r.least <= s || r.pending.size() >= WHOLE) look(inner[q].role, s);
         }
-        std::sort(looked.begin(), looked.end());
-        looked.erase(std::unique(looked.begin(), looked.end()), looked.end());
         for (uint32_t k : looked) {
-            std::vector<uint32_t> &p = pending[k];
-            size_t n = p.size();   // how many walk now
-            if (total[k] >= 3 && std::none_of(p.begin(), p.end(), [&](uint32_t i) { return limit[i] <= s; })) {
+            Role &r = roles[k];
+            size_t n = r.pending.size();   // how many walk now
+            if (r.total >= 3 && r.least > s) {
                 n = n / WHOLE * WHOLE;
-                if (n) std::sort(p.begin(), p.end(), [&](uint32_t x, uint32_t y) { return limit[x] != limit[y] ? limit[x] < limit[y] : x < y; });
+                if (n && n < r.pending.size())
+                    std::nth_element(r.pending.begin(), r.pending.begin() + (ptrdiff_t)n, r.pending.end(),
+                                     [&](uint32_t x, uint32_t y) {
+                                         return inner[x].limit != inner[y].limit ? inner[x].limit < inner[y].limit : x < y;
+                                     });
             }
             if (n == 0) continue;
             for (size_t q = 0; q < n; ++q) {
-                const uint32_t i = p[q];
-                done[i] = stage[i] = s, key_of[i] = (uint32_t)key_size.size();
-                stack.push_back(i);
+                Inner &x = inner[r.pending[q]];
+                x.ready = stage[x.node] = s, key_of[x.node] = (uint32_t)key_size.size();
+                finished.push_back(r.pending[q]);
             }
             key_size.push_back((uint32_t)n);
-            p.erase(p.begin(), p.begin() + (ptrdiff_t)n);
+            r.pending.erase(r.pending.begin(), r.pending.begin() + (ptrdiff_t)n);
+            r.least = NONE;
+            if (!r.pending.empty()) when_due(k, inner[r.pending[0]].limit);   // the first of the rest is the least
         }
         looked.clear();
         spread();
