@@ -573,3 +573,29 @@ def test_planning_time_follows_the_batch():
         base = seconds(few, progs, H.HEDL_NO_SLICE)
         assert seconds(hk, progs, 0) < 8 * base
         assert seconds(hk, progs, H.HEDL_SLICE_ALL) < 16 * base
+
+
+# A transpose runs a level after its fillers (a concept row: level 0), its walk the next one, a reader of a slot one
+# later; a group holds at most 64 restrictions.  By nesting depth alone: other groups or levels, as stated.
+WAITING = [
+    # three restrictions on r1 make one group at the depth of the deepest (by depth: a pair, walked at once: 3 levels)
+    (["(some r1 A2)", "(all r1 A5)", "(some r1 (some r2 A3))"], 1, 4),
+    # 62 shallow and two deep ones are one full group (by depth: 3 groups with the two on r2)
+    ([f"(some r1 A{k})" for k in range(62)] + ["(some r1 (some r2 A63))", "(all r1 (some r2 A64))"], 2, 5),
+    # 65 shallow ones: a full group walks at once, the last one waits for the two deep ones (by depth: 4 groups)
+    ([f"(some r1 A{k})" for k in range(65)] + ["(some r1 (some r2 A66))", "(all r1 (some r2 A67))"], 3, 5),
+    # a restriction that another one needs cannot wait, and the ready ones walk with it: a group of three, the deep one alone
+    (["(some r2 (some r1 A0))", "(some r1 A1)", "(some r1 A2)", "(some r1 (some r3 A4))"], 1, 3),
+    # without it they wait for the deep one (the two on r3 walk first)
+    (["(some r2 (some r3 A0))", "(some r1 A1)", "(some r1 A2)", "(some r1 (some r3 A4))"], 2, 5),
+    # one or two restrictions of a role and direction do not wait
+    (["(some r1 A2)", "(some r1 (some r2 A3))"], 0, 2),
+    (["(some r1 A2)", "(some r1 A4)", "(some r1- (some r2 A3))"], 1, 3),
+]
+
+
+@pytest.mark.parametrize("texts,groups,levels", WAITING)
+def test_restrictions_wait_to_share_a_walk(texts, groups, levels):
+    hk = H.hedl_kb_plan_only(1_000_000, 80, [8_000_000] * 6, 2)
+    info = H.hedl_plan_info_get(H.hedl_plan_batch(hk, *P.pack_batch([P.compile_text(t) for t in texts])))
+    assert (info["n_role_groups"], info["n_levels"]) == (groups, levels)
