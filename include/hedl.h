@@ -408,7 +408,7 @@ int hedl_tuning_get(const hedl_kb *kb, hedl_tuning *t);
 int hedl_tuning_set(hedl_kb *kb, const hedl_tuning *t);
 
 /* Workspace bytes hedl_autotune needs for this probe batch: the largest plan
- * over every candidate launch shape.  Host-only. */
+ * over every candidate launch shape, and the probe's counts.  Host-only. */
 int hedl_autotune_workspace_size(hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, uint32_t H,
                                  size_t *bytes);
 

@@ -107,7 +107,7 @@ extern "C" int hedl_autotune_workspace_size(hedl_kb *kb, const uint64_t *progs, 
         need = std::max<size_t>(need, p->ws_bytes);
         delete p;
     }
-    *bytes = need;
+    *bytes = ((need + 255) & ~size_t(255)) + 16ull * H;   // the probe's counts lie behind the largest plan
     return HEDL_OK;
 }
 
@@ -123,16 +123,13 @@ extern "C" int hedl_autotune(hedl_kb *kb, const uint64_t *progs, const uint32_t 
     if (!cached) {
         cudaStream_t st = (cudaStream_t)s;
         uint32_t *counts = nullptr;
-        // counts live at the end of ws, past every candidate's plan
-        size_t cbytes = 16ull * H;
         size_t need = 0;
         int e = hedl_autotune_workspace_size(kb, progs, offs, H, &need);
         if (e) return e;
-        size_t coff = (need + 255) & ~size_t(255);
-        if (!ws || ws_bytes < coff + cbytes)
+        if (!ws || ws_bytes < need)
             return fail(HEDL_ERR_WORKSPACE_TOO_SMALL, "autotune workspace of " + std::to_string(ws_bytes) +
-                                                          " bytes, " + std::to_string(coff + cbytes) + " needed");
-        counts = (uint32_t *)((uint8_t *)ws + coff);
+                                                          " bytes, " + std::to_string(need) + " needed");
+        counts = (uint32_t *)((uint8_t *)ws + need - 16ull * H);
         cudaEvent_t a, b;
         cudaEventCreate(&a);
         cudaEventCreate(&b);
@@ -144,11 +141,11 @@ extern "C" int hedl_autotune(hedl_kb *kb, const uint64_t *progs, const uint32_t 
             PlanImpl *p = nullptr;
             e = build_plan(kb, progs, offs, H, HEDL_NO_GRAPH, &p);
             if (e) break;
-            e = execute(kb, p, counts, nullptr, ws, coff, s, true);
+            e = execute(kb, p, counts, nullptr, ws, need - 16ull * H, s, true);
             float ms = 0;
             for (int rep = 0; rep < 3 && !e; ++rep) {
                 cudaEventRecord(a, st);
-                e = execute(kb, p, counts, nullptr, ws, coff, s, false);
+                e = execute(kb, p, counts, nullptr, ws, need - 16ull * H, s, false);
                 cudaEventRecord(b, st);
                 cudaError_t ce = cudaEventSynchronize(b);
                 if (ce) e = cuda_fail(ce, "autotune timing");

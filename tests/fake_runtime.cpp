@@ -267,6 +267,28 @@ int role_block() {
     free(ws);
     return 0;
 }
+
+// A workspace of the size that hedl_autotune_workspace_size gives is enough for hedl_autotune.
+int autotune_workspace() {
+    static Row bits, ex[2];
+    hedl_kb *kb = load(bits);
+    REQUIRE(kb);
+    REQUIRE(hedl_examples_set(kb, ex[0].w, ex[1].w, nullptr) == HEDL_OK);
+    for (uint32_t hyps : {1u, 3u, 1000u}) {
+        const std::vector<uint64_t> progs(hyps, HEDL_OP_ATOM);
+        std::vector<uint32_t> offs(hyps + 1);
+        for (uint32_t h = 0; h <= hyps; ++h) offs[h] = h;
+        size_t bytes = 0;
+        REQUIRE(hedl_autotune_workspace_size(kb, progs.data(), offs.data(), hyps, &bytes) == HEDL_OK);
+        void *ws = aligned_alloc(256, (bytes + 255) / 256 * 256);
+        REQUIRE(hedl_autotune(kb, progs.data(), offs.data(), hyps, ws, bytes, nullptr, nullptr, nullptr) == HEDL_OK);
+        REQUIRE(hedl_autotune(kb, progs.data(), offs.data(), hyps, ws, bytes - 1, nullptr, nullptr, nullptr) ==
+                HEDL_ERR_WORKSPACE_TOO_SMALL);
+        free(ws);
+    }
+    hedl_kb_free(kb);
+    return 0;
+}
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -276,5 +298,6 @@ int main(int argc, char **argv) {
     if (s == "second_device") return second_device();
     if (s == "split_products") return split_products();
     if (s == "role_block") return role_block();
+    if (s == "autotune_workspace") return autotune_workspace();
     return 2;
 }

@@ -22,7 +22,8 @@ def program(tmp_path_factory):
     return str(exe)
 
 
-@pytest.mark.parametrize("scenario", ["examples_plan", "examples_one_shot", "second_device", "split_products", "role_block"])
+@pytest.mark.parametrize("scenario", ["examples_plan", "examples_one_shot", "second_device", "split_products", "role_block",
+                                      "autotune_workspace"])
 def test_scenario(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
