@@ -434,7 +434,7 @@ def numeric_run(args, dev):
     cpu = _oracle_rate(dc_replace(kb, num_row_ptr=kb.num_row_ptr[:2], num_vals=kb.num_vals[:2]), three[:6])
     return {"workload": "N=10,000,000 individuals, 8 numeric concrete roles, Poisson(4) values per individual "
                         "U[0,1000] (~4*10^7 values, 200 MB per role)", "kb_gen_s": gen_s, "cpu_baseline": cpu,
-            "values": [int(v.size) for v in kb.num_vals], "kernel": "exec_kernel (exist_words)",
+            "values": [int(v.size) for v in kb.num_vals], "kernel": "exec_kernel (exist_run)",
             "peak": peak, "peak_kind": f"{kind} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
             "one_per_role": a, "three_per_role": b, "plain_three_per_role": c,
             "plain_counts_identical": bool(torch.equal(cb, cp)), "clocks": clk.summary()}
@@ -473,7 +473,7 @@ def string_run(args, dev):
     return {"workload": "N=10,000,000 individuals, 8 string concrete roles, Poisson(2) values per individual "
                         "(~2*10^7 ids, 120 MB per role) into 100,000 distinct strings of 3-12 letters; 64 "
                         "patterns", "kb_gen_s": gen_s, "kb_load_s_with_bitmap": load_s, "cpu_baseline": cpu,
-            "values": [int(v.size) for v in kb.str_ids], "kernel": "exec_kernel (exist_words)",
+            "values": [int(v.size) for v in kb.str_ids], "kernel": "exec_kernel (exist_run)",
             "peak": peak, "peak_kind": f"{kind} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
             "equal_one_per_role": a, "equal_and_contain": b, "plain_equal_and_contain": c,
             "plain_counts_identical": bool(torch.equal(cb, cp)), "clocks": clk.summary()}

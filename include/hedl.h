@@ -550,7 +550,8 @@ int hedl_scores_from_counts(const uint32_t *counts, uint32_t H, float *scores, h
 
 /* Indices (DEVICE uint32 [k], ascending) of the k best rows of Y (DEVICE
  * float [H][2]) ordered by Y[.][0] descending, then Y[.][1] descending, then
- * index ascending (NaN last).  ws >= hedl_select_workspace_size(H). */
+ * index ascending (NaN last).  ws >= hedl_select_workspace_size(H), which is
+ * checked; the selection works in shared memory and writes nothing there. */
 int hedl_select_workspace_size(uint32_t H, size_t *bytes);
 int hedl_select_top(const float *Y, uint32_t H, uint32_t k, uint32_t *idx, void *ws, size_t ws_bytes,
                     hedl_stream s);

@@ -124,16 +124,6 @@ __device__ __forceinline__ void prefetch_range(const uint32_t *a, uint32_t lo, u
     if (bytes) prefetch_l2(a + lo, bytes);
 }
 
-// the same for four consecutive words (p 16-byte aligned)
-__device__ __forceinline__ uint4 ld_stream4(const uint32_t *p) {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
-}
-
-
 // Role restriction over the warp's 32*WPL words (Algorithms 3-8 of the
 // paper, recast).  For each word (32 individuals) the warp walks the word's
 // CSR edge range, a block of BLK (<= 32) chunks of 32 edges at a time: lane e

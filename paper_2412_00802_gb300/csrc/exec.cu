@@ -442,9 +442,13 @@ constexpr uint32_t WALK_BUF = 256;   // 32-bit words of a warp's window buffer
 // are skipped.  Rows longer than HEAVY_ROW are walked by the whole warp,
 // HEAVY_LOADS edges a lane in flight, and their counts reduced across lanes.
 //
-// Bound: the gathers, one L1 miss an SM and clock (280 G/s over the chip, for
-// 4, 8 or 16 bytes alike).  2,048 refinements at 4 * 10^6 individuals (134
-// walks of 40 M edges of Zipf lengths): 35.4 -> 33.9 ms, with the work items of several segments.
+// Floor: the gathers, one L1 miss an SM and clock (280 G/s over the chip, for
+// 4, 8 or 16 bytes alike).  2,048 refinements at 4 * 10^6 individuals (137
+// walks of 40 M edges of Zipf lengths, 5.5 G gathers, 20 ms) take 34.6 ms, 35.4
+// without the work items of several segments; 4,096 hypotheses on 10^6 (177
+// walks of 6 M edges, 1.1 G gathers, 3.9 ms) 15.9.  What is above it: only the
+// edges are loaded a window ahead, so that a warp has no gather in flight while
+// it adds, and with short rows most lanes have nothing to add.
 //
 // The tile's words are wb .. wb + K - 1 (K a multiple of 4) of wp; n_words hold
 // the n_indiv individuals; *chunk counts from 0.  A function of its own:
@@ -853,8 +857,6 @@ size_t smem_bytes(const hedl_kb *kb, const Tuning &t, bool stage) {
 bool use_staging(const hedl_kb *kb, const Tuning &t) {
     return t.stage && t.warps >= 4 && smem_bytes(kb, t, true) <= kb->smem_optin;
 }
-
-size_t exec_smem_bytes(const Tuning &t) { return stack_smem_bytes(t) + 16; }
 
 int exec_occupancy(const hedl_kb *kb, const Tuning &t, bool groups, int *blocks_per_sm) {
     const bool stage = use_staging(kb, t);

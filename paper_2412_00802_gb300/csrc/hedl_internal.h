@@ -103,8 +103,8 @@ struct Seg {
     uint32_t kind;       // TASK_*
 };
 
-// Up to 64 role restrictions of one role, direction and role depth,
-// evaluated together: the transpose turns the fillers into `parts` words per
+// Up to 64 role restrictions of one role, direction and level, evaluated
+// together: the transpose turns the fillers into `parts` words per
 // individual (bit s of word p = slice 32p + s's filler), the walk adds those
 // words over each individual's successors in bit-sliced 3-bit saturating
 // counters and maps the counts through a truth table per word.
@@ -356,6 +356,5 @@ int exec_occupancy(const hedl_kb *kb, const Tuning &t, bool groups, int *blocks_
 int kb_validate_device(const hedl_kb *kb, void *stream, std::string *why);
 int contain_bitmap_device(const hedl_kb *kb, void *stream);
 int examples_count_device(const hedl_kb *kb, void *stream, uint32_t *np, uint32_t *nn);
-size_t exec_smem_bytes(const Tuning &t);
 
 }  // namespace hedl

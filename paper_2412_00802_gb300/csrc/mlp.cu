@@ -15,7 +15,7 @@
 // to gradients, Adam).  Every sum over the batch is first a partial sum of a
 // chunk of rows and then a sum over chunks in a fixed order, so a step's
 // gradients do not depend on timing.  At batches of 4,096 this took a step
-// from 785 us to 61 us: the weight gradient of the output layer
+// from 785 us to 57 us: the weight gradient of the output layer
 // (584 us) and the bias gradients (2 x 238 us) had been two blocks' loops over
 // the whole batch, and the weight gradients had needed four transposes.
 #include <cuda_bf16.h>
@@ -441,11 +441,9 @@ int gemm(const GemmArgs &a0, bool a_km, bool b_kn, int splits, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ output layer (N = 2)
-// Y[b][j] = sum_i H2[b][i] W3[j][i] + b3[j]: one warp per row.
+// Y = u + b3 from the fused output layer's sums u [parts][B][2], a thread a row.
 // With map (DEVICE float[5]: mean0, mean1, scale0, scale1, tail weight), the
-// raw output u is mapped back to the target scale: Y = u * scale + mean.
-// y = (u + b3), mapped back to the target scale when map is set, from the
-// fused output layer's sums u [parts][B][2] (the unfused path's out_fwd_kernel semantics).
+// output is mapped back to the target scale: Y = (u + b3) * scale + mean.
 __global__ void out_map_kernel(const float *u, int parts, const float *b3, float *Y, int B, const float *map) {
     pdl_trigger();
     pdl_wait();
@@ -465,6 +463,8 @@ __global__ void out_map_kernel(const float *u, int parts, const float *b3, float
     }
 }
 
+// The output layer of the mma.sync engine: Y[b][j] = sum_i H2[b][i] W3[j][i] + b3[j],
+// mapped as above; one warp per row.
 __global__ void out_fwd_kernel(const __nv_bfloat16 *H2, const __nv_bfloat16 *W3, const float *b3, float *Y, int B,
                                const float *map) {
     // warp per row (grid-stride); lane l holds columns 16l .. 16l+15 of both W3 rows

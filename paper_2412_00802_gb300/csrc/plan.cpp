@@ -205,9 +205,14 @@ uint64_t put(std::vector<uint8_t> &img, const std::vector<T> &v) {
 // and direction of one or two restrictions does not wait: two lone walks over
 // bitset fillers cost about as much as a shared one with its transpose.
 // Walking every restriction as soon as it is ready (one group per role,
-// direction and nesting depth) took 261 walks for 2,048 refinements over 64
-// roles and directions and 244 for a batch of 4,096 over 32; this takes 134
-// and 186 (2,048 refinements at 4 * 10^6 individuals 57.3 -> 35.4 ms).
+// direction and nesting depth) takes 231 walks for 2,048 refinements over 64
+// roles and directions and 225 for a batch of 4,096 over 32; this takes 137
+// and 177 (2,048 refinements at 4 * 10^6 individuals 57.3 -> 35.4 ms).  A plan
+// may get more levels for it, without fewer walks in some batches of a few
+// hypotheses.  Over 738 batches of 16 to 2,000 hypotheses on 10^4 to 4 * 10^6
+// individuals waiting takes 0.85 to 0.93 of the time (geometric mean of each size
+// and degree law), 0.90 also where it saves no walk and adds levels; one batch in
+// nine gets more than 5 % slower, and neither the walks nor the levels tell which.
 // key_of numbers the (stage, role, direction) triples 0, 1, ... by stage; key_size counts their restrictions.
 //
 // Each node is finished once, when its last operand is, and a role and
@@ -758,8 +763,9 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     for (uint32_t sidx = 0; sidx < NSEG; ++sidx)
         if (segs[sidx].hyp != NO_HYP) seg_level[sidx] = seg_lvl(sidx);
 
-    // role groups: sliced restrictions keyed by (stage, role, direction), up to
-    // SLICES * MAX_PARTS at a time (one FT word per 32 of them)
+    // role groups: sliced restrictions keyed by (level, role, direction), up to
+    // SLICES * MAX_PARTS at a time (one FT word per 32 of them); those of
+    // a (stage, role, direction) share a level, and stages that come out on one level share groups
     std::vector<RGroup> rgroups;
     std::vector<uint32_t> task_level(seg_level);
     std::vector<uint32_t> task_key(role_key);
@@ -865,8 +871,8 @@ int build_plan(const hedl_kb *kb, const uint64_t *progs, const uint32_t *offs, u
     // busy, each walking 32 words in sequence: then a warp covers fewer words
     // (down to 4, one round per item) so that the level spreads over about
     // four times as many warp-rounds as there are resident warps (32 per SM at
-    // 64 registers), which also balances rows of very different degree.  Role
-    // groups walk 32 words per warp and keep the default shape.
+    // 64 registers), which also balances rows of very different degree.  Plans
+    // with role groups keep the default shape for their segments.
     const Tuning &t = p->tuning;
     uint32_t WW = 32, rounds = t.rounds;
     if (rgroups.empty() && kb->n_sms > 0) {
