@@ -469,12 +469,13 @@ struct ValueTest {
 // early exit): a heavy subject costs its values up to the piece of its first
 // pass.
 //
-// Bound: HBM (4(N+1) + 4M bytes a restriction), as long as the instructions
-// stay few and fit the instruction cache: about 60 a word of 32 individuals
-// with four values each.  Packing 16-byte loads into masks by shuffles took
-// 138, and with a function a kind of test and the row batches in two register
-// sets warps waited 47 % of their time for instructions.  24 restrictions on 8
-// roles at 10^7 individuals (3.8 GB by the model, each role read three times):
+// Bound: instruction issue, 83 % of the cycles for 12 restrictions on 4 numeric
+// roles of four values a subject at 10^7 individuals (593 us, 160 instructions a
+// word of 32 individuals and restriction, the stack machine's included).  With
+// the values loaded into registers and packed into masks by shuffles it was 142
+// instructions, but issue at 51 %: warps waited for their loads (864 us).  A
+// function for each kind of test made warps wait for instructions.  24
+// restrictions on 8 roles (3.8 GB by the model, each role read three times):
 // 1.96 ms -> 1.26 ms, with rings half as large 1.10 ms.
 static_assert(EX_RING % EX_LOADS == 0 && EX_LOADS % 4 == 0, "a window's masks are whole 16-byte stores");
 
