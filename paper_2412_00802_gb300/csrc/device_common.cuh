@@ -239,9 +239,10 @@ __device__ __forceinline__ void role_words(const DevCSR g, const uint32_t *fille
 // A word whose every lane is decided (cap reached or row ended) makes the
 // stream jump to the next word's first edge.  Word k of the warp goes to lane
 // k / WPL, slot k % WPL.  n_words bounds the warp's words; lanes of
-// individuals >= n hold empty rows and emit 0.  SMEM: the filler row is staged
-// in shared memory.  A function of its own, with registers of its own: inlined,
-// the stack machine around it spilled.
+// individuals >= n hold empty rows and emit 0.  GLOBAL: the filler row is said
+// to lie in global memory (else it may be staged in shared memory).  A function
+// of its own, with registers of its own: inlined, the stack machine around it
+// spilled.
 //
 // Bound: latency and the filler's gathers.  Which block is faster depends on
 // the rows, which the plan does not know: on heavy-tailed ones a block of 8
@@ -254,11 +255,11 @@ template <int WPL>
 struct RowWords {
     uint32_t v[WPL];
 };
-template <int WPL, uint32_t BLK, bool SMEM>
+template <int WPL, uint32_t BLK, bool GLOBAL>
 __device__ __noinline__ RowWords<WPL> role_stream(const uint32_t *rp, const uint32_t *col, const uint32_t *filler,
                                                   uint32_t kind, uint32_t n_arg, uint32_t n, uint32_t n_words,
                                                   uint32_t wb, bool filler_inverted) {
-    if constexpr (BLK == 8u && !SMEM) __builtin_assume(__isGlobal(filler));   // loads of blocks of 4 got 1 % slower
+    if constexpr (GLOBAL) __builtin_assume(__isGlobal(filler));
     constexpr uint32_t BE = 32u * BLK;              // edges per block
     const uint32_t lane = threadIdx.x & 31u;
     RowWords<WPL> out;
