@@ -572,7 +572,7 @@ def test_planning_time_follows_the_batch():
     for hk, progs in ((few, chain), (many, chain), (many, lone)):
         base = seconds(few, progs, H.HEDL_NO_SLICE)
         assert seconds(hk, progs, 0) < 8 * base
-        assert seconds(hk, progs, H.HEDL_SLICE_ALL) < 16 * base
+        assert seconds(hk, progs, H.HEDL_SLICE_ALL) < 32 * base   # 10,000 groups of one: 6 to 12 times the image
 
 
 # A transpose runs a level after its fillers (a concept row: level 0), its walk the next one, a reader of a slot one
